@@ -1,0 +1,1154 @@
+// Algorithm 1 (Section 2.2.1, Eq. 3-4) on the GPU, one CTA per folded
+// profile at a time (persistent over a run of consecutive trials), with the
+// last FFA stage (Section 2.1) fused into the load.
+//
+// The profile lives in shared memory only (score.cuh's swizzled layout, no
+// padding, nothing held in registers between steps), so a CTA is as small as
+// the profile's length asks for -- one warp for the shortest ones -- and
+// several profiles share an SM: one's serial steps (selections, reductions,
+// barriers) run under the others' arithmetic.
+//
+// Median and MAD (exact).  The profile's mean and standard deviation, taken
+// while it is loaded, and the offset and ratio that the CTA's previous trial
+// showed, predict the median (then the MAD) to within a few sigma / sqrt(N).
+// One pass over the profile counts the samples below a window of that width
+// and lists those inside it; if the wanted ranks lie in the window, one warp
+// finds the order statistics in the list (a few counting passes at
+// interpolated pivots), otherwise the window is moved and the pass repeated,
+// and after a few attempts an exact radix select over the profile takes over.
+// A window's bounds are monotone functions of the value, so the counts are
+// exact whatever the prediction was.  Int profiles need no list: their
+// window holds one bucket per integer.
+//
+// Box sums.  With the in-block exclusive prefix c_b[o] (blocks of R bins, the
+// cyclic extension included) and the block offsets C[b] = sum of earlier
+// blocks (float-float, or wrapping int32), the box of width w = R * d at bin
+// R b + o is (C[b + d] - C[b]) + (c_{b+d}[o] - c_b[o]); widths below R
+// use the block itself and the next one.  Rounding is monotone, so a block's
+// largest box is D + max_o (c_{b+d}[o] - c_b[o]): the offset D is added once
+// per block and width, not per bin.  Only the maximum of each width is kept;
+// the winning width's first argmax is found afterwards by recomputing that
+// width in the threads that hold its maximum.  The block that runs past p0
+// scores all its bins (its extra boxes are cyclic boxes of the first bins
+// again).
+#include <cuda_runtime.h>
+#include <math.h>
+#include <stdint.h>
+
+#include <map>
+#include <mutex>
+#include <tuple>
+#include <type_traits>
+
+#include "score.cuh"
+
+namespace ffa {
+
+namespace {
+
+template <class V>
+struct IsInt {
+    static constexpr bool value = std::is_integral<V>::value;
+};
+
+// Where a CTA's regions start in dynamic shared memory (bytes); the profile
+// is at 0.  `offs` (block offsets) and `list` (window members, `cap` slots
+// per thread) share a region: the list is dead before the offsets are formed.
+// `aux`: the window's members packed (float), its histogram (int), or the
+// radix select's.
+struct ScoreLay {
+    uint32_t offs, list, aux;
+    int32_t cap;
+};
+
+constexpr int score_pack(int r) { return r == 8 ? 256 : 768; }  // members a float window may have
+constexpr int score_nb(int r) { return r == 8 ? 256 : 512; }    // buckets of an int window
+constexpr int S1_NC = 64;                                       // near-ties of one pick
+constexpr int S1_MAXSEG = 16;
+
+struct S1Sh {
+    unsigned long long cand[S1_NC], key[2];
+    float fa[32], fb[32], fc[32];
+    uint2 wc[2][32];          // per-warp counts of a window pass (two slots, alternating)
+    float2 seg[S1_MAXSEG];    // segment totals of the offset scan
+    uint32_t wkey[16];        // per-width maxima as order-preserving keys
+    uint32_t npack, ncand;
+    int bin_a, bin_b;
+    uint32_t below_a;
+    int ok;
+    uint32_t pos;
+    float best;
+    int bw;
+};
+
+__device__ __forceinline__ unsigned long long ff_key(float h, float l) {
+    return ((unsigned long long)fkey(h) << 32) | fkey(l);
+}
+
+// |x - (mh + ml)| as a canonical float-float pair
+__device__ __forceinline__ void ff_dev(float x, float mh, float ml, float& h, float& l) {
+    two_sum(x, -mh, h, l);
+    l = __fsub_rn(l, ml);
+    ff_norm(h, l);
+    if (h < 0.0f || (h == 0.0f && l < 0.0f)) {
+        h = -h;
+        l = -l;
+    }
+}
+
+// 2^(n/2) as the correctly rounded square root of 2^n
+__device__ __forceinline__ float sqrt_pow2(int n) {
+    return __int_as_float((127 + (n >> 1)) << 23) * ((n & 1) ? 1.41421356237309515f : 1.0f);
+}
+
+template <bool ONE>
+__device__ __forceinline__ void cta_sync() {
+    if (ONE) __syncwarp();
+    else __syncthreads();
+}
+
+// Warp 0: the buckets of hist[0, n) (n a multiple of 128) that hold ranks
+// ta <= tb (both below the total), and the count before the first one.
+template <bool ONE>
+__device__ __forceinline__ void hist_find(const uint32_t* hist, int n, uint32_t ta, uint32_t tb, S1Sh& sh) {
+    const int lane = threadIdx.x & 31;
+    if (ONE || threadIdx.x < 32) {
+        const int per = n >> 5, b0 = lane * per;
+        uint32_t s = 0;
+        for (int t = 0; t < per; t += 4) {
+            const uint4 h = *reinterpret_cast<const uint4*>(hist + b0 + t);
+            s += (h.x + h.y) + (h.z + h.w);
+        }
+        uint32_t x = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += u;
+        }
+        uint32_t c = x - s;
+        if (tb >= c && ta < x) {
+            for (int t = 0; t < per; ++t) {
+                const uint32_t h = hist[b0 + t];
+                if (ta >= c && ta < c + h) {
+                    sh.bin_a = b0 + t;
+                    sh.below_a = c;
+                }
+                if (tb >= c && tb < c + h) sh.bin_b = b0 + t;
+                c += h;
+            }
+        }
+    }
+    cta_sync<ONE>();
+}
+
+// Exact rank-`rank` key over the whole profile by an 8-bit radix select (the
+// rare case: no spread, or a window that could not be placed).  Keys: the
+// value, or with MAD its deviation from the median (float: from mh + ml;
+// int: 2|x - med| with s2 = 2 med).
+template <class V, int R, bool ONE, bool MAD>
+__device__ __noinline__ unsigned long long radix_rank(const unsigned char* smem, uint32_t* hist, S1Sh& sh, int p0,
+                                                      uint32_t rank, float mh, float ml, long long s2) {
+    const int T = ONE ? 32 : (int)blockDim.x, tid = threadIdx.x;
+    unsigned long long prefix = 0, mask = 0;
+    for (int shift = 56; shift >= 0; shift -= 8) {
+        cta_sync<ONE>();
+        for (int b = tid; b < 256; b += T) hist[b] = 0;
+        cta_sync<ONE>();
+        for (int j = tid; j < p0; j += T) {
+            const V v = *reinterpret_cast<const V*>(smem + bin_addr<R>((uint32_t)j));
+            unsigned long long kk;
+            if constexpr (std::is_integral<V>::value) {
+                const long long e = 2 * (long long)v - s2;
+                kk = MAD ? (unsigned long long)(e < 0 ? -e : e) : (unsigned long long)ikey((int32_t)v);
+            } else {
+                float h = (float)v, l = 0.0f;
+                if (MAD) ff_dev((float)v, mh, ml, h, l);
+                kk = ff_key(h, l);
+            }
+            if ((kk & mask) == prefix) atomicAdd(&hist[(kk >> shift) & 0xff], 1u);
+        }
+        cta_sync<ONE>();
+        hist_find<ONE>(hist, 256, rank, rank, sh);
+        rank -= sh.below_a;
+        prefix |= (unsigned long long)sh.bin_a << shift;
+        mask |= 0xffull << shift;
+    }
+    cta_sync<ONE>();
+    return prefix;
+}
+
+// One warp: the values of ranks t1 <= t2 <= t1 + 1 among the n members of a
+// window at `pack` (padded to a multiple of 128 with +inf), all between lo
+// and hi.  MAD: of |x - mh|.  Counting passes at interpolated pivots; each
+// pass also yields the pivot's neighbours on both sides.
+template <bool MAD>
+__device__ __forceinline__ bool pick2(const float* pack, uint32_t n, uint32_t t1, uint32_t t2, float lo, float hi,
+                                      float mh, float& va, float& vb) {
+    const int lane = threadIdx.x & 31;
+    uint32_t cl = 0, ch = n;  // members <= lo, <= hi
+    bool exact = false;       // the pivot is the next member above lo
+    float next = 0.0f;
+    for (int a = 0; a < 24; ++a) {
+        float p;
+        if (exact) {
+            p = next;
+        } else {
+            p = fmaf(__fdividef((float)(2 * (t1 - cl) + 1), (float)(2 * (ch - cl))), hi - lo, lo);
+            if (!(p < hi)) p = lo;
+        }
+        uint32_t c = 0;
+        float above = INFINITY, upto = -INFINITY;
+        for (uint32_t i = 4 * lane; i < n; i += 128) {
+            const float4 q = *reinterpret_cast<const float4*>(pack + i);
+            const float v[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float d = MAD ? fabsf(__fsub_rn(v[e], mh)) : v[e];
+                const bool in = d <= p;
+                c += in;
+                upto = fmaxf(upto, in ? d : -INFINITY);
+                above = fminf(above, in ? INFINITY : d);
+            }
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        above = -warp_max(-above);
+        upto = warp_max(upto);
+        if (c <= t1) {
+            if (c == t1 && t2 == t1) {
+                va = vb = above;
+                return true;
+            }
+            // near the rank, or nothing between the pivot and hi: step to the
+            // next member
+            exact = t1 - c <= 1 || above >= hi || p <= lo;
+            lo = p;
+            cl = c;
+            next = above;
+        } else {
+            if (exact || c == t1 + 1) {
+                va = upto;
+                vb = c > t2 ? upto : above;
+                return true;
+            }
+            hi = upto;
+            ch = c;
+        }
+    }
+    return false;
+}
+
+// R: bins per block.  ONE: the CTA is one warp.
+template <class V, int R, bool ONE, bool FUSED, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB)
+    k_score1(const V* __restrict__ prof_all, const ScoreGroup sg, int64_t m_rows, int64_t trial0, int64_t count,
+             uint32_t wmask, int wtop, const ScoreLay lay, int32_t* d_status) {
+    constexpr bool INT = IsInt<V>::value;
+    constexpr int P = R < 16 ? R : 16;  // bins per item of the width pass
+    constexpr int PARTS = R / P;
+    constexpr int LR = R == 8 ? 3 : (R == 16 ? 4 : 5);
+    constexpr int NS = R == 8 ? 12 : 16;  // widths 2^0 .. 2^(NS-1)
+    constexpr int NB = score_nb(R);
+    constexpr int NP = score_pack(R);
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ S1Sh sh;
+    const int T = ONE ? 32 : (int)blockDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = ONE ? 0 : tid >> 5;
+    const int NW = T >> 5;
+    float2* offs = reinterpret_cast<float2*>(smem + lay.offs);
+    int* offi = reinterpret_cast<int*>(smem + lay.offs);
+    uint32_t* hist = reinterpret_cast<uint32_t*>(smem + lay.aux);
+    float* pack = reinterpret_cast<float*>(smem + lay.aux);
+    auto sync = [&]() { cta_sync<ONE>(); };
+    auto quad = [&](uint32_t a, V (&v)[4]) {
+        *reinterpret_cast<int4*>(v) = *reinterpret_cast<const int4*>(smem + a);
+    };
+    auto value = [&](uint32_t j) -> V { return *reinterpret_cast<const V*>(smem + bin_addr<R>(j)); };
+    // block sums of two counts per thread (one barrier); slot alternates
+    auto sum2 = [&](uint32_t a, uint32_t b, int slot) -> uint2 {
+        a = __reduce_add_sync(0xffffffffu, a);
+        b = __reduce_add_sync(0xffffffffu, b);
+        if (ONE) {
+            __syncwarp();
+            return make_uint2(a, b);
+        }
+        if (lane == 0) sh.wc[slot][warp] = make_uint2(a, b);
+        __syncthreads();
+        const uint2 v = lane < NW ? sh.wc[slot][lane] : make_uint2(0u, 0u);
+        return make_uint2(__reduce_add_sync(0xffffffffu, v.x), __reduce_add_sync(0xffffffffu, v.y));
+    };
+    // this CTA's run of consecutive trials
+    const int64_t it_end = count * (int64_t)(blockIdx.x + 1) / gridDim.x;
+    int64_t it = count * (int64_t)blockIdx.x / gridDim.x;
+    float hint_med = 0.0f, hint_mad = 0.6745f;  // (median - mean) / sigma, MAD / sigma of the trials before
+    int ei = it < it_end ? score_entry(sg, it) : 0;
+    for (; it < it_end; ++it) {
+        if (it >= sg.t0[ei + 1]) ++ei;
+        const int p0 = sg.p0[ei];
+        const int64_t ld = sg.ld[ei];
+        const V* __restrict__ prof = prof_all + sg.off[ei];
+        const int64_t k = trial0 + (it - sg.t0[ei]);
+        const int nblk = (p0 + R - 1) / R;
+        const int next = (1 << wtop) > R ? (1 << wtop) / R : 1;  // extension blocks
+        const int nbx = nblk + next;
+
+        // The in-block prefixes, in place (exclusive within each block) with
+        // the block totals in `offs`: threads first, first + step, ...
+        auto prefix = [&](int first, int step) {
+            for (int b = first; b < nbx; b += step) {
+                const uint32_t a = blk_addr<R>((uint32_t)b);
+                V t = 0;
+#pragma unroll
+                for (int s = 0; s < R / 4; ++s) {
+                    V v[4], c[4];
+                    quad(a ^ (s << 4), v);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        c[i] = t;
+                        t = t + v[i];
+                    }
+                    *reinterpret_cast<int4*>(smem + (a ^ (s << 4))) = *reinterpret_cast<const int4*>(c);
+                }
+                if constexpr (INT) offi[b] = (int)t;
+                else offs[b].x = (float)t;
+            }
+        };
+        bool prefixed = false;
+        float mh = 0.0f, ml = 0.0f;    // float: median = mh + ml
+        float kmh = 0.0f, kml = 0.0f;  // float: MAD = kmh + kml
+        long long s2 = 0, e2 = 0;      // int: 2 * median; 4 * MAD
+        // A second round only if the MAD's pick failed after the prefixes had
+        // replaced the profile (`redo`: the profile again, no windows).
+        for (bool redo = false;; redo = true) {
+        // ---- load; fused last FFA stage: head row k>>1 plus tail row M/2 +
+        // (k>>1) read ceil(k/2) bins further on, four bins at a time.  The
+        // sum, sum of squares and (int) largest |x| accumulate meanwhile.
+        float fs = 0.0f, fq = 0.0f, fm = 0.0f;
+        auto acc = [&](V v) {
+            const float f = (float)v;
+            fs += f;
+            fq = fmaf(f, f, fq);
+            if (INT) fm = fmaxf(fm, fabsf(f));
+        };
+        const bool two = FUSED && m_rows > 1;
+        const V* __restrict__ hrow = prof + (FUSED ? (k >> 1) * ld : k * ld);
+        const V* __restrict__ trow = prof + ((m_rows >> 1) + (k >> 1)) * ld;  // two only
+        const int sft = two ? (int)((uint32_t)((k + 1) >> 1) % (uint32_t)p0) : 0;
+        // pull the next rows towards L2 while this profile is scored (an even
+        // trial's partner reads the same two rows)
+        if (it + 1 < it_end && (FUSED ? (k & 1) && k + 1 < m_rows : true)) {
+            const int lines = (int)((p0 * (int64_t)sizeof(V) + 127) / 128);
+            for (int l = tid; l < lines; l += T) {
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(hrow + ld + l * (128 / sizeof(V))));
+                if (FUSED) asm volatile("prefetch.global.L2 [%0];" ::"l"(trow + ld + l * (128 / sizeof(V))));
+            }
+        }
+        auto store_quad = [&](int q, const V (&v)[4]) {
+            *reinterpret_cast<int4*>(smem + (((uint32_t)q ^ (((uint32_t)q >> 3) & (R / 4 - 1))) << 4)) =
+                *reinterpret_cast<const int4*>(v);
+        };
+        const bool al = ((reinterpret_cast<uintptr_t>(hrow)) & 15) == 0;
+        const int nq4 = p0 >> 2;
+        auto load_head = [&](int q, V (&h)[4]) {
+            if (al) {
+                *reinterpret_cast<int4*>(h) = *reinterpret_cast<const int4*>(hrow + 4 * q);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) h[i] = hrow[4 * q + i];
+            }
+        };
+        if (two) {
+#pragma unroll 4
+            for (int q = tid; q < nq4; q += T) {
+                V h[4], t[4];
+                load_head(q, h);
+                int o = 4 * q + sft;
+                if (o >= p0) o -= p0;
+                if (o + 3 < p0) {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) t[i] = trow[o + i];
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) t[i] = trow[o + i < p0 ? o + i : o + i - p0];
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    h[i] = h[i] + t[i];
+                    acc(h[i]);
+                }
+                store_quad(q, h);
+            }
+        } else {
+#pragma unroll 4
+            for (int q = tid; q < nq4; q += T) {
+                V h[4];
+                load_head(q, h);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc(h[i]);
+                store_quad(q, h);
+            }
+        }
+        if (tid < (p0 & 3)) {
+            const int j = 4 * nq4 + tid;
+            V v = hrow[j];
+            if (two) v = v + trow[j + sft < p0 ? j + sft : j + sft - p0];
+            *reinterpret_cast<V*>(smem + bin_addr<R>(j)) = v;
+            acc(v);
+        }
+        if (INT)
+            for (int b = 4 * tid; b < NB; b += 4 * T) *reinterpret_cast<int4*>(hist + b) = make_int4(0, 0, 0, 0);
+        if (tid < 16) sh.wkey[tid] = 0u;
+        if (tid == 16) sh.pos = 0x7fffffffu;
+        if (tid == 17) sh.npack = 0;
+        if (tid == 18) sh.ncand = 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            fs += __shfl_xor_sync(0xffffffffu, fs, o);
+            fq += __shfl_xor_sync(0xffffffffu, fq, o);
+        }
+        if (INT) fm = warp_max(fm);
+        if (!ONE) {
+            if (lane == 0) {
+                sh.fa[warp] = fs;
+                sh.fb[warp] = fq;
+                if (INT) sh.fc[warp] = fm;
+            }
+            __syncthreads();
+            fs = lane < NW ? sh.fa[lane] : 0.0f;
+            fq = lane < NW ? sh.fb[lane] : 0.0f;
+            if (INT) fm = warp_max(lane < NW ? sh.fc[lane] : 0.0f);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                fs += __shfl_xor_sync(0xffffffffu, fs, o);
+                fq += __shfl_xor_sync(0xffffffffu, fq, o);
+            }
+        } else {
+            __syncwarp();
+        }
+        const float rn = 1.0f / (float)p0;
+        const float mean = fs * rn;
+        const float sig = sqrtf(fmaxf(fmaf(fq, rn, -mean * mean), 0.0f));
+        const float rsn = sqrtf(rn) * sig;  // sigma / sqrt(N)
+        // cyclic extension: bins past p0 repeat the profile
+        bool extended = false;
+        auto extend = [&](int first, int step) {
+            const int ext = nbx * R - p0;
+            for (int j = first; j < ext; j += step) {
+                int s = j;
+                while (s >= p0) s -= p0;  // at most once for profiles longer than the extension
+                *reinterpret_cast<V*>(smem + bin_addr<R>(p0 + j)) = value(s);
+            }
+        };
+
+        // ---- median and MAD (Eq. 3), exact ----
+        const uint32_t r1 = (uint32_t)((p0 - 1) / 2), r2 = (uint32_t)(p0 / 2);
+        // quads entirely inside groups of 32 bins need no bound check
+        const int nq = (p0 >> 5) << 3, jt = (p0 & ~31) + tid;
+        bool spread = !redo && sig > 0.0f && sig < 1e30f;  // windows make sense (block-uniform)
+        if (INT) spread = spread && fm < 5e8f;    // 2 |x| and window sums stay in int32
+        if constexpr (!INT) {
+            mh = ml = 0.0f;
+            // One window [g - r, g + r] after another.  MAD: on |x - mh|.
+            auto select = [&](auto mad_tag, float g, float r, unsigned long long& ka, unsigned long long& kb) -> bool {
+                constexpr bool MAD = decltype(mad_tag)::value;
+                const uint32_t lbase = (uint32_t)__cvta_generic_to_shared(smem) + lay.list + (uint32_t)(tid * lay.cap) * 4u;
+                const uint32_t lim = lbase + (uint32_t)(lay.cap - 1) * 4u;
+                const float* mine = reinterpret_cast<const float*>(smem + lay.list) + tid * lay.cap;
+                for (int a = 0; a < 5; ++a) {
+                    const float lo = g - r, hi = g + r;
+                    uint32_t ptr = lbase, below = 0;
+                    auto take = [&](float v) {
+                        const float d = MAD ? fabsf(__fsub_rn(v, mh)) : v;
+                        asm volatile(
+                            "{\n\t.reg .pred p, q;\n\t"
+                            "setp.lt.f32 p, %2, %3;\n\t"
+                            "setp.le.and.f32 q, %2, %4, !p;\n\t"
+                            "@p add.u32 %1, %1, 1;\n\t"
+                            "@q st.shared.f32 [%0], %5;\n\t"
+                            "@q add.u32 %0, %0, 4;\n\t"
+                            "@q min.u32 %0, %0, %6;\n\t}"
+                            : "+r"(ptr), "+r"(below)
+                            : "f"(d), "f"(lo), "f"(hi), "f"(v), "r"(lim));
+                    };
+                    for (int q = tid; q < nq; q += T) {
+                        V v[4];
+                        quad((uint32_t)q << 4, v);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) take(v[i]);
+                    }
+                    for (int j = jt; j < p0; j += T) take(value(j));
+                    // pack the threads' lists
+                    const uint32_t nl = (ptr - lbase) >> 2;
+                    if (nl) {
+                        const uint32_t at = atomicAdd(&sh.npack, nl);
+                        if (at + nl <= NP)
+                            for (uint32_t i = 0; i < nl; ++i) pack[at + i] = mine[i];
+                    }
+                    const uint2 c = sum2(below + (ptr == lim ? 1u << 17 : 0u), nl, a & 1);
+                    const uint32_t cl = c.x & 0x1ffffu;
+                    if (c.x >> 17 || c.y > NP) {  // a thread's list, or the packed one, overflowed
+                        if (tid == 0) sh.npack = 0;
+                        r *= 0.5f;
+                        sync();
+                        continue;
+                    }
+                    if (r1 < cl || r2 >= cl + c.y) {
+                        const float dens = fmaxf((float)c.y, 1.0f) / (2.0f * r);
+                        if (r1 < cl) g -= r + (float)(cl - r1) / dens;
+                        else g += r + (float)(r2 + 1 - cl - c.y) / dens;
+                        r *= 1.5f;
+                        if (tid == 0) sh.npack = 0;
+                        sync();
+                        continue;
+                    }
+                    if (warp == 0) {
+                        // pad, pick, then settle near-ties exactly
+                        const uint32_t n = c.y, t1 = r1 - cl, t2 = r2 - cl;
+                        for (uint32_t i = n + lane; i < ((n + 127) & ~127u); i += 32) pack[i] = INFINITY;
+                        __syncwarp();
+                        float va, vb;
+                        int ok = pick2<MAD>(pack, n, t1, t2, lo, hi, mh, va, vb);
+                        if constexpr (!MAD) {
+                            if (lane == 0) {
+                                sh.key[0] = ff_key(va, 0.0f);
+                                sh.key[1] = ff_key(vb, 0.0f);
+                            }
+                        } else if (ok) {
+                            // |x - mh| in FP32 is within E of the exact
+                            // deviation: the wanted ranks are among the members
+                            // within 2 E of va, vb; rank those exactly
+                            const float E = (hi + fabsf(mh)) * 1.2e-7f;
+                            const float ca = va - 3.0f * E, cb = vb + 3.0f * E;
+                            uint32_t less = 0;
+                            for (uint32_t i = lane; i < n; i += 32) {
+                                const float v = pack[i], d = fabsf(__fsub_rn(v, mh));
+                                less += d < ca;
+                                if (d >= ca && d <= cb) {
+                                    const uint32_t s = atomicAdd(&sh.ncand, 1u);
+                                    float h, l;
+                                    ff_dev(v, mh, ml, h, l);
+                                    if (s < S1_NC) sh.cand[s] = ff_key(h, l);
+                                }
+                            }
+                            less = __reduce_add_sync(0xffffffffu, less);
+                            __syncwarp();
+                            const uint32_t m = sh.ncand;
+                            if (m > S1_NC || ca < lo || cb > hi) {  // too many, or too near the window's edge
+                                ok = 0;
+                            } else {
+                                for (uint32_t i = lane; i < m; i += 32) {
+                                    const unsigned long long ki = sh.cand[i];
+                                    uint32_t rk = 0;
+                                    for (uint32_t j = 0; j < m; ++j) {
+                                        const unsigned long long kj = sh.cand[j];
+                                        rk += (kj < ki) || (kj == ki && j < i);
+                                    }
+                                    if (rk == t1 - less) sh.key[0] = ki;
+                                    if (rk == t2 - less) sh.key[1] = ki;
+                                }
+                            }
+                        }
+                        if (lane == 0) {
+                            sh.ok = ok;
+                            sh.npack = 0;
+                            sh.ncand = 0;
+                        }
+                    } else if (!ONE) {  // meanwhile
+                        if (MAD) prefix(tid - 32, T - 32);
+                        else extend(tid - 32, T - 32);
+                    }
+                    if (!ONE) (MAD ? prefixed : extended) = true;
+                    sync();
+                    ka = sh.key[0];
+                    kb = sh.key[1];
+                    return sh.ok != 0;
+                }
+                return false;
+            };
+            unsigned long long ka = 0, kb = 0;
+            bool done = false;
+            if (spread) done = select(std::false_type{}, fmaf(hint_med, sig, mean), 3.2f * rsn, ka, kb);
+            if (!done) {
+                ka = radix_rank<V, R, ONE, false>(smem, hist, sh, p0, r1, 0.0f, 0.0f, 0);
+                kb = r1 == r2 ? ka : radix_rank<V, R, ONE, false>(smem, hist, sh, p0, r2, 0.0f, 0.0f, 0);
+            }
+            // the median as a float pair: (a + b) / 2 exactly
+            {
+                const float a = fkey_inv((uint32_t)(ka >> 32)), b = fkey_inv((uint32_t)(kb >> 32));
+                if (r1 == r2) {
+                    mh = a;
+                } else {
+                    two_sum(a, b, mh, ml);
+                    mh *= 0.5f;
+                    ml *= 0.5f;
+                }
+            }
+            if (!extended) {  // read after the barriers of the MAD's selection
+                extend(tid, T);
+                extended = true;
+            }
+            done = false;
+            if (spread) done = select(std::true_type{}, hint_mad * sig, 2.6f * rsn, ka, kb);
+            if (!done && prefixed) {  // the profile is gone: once more
+                prefixed = false;
+                sync();
+                continue;
+            }
+            if (!done) {
+                ka = radix_rank<V, R, ONE, true>(smem, hist, sh, p0, r1, mh, ml, 0);
+                kb = r1 == r2 ? ka : radix_rank<V, R, ONE, true>(smem, hist, sh, p0, r2, mh, ml, 0);
+            }
+            kmh = fkey_inv((uint32_t)(ka >> 32));
+            kml = fkey_inv((uint32_t)ka);
+            if (r1 != r2) {
+                ff_acc(kmh, kml, fkey_inv((uint32_t)(kb >> 32)), fkey_inv((uint32_t)kb));
+                ff_norm(kmh, kml);
+                kmh *= 0.5f;
+                kml *= 0.5f;
+            }
+            if (spread) {
+                const float is = 1.0f / sig;
+                hint_med += 0.3f * ((mh - mean) * is - hint_med);
+                hint_mad += 0.3f * (kmh * is - hint_mad);
+            }
+        } else {
+            extend(tid, T);  // read after the barriers of the selections
+            extended = true;
+            // Int profiles: a window of at most NB consecutive integers (of
+            // the value, or of the deviation 2|x - med| in steps of two), one
+            // bucket each, so that the bucket is the value.
+            auto select = [&](auto mad_tag, int lo, int width, long long& va, long long& vb) -> bool {
+                constexpr bool MAD = decltype(mad_tag)::value;
+                const int m2 = (int)s2;
+                for (int a = 0; a < 5; ++a) {
+                    if (MAD || a > 0) {
+                        for (int b = 4 * tid; b < NB; b += 4 * T)
+                            *reinterpret_cast<int4*>(hist + b) = make_int4(0, 0, 0, 0);
+                        sync();
+                    }
+                    uint32_t below = 0, in = 0;
+                    auto take = [&](int v) {
+                        const int e = MAD ? abs(2 * v - m2) : v;
+                        const uint32_t t = (uint32_t)(e - lo) >> (MAD ? 1 : 0);
+                        if (e < lo) ++below;
+                        else if (t < (uint32_t)width) {
+                            atomicAdd(&hist[t], 1u);
+                            ++in;
+                        }
+                    };
+                    for (int q = tid; q < nq; q += T) {
+                        V v[4];
+                        quad((uint32_t)q << 4, v);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) take((int)v[i]);
+                    }
+                    for (int j = jt; j < p0; j += T) take((int)value(j));
+                    const uint2 c = sum2(below, in, a & 1);
+                    if (r1 < c.x || r2 >= c.x + c.y) {
+                        const int step = MAD ? 2 : 1;
+                        const float dens = fmaxf((float)c.y, 1.0f) / (float)width;
+                        const float miss = r1 < c.x ? (float)(c.x - r1) : (float)(r2 + 1 - c.x - c.y);
+                        const int move = step * (int)fminf((float)(width / 2) + miss / dens, 1e8f);
+                        lo += r1 < c.x ? -move : move;
+                        width = width + width / 2 < NB ? width + width / 2 : NB;
+                        if (lo < -1000000000 || lo > 1000000000) return false;
+                        sync();  // hist complete before it is cleared
+                        continue;
+                    }
+                    hist_find<ONE>(hist, NB, r1 - c.x, r2 - c.x, sh);
+                    va = lo + (MAD ? 2 : 1) * sh.bin_a;
+                    vb = lo + (MAD ? 2 : 1) * sh.bin_b;
+                    return true;
+                }
+                return false;
+            };
+            long long va = 0, vb = 0;
+            bool done = false;
+            if (spread) {
+                const int r = 1 + (int)fminf(3.2f * rsn, (float)(NB / 2 - 2));
+                done = select(std::false_type{}, __float2int_rn(fmaf(hint_med, sig, mean)) - r, 2 * r + 1, va, vb);
+            }
+            if (!done) {
+                auto rank = [&](uint32_t r) -> long long {
+                    return (int32_t)((uint32_t)radix_rank<V, R, ONE, false>(smem, hist, sh, p0, r, 0.0f, 0.0f, 0) ^ 0x80000000u);
+                };
+                va = rank(r1);
+                vb = r1 == r2 ? va : rank(r2);
+            }
+            s2 = va + vb;
+            sync();  // hist and bin_a read by all
+            done = false;
+            long long ea = 0, eb = 0;
+            if (spread) {
+                const int r = 1 + (int)fminf(2.6f * rsn, (float)(NB / 2 - 2));
+                int lo = 2 * (__float2int_rn(hint_mad * sig) - r);
+                if (lo < 0) lo = 0;
+                lo += (int)(s2 & 1);  // deviations 2|x - med| have s2's parity
+                done = select(std::true_type{}, lo, 2 * r + 1, ea, eb);
+            }
+            if (!done) {
+                ea = (long long)radix_rank<V, R, ONE, true>(smem, hist, sh, p0, r1, 0.0f, 0.0f, s2);
+                eb = r1 == r2 ? ea : (long long)radix_rank<V, R, ONE, true>(smem, hist, sh, p0, r2, 0.0f, 0.0f, s2);
+            }
+            e2 = ea + eb;
+            if (spread) {
+                const float is = 1.0f / sig;
+                hint_med += 0.3f * ((0.5f * (float)s2 - mean) * is - hint_med);
+                hint_mad += 0.3f * (0.25f * (float)e2 * is - hint_mad);
+            }
+        }
+        break;
+        }
+        if (!prefixed) sync();  // the window list gives way to the offsets
+
+        if (!prefixed) {
+            prefix(tid, T);
+            sync();
+        }
+        // block offsets: exclusive scan of the totals, in segments of 128
+        // blocks (four per lane; the same tree whatever the CTA's size)
+        {
+            const int nseg = (nbx + 127) >> 7;
+            float ch = 0.0f, cl = 0.0f;  // ONE: carry
+            uint32_t ci = 0;
+            for (int sgm = warp; sgm < nseg; sgm += NW) {
+                const int b0 = (sgm << 7) + 4 * lane;
+                if constexpr (INT) {
+                    uint32_t v[4], s = 0;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) v[i] = b0 + i < nbx ? (uint32_t)offi[b0 + i] : 0u;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const uint32_t u = v[i];
+                        v[i] = s;
+                        s += u;
+                    }
+                    uint32_t x = s;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const uint32_t u = __shfl_up_sync(0xffffffffu, x, o);
+                        if (lane >= o) x += u;
+                    }
+                    const uint32_t ex = x - s + ci;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (b0 + i < nbx) offi[b0 + i] = (int)(ex + v[i]);
+                    const uint32_t tot = __shfl_sync(0xffffffffu, x, 31);
+                    if (ONE) ci += tot;
+                    else if (lane == 0) sh.seg[sgm].x = __uint_as_float(tot);
+                } else {
+                    float v[4], h[4], l[4], sh_ = 0.0f, sl = 0.0f;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) v[i] = b0 + i < nbx ? offs[b0 + i].x : 0.0f;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        h[i] = sh_;
+                        l[i] = sl;
+                        ff_acc(sh_, sl, v[i], 0.0f);
+                    }
+                    float xh = sh_, xl = sl;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const float uh = __shfl_up_sync(0xffffffffu, xh, o);
+                        const float ul = __shfl_up_sync(0xffffffffu, xl, o);
+                        if (lane >= o) ff_acc(xh, xl, uh, ul);
+                    }
+                    ff_norm(xh, xl);
+                    float eh = __shfl_up_sync(0xffffffffu, xh, 1), el = __shfl_up_sync(0xffffffffu, xl, 1);
+                    if (lane == 0) eh = el = 0.0f;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        ff_acc(h[i], l[i], eh, el);
+                        ff_norm(h[i], l[i]);
+                        if (ONE) {
+                            ff_acc(h[i], l[i], ch, cl);
+                            ff_norm(h[i], l[i]);
+                        }
+                        if (b0 + i < nbx) offs[b0 + i] = make_float2(h[i], l[i]);
+                    }
+                    const float th = __shfl_sync(0xffffffffu, xh, 31), tl = __shfl_sync(0xffffffffu, xl, 31);
+                    if (ONE) {
+                        ff_acc(ch, cl, th, tl);
+                        ff_norm(ch, cl);
+                    } else if (lane == 0) {
+                        sh.seg[sgm] = make_float2(th, tl);
+                    }
+                }
+            }
+            sync();
+            if (!ONE && nseg > 1) {
+                // add the earlier segments' totals
+                for (int sgm = warp ? warp : NW; sgm < nseg; sgm += NW) {
+                    if constexpr (INT) {
+                        uint32_t base = 0;
+                        for (int i = 0; i < sgm; ++i) base += __float_as_uint(sh.seg[i].x);
+                        for (int b = (sgm << 7) + lane; b < nbx && b < (sgm + 1) << 7; b += 32)
+                            offi[b] = (int)((uint32_t)offi[b] + base);
+                    } else {
+                        float bh = 0.0f, bl = 0.0f;
+                        for (int i = 0; i < sgm; ++i) {
+                            const float2 t = sh.seg[i];
+                            ff_acc(bh, bl, t.x, t.y);
+                            ff_norm(bh, bl);
+                        }
+                        for (int b = (sgm << 7) + lane; b < nbx && b < (sgm + 1) << 7; b += 32) {
+                            float2 o = offs[b];
+                            ff_acc(o.x, o.y, bh, bl);
+                            ff_norm(o.x, o.y);
+                            offs[b] = o;
+                        }
+                    }
+                }
+                __syncthreads();
+            }
+        }
+
+        // ---- widths: the largest box of each, per thread ----
+        auto boff = [&](int b) {
+            if constexpr (INT) return offi[b];
+            else return offs[b];
+        };
+        auto bdiff = [&](auto o2, auto o1) -> V {
+            if constexpr (INT) return (V)((uint32_t)o2 - (uint32_t)o1);
+            else return __fadd_rn(__fsub_rn(o2.x, o1.x), __fsub_rn(o2.y, o1.y));
+        };
+        auto sub = [](V a, V b) -> V {
+            if constexpr (INT) return (V)((uint32_t)a - (uint32_t)b);
+            else return __fsub_rn(a, b);
+        };
+        auto add = [](V a, V b) -> V {
+            if constexpr (INT) return (V)((uint32_t)a + (uint32_t)b);
+            else return __fadd_rn(a, b);
+        };
+        V lowest;
+        if constexpr (INT) lowest = INT32_MIN;
+        else lowest = -INFINITY;
+        V M[NS];
+#pragma unroll
+        for (int n = 0; n < NS; ++n) M[n] = lowest;
+        const int nitem = nblk * PARTS;
+        for (int im = tid; im < nitem; im += T) {
+            const int b = im / PARTS, hf = im % PARTS;
+            const uint32_t a = blk_addr<R>((uint32_t)b) ^ (uint32_t)(hf * (P * 4));
+            const auto o1 = boff(b);
+            V c[P];
+#pragma unroll
+            for (int s = 0; s < P / 4; ++s) quad(a ^ (s << 4), *reinterpret_cast<V(*)[4]>(&c[4 * s]));
+            // the next part: the same block's (offset 0), or the next block's
+            const bool last = hf == PARTS - 1;
+            const uint32_t an = last ? blk_addr<R>((uint32_t)b + 1) : a ^ (uint32_t)(P * 4);
+            V xd = 0;
+            if (last) xd = bdiff(boff(b + 1), o1);
+            if (wmask & 15u) {
+                V nx[8];
+                quad(an, *reinterpret_cast<V(*)[4]>(&nx[0]));
+                if (R > 8) quad(an ^ 16, *reinterpret_cast<V(*)[4]>(&nx[4]));
+#pragma unroll
+                for (int n = 0; n < 4; ++n) {
+                    if ((1 << n) >= R || !(wmask >> n & 1u)) continue;
+                    const int w = 1 << n;
+                    V m = lowest, mx = lowest;
+#pragma unroll
+                    for (int r = 0; r + w < P; r += 2) {
+                        if (r + 1 + w < P) m = max3(m, sub(c[r + w], c[r]), sub(c[r + 1 + w], c[r + 1]));
+                        else m = max3(m, m, sub(c[r + w], c[r]));
+                    }
+#pragma unroll
+                    for (int i = 0; i < w; i += 2) {
+                        if (i + 1 < w) mx = max3(mx, sub(nx[i], c[P - w + i]), sub(nx[i + 1], c[P - w + i + 1]));
+                        else mx = max3(mx, mx, sub(nx[i], c[P - w + i]));
+                    }
+                    M[n] = max3(M[n], m, add(xd, mx));
+                }
+            }
+            if (R == 32 && (wmask >> 4 & 1u)) {  // width 16 = one part further on
+                V m = lowest;
+#pragma unroll
+                for (int s = 0; s < P / 4; ++s) {
+                    V v[4];
+                    quad(an ^ (s << 4), v);
+                    m = max3(m, sub(v[0], c[4 * s]), sub(v[1], c[4 * s + 1]));
+                    m = max3(m, sub(v[2], c[4 * s + 2]), sub(v[3], c[4 * s + 3]));
+                }
+                M[4] = max3(M[4], M[4], add(xd, m));
+            }
+#pragma unroll
+            for (int n = LR; n < NS; ++n) {
+                if (!(wmask >> n & 1u)) continue;
+                const int d = 1 << (n - LR);
+                // eight or more blocks on, the swizzle is the same
+                const uint32_t a2 = d >= 8 ? a + (uint32_t)(d * R * 4)
+                                           : blk_addr<R>((uint32_t)(b + d)) ^ (uint32_t)(hf * (P * 4));
+                const V D = bdiff(boff(b + d), o1);
+                V m = lowest;
+#pragma unroll
+                for (int s = 0; s < P / 4; ++s) {
+                    V v[4];
+                    quad(d >= 8 ? (a ^ (s << 4)) + (uint32_t)(d * R * 4) : a2 ^ (s << 4), v);
+                    if constexpr (INT) {
+                        m = max3(m, sub(v[0], c[4 * s]), sub(v[1], c[4 * s + 1]));
+                        m = max3(m, sub(v[2], c[4 * s + 2]), sub(v[3], c[4 * s + 3]));
+                    } else {
+                        float d0, d1, d2, d3;
+                        asm("{\n\t.reg .b64 x, y, z;\n\t"
+                            "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+                            : "=f"(d0), "=f"(d1)
+                            : "f"(v[0]), "f"(v[1]), "f"(c[4 * s]), "f"(c[4 * s + 1]));
+                        asm("{\n\t.reg .b64 x, y, z;\n\t"
+                            "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+                            : "=f"(d2), "=f"(d3)
+                            : "f"(v[2]), "f"(v[3]), "f"(c[4 * s + 2]), "f"(c[4 * s + 3]));
+                        m = max3(m, d0, d1);
+                        m = max3(m, d2, d3);
+                    }
+                }
+                M[n] = max3(M[n], M[n], add(D, m));
+            }
+        }
+        // lane n of each warp: the warp's maximum of width 2^n; then the CTA's
+        uint32_t wk = 0;
+#pragma unroll
+        for (int n = 0; n < NS; ++n) {
+            const V m = warp_max(M[n]);  // (widths not asked for: the lowest value)
+            wk = lane == n ? (uint32_t)as_bits(m) : wk;
+        }
+        if constexpr (INT) wk = ikey((int32_t)wk);
+        else wk = fkey(__uint_as_float(wk));
+        if (!ONE) {
+            if (lane < 16 && (wmask >> lane & 1u)) atomicMax(&sh.wkey[lane], wk);
+            __syncthreads();
+        }
+        // ---- S/N_w = (B_w - w*med) / (K*MAD*sqrt(w)) for w = 2^n in lane n of
+        // warp 0; the best, ties to the smaller width.  sqrt(w) is 2^(n/2), or
+        // 2^((n-1)/2) times the rounded sqrt(2).
+        bool madpos;
+        if constexpr (INT) madpos = e2 > 0;
+        else madpos = kmh > 0.0f || kml > 0.0f;
+        if (warp == 0) {
+            if (!ONE) wk = lane < 16 ? sh.wkey[lane] : 0u;
+            const bool on = lane < 16 && (wmask >> (lane & 15) & 1u);
+            const int n = lane & 15;
+            float key = -INFINITY;
+            if constexpr (INT) {
+                // 2 * (B - w * med) is an exact integer
+                const long long num2 = 2 * (long long)(int32_t)(wk ^ 0x80000000u) - ((long long)s2 << n);
+                // 1/sqrt(w): 2^(-n/2) for even n, else 2^(-(n-1)/2)/sqrt(2)
+                const float rs = __int_as_float((127 - (n >> 1)) << 23) * ((n & 1) ? 0.70710678f : 1.0f);
+                if (on) key = 0.5f * __ll2float_rn(num2) * rs;
+            } else {
+                // numerator in float-float (w * mh, w * ml exact: w is a power
+                // of two), K * MAD in float-float rounded once, one division
+                constexpr float KH = (float)KMAD, KL = (float)(KMAD - (double)KH);
+                const float ph = __fmul_rn(kmh, KH);
+                const float pl = __fadd_rn(__fmaf_rn(kmh, KH, -ph), __fmaf_rn(kmh, KL, __fmul_rn(kml, KH)));
+                const float kf = __fadd_rn(ph, pl);
+                const float w = (float)(1 << n);
+                float hi, lo;
+                two_sum(fkey_inv(wk), -(w * mh), hi, lo);
+                const float num = __fadd_rn(hi, __fsub_rn(lo, w * ml));
+                if (on) key = __fdiv_rn(num, __fmul_rn(kf, sqrt_pow2(n)));
+            }
+            int bw = on ? n : 31;
+            float bk = key;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float ok = __shfl_xor_sync(0xffffffffu, bk, o);
+                const int ob = __shfl_xor_sync(0xffffffffu, bw, o);
+                if (ok > bk || (ok == bk && ob < bw)) {
+                    bk = ok;
+                    bw = ob;
+                }
+            }
+            if (bw > 15) bw = __ffs(wmask) - 1;  // every score NaN
+            if constexpr (INT) {
+                if (lane == bw) {
+                    const double num = __dmul_rn(
+                        0.5, (double)(2 * (long long)(int32_t)(wk ^ 0x80000000u) - ((long long)s2 << n)));
+                    const double kmad = __dmul_rn(KMAD, (double)e2 * 0.25);
+                    constexpr double SQRT2 = 1.4142135623730951;  // sqrt(2) rounded to nearest
+                    const double sq = __dmul_rn((double)(1 << (n >> 1)), (n & 1) ? SQRT2 : 1.0);
+                    sh.best = __double2float_rn(__ddiv_rn(num, __dmul_rn(kmad, sq)));
+                }
+            } else if (lane == bw) {
+                sh.best = bk;
+            }
+            if (lane == 0) sh.bw = bw;
+            if (ONE && lane == bw) sh.wkey[bw] = wk;
+        }
+        sync();
+        // ---- first argmax of the winning width, recomputed bit-identically
+        // in the threads whose own maximum is the CTA's: a warp takes such a
+        // thread's items together, one bin per lane
+        const int bw = sh.bw;
+        if (madpos) {
+            V target;
+            if constexpr (INT) target = (V)(int32_t)(sh.wkey[bw] ^ 0x80000000u);
+            else target = (V)fkey_inv(sh.wkey[bw]);
+            V own = lowest;
+#pragma unroll
+            for (int n = 0; n < NS; ++n)
+                if (n == bw) own = M[n];
+            const int w = 1 << bw;
+            unsigned who = __ballot_sync(0xffffffffu, own == target && tid < nitem);
+            while (who) {
+                const int src = warp * 32 + __ffs(who) - 1;
+                who &= who - 1;
+                const int nk = (nitem - src + T - 1) / T;
+                for (int i0 = 0; i0 < nk; i0 += 32 / P) {
+                    const int im = src + (i0 + lane / P) * T;
+                    uint32_t f = 0x7fffffffu;
+                    if (im < nitem) {
+                        const int b = im / PARTS, r = (im % PARTS) * P + lane % P;
+                        const int j = b * R + r, b2 = (j + w) / R;
+                        V bx = sub(value(j + w), value(j));
+                        if (b2 != b) bx = add(bdiff(boff(b2), boff(b)), bx);
+                        if (bx == target) f = (uint32_t)(j < p0 ? j : j % p0);
+                    }
+                    f = __reduce_min_sync(0xffffffffu, f);
+                    if (lane == 0 && f != 0x7fffffffu) atomicMin(&sh.pos, f);
+                }
+            }
+        }
+        sync();
+        if (tid == 0) {
+            ffa_record out;
+            if (!madpos) {
+                out.snr = 0.0f;
+                out.width = wmask & (0u - wmask);
+                out.phase = 0;
+                out.flags = 1;
+            } else {
+                const uint32_t pos = sh.pos;
+                out.snr = sh.best;
+                out.width = 1 << bw;
+                out.phase = pos == 0x7fffffffu ? 0 : (int32_t)pos;
+                out.flags = 0;
+                if (pos == 0x7fffffffu) dev_fail(d_status, FFA_ERR_DEVICE);
+            }
+            sg.rec[ei][it - sg.t0[ei]] = out;
+        }
+        sync();
+    }
+}
+
+
+// ---- launches -----------------------------------------------------------------
+
+// The CTA for profiles of up to p0 bins in blocks of R: threads, shared
+// memory.  The width pass deals out items of min(R, 16) bins, so the thread
+// count divides them into whole rounds.
+template <class V, int R>
+void score1_shape(int64_t p0, int wtop, int rounds, int tmin, int tmax, int cap, int* threads, ScoreLay* lay, size_t* smem) {
+    const int64_t nblk = (p0 + R - 1) / R;
+    const int64_t nbx = nblk + ((1 << wtop) > R ? (1 << wtop) / R : 1);
+    const int64_t items = nblk * (R / (R < 16 ? R : 16));
+    int64_t t = ((items + rounds - 1) / rounds + 31) / 32 * 32;
+    t = t < tmin ? tmin : (t > tmax ? tmax : t);
+    *threads = (int)t;
+    size_t off = (size_t)nbx * R * 4;
+    lay->cap = cap;
+    lay->offs = lay->list = (uint32_t)off;
+    const size_t offs = (size_t)nbx * (std::is_integral<V>::value ? 4 : 8);
+    const size_t list = std::is_integral<V>::value ? 0 : (size_t)t * (size_t)lay->cap * 4;
+    off += ((offs > list ? offs : list) + 15) & ~(size_t)15;
+    lay->aux = (uint32_t)off;
+    *smem = off + 4 * (std::is_integral<V>::value ? score_nb(R) : score_pack(R));
+}
+
+template <class V, int R, bool ONE, bool FF, int MAXT, int MINB>
+ffa_status score1_launch(const void* d_prof, const ScoreGroup& sg, int64_t count, int64_t trial0, int64_t m_rows,
+                         uint32_t wmask, int wtop, int threads, const ScoreLay& lay, size_t smem, int32_t* d_status,
+                         cudaStream_t st) {
+    const void* fn = (const void*)k_score1<V, R, ONE, FF, MAXT, MINB>;
+    if (smem + sizeof(S1Sh) > 227 * 1024) return fail(FFA_ERR_UNSUPPORTED, "score: profile too long for shared memory");
+    ffa_status es = ensure_smem(fn, smem);
+    if (es != FFA_OK) return es;
+    int64_t resident = 0;  // persistent: every CTA resident
+    es = resident_ctas(fn, threads, smem, &resident);
+    if (es != FFA_OK) return es;
+    const unsigned grid = (unsigned)(count < resident ? count : resident);
+    k_score1<V, R, ONE, FF, MAXT, MINB>
+        <<<grid, threads, smem, st>>>((const V*)d_prof, sg, m_rows, trial0, count, wmask, wtop, lay, d_status);
+    FFA_LAUNCH_CHECK("k_score1");
+    count_launch();
+    return FFA_OK;
+}
+
+// p0: the longest profile of the group
+template <class V, bool FF>
+ffa_status score1_t(const void* d_prof, const ScoreGroup& sg, int64_t count, int64_t trial0, int64_t p0,
+                    int64_t m_rows, const ScoreWidths& wd, int32_t* d_status, cudaStream_t st) {
+    uint32_t wmask = 0;
+    int wtop = 0;
+    for (int i = 0; i < wd.n; ++i) {
+        int n = 0;
+        while ((1 << n) < wd.w[i]) ++n;
+        wmask |= 1u << n;
+        wtop = n > wtop ? n : wtop;
+    }
+    int threads = 0;
+    ScoreLay lay;
+    size_t smem = 0;
+#define FFA_SCORE1(RR, ONE, MAXT, MINB)                                                                          \
+    score1_launch<V, RR, ONE, FF, MAXT, MINB>(d_prof, sg, count, trial0, m_rows, wmask, wtop, threads, lay, smem, \
+                                              d_status, st)
+    // CTA shapes, measured with ready profiles of 366..30000 bins: threads
+    // against registers.  Fewer threads that hold their item in registers
+    // beat more threads that spill (20000 bins: 27.7k SM cycles a profile
+    // with 448 threads of 72 registers, 35.7k with 640 of 48).
+    switch (score_shape(p0, wd.w[wd.n - 1])) {
+        case 0:
+            // one warp a profile up to 1200 bins (1100 bins: 2.1k SM cycles,
+            // 2.7k with two warps; 366 bins: 1.2k and 2.2k), two above
+            // (1900 bins: 3.6k and 3.7k)
+            if (p0 <= 1200) {
+                score1_shape<V, 8>(p0, wtop, 1, 32, 32, 13, &threads, &lay, &smem);
+                return FFA_SCORE1(8, true, 32, 24);
+            }
+            score1_shape<V, 8>(p0, wtop, 3, 64, 64, 9, &threads, &lay, &smem);
+            return FFA_SCORE1(8, false, 64, 12);
+        case 1:
+        case 2:
+            score1_shape<V, 16>(p0, wtop, p0 <= 10240 ? 3 : 2, 64, 384, 9, &threads, &lay, &smem);
+            return FFA_SCORE1(16, false, 384, 2);
+        default:
+            // two profiles an SM while their shared memory fits, else one
+            score1_shape<V, 32>(p0, wtop, 3, 320, 448, 7, &threads, &lay, &smem);
+            if (2 * (smem + sizeof(S1Sh) + 1024) <= 228 * 1024) return FFA_SCORE1(32, false, 448, 2);
+            score1_shape<V, 32>(p0, wtop, 3, 512, 640, 9, &threads, &lay, &smem);
+            return FFA_SCORE1(32, false, 640, 1);
+    }
+#undef FFA_SCORE1
+}
+
+ffa_status score1_dispatch(const void* d_prof, const ScoreGroup& sg, int32_t precision, bool fused, int64_t count,
+                           int64_t trial0, int64_t p0max, int64_t m_rows, const ScoreWidths& wd, int32_t* d_status,
+                           cudaStream_t st) {
+    if (count <= 0) return FFA_OK;
+    if (score_shape(p0max, wd.w[wd.n - 1]) < 0)
+        return fail(FFA_ERR_UNSUPPORTED, "score: profile longer than 32768 bins");
+    if (precision == FFA_FOLD_F32)
+        return fused ? score1_t<float, true>(d_prof, sg, count, trial0, p0max, m_rows, wd, d_status, st)
+                     : score1_t<float, false>(d_prof, sg, count, trial0, p0max, m_rows, wd, d_status, st);
+    return fused ? score1_t<int32_t, true>(d_prof, sg, count, trial0, p0max, m_rows, wd, d_status, st)
+                 : score1_t<int32_t, false>(d_prof, sg, count, trial0, p0max, m_rows, wd, d_status, st);
+}
+
+}  // namespace
+
+ffa_status launch_score2(const void* d_prof, int32_t precision, bool fused, int64_t count, int64_t trial0, int64_t p0,
+                         int64_t ld, int64_t m_rows, const ScoreWidths& wd, ffa_record* d_rec, int32_t* d_status,
+                         cudaStream_t st) {
+    return score1_dispatch(d_prof, score_single(p0, ld, count, d_rec), precision, fused, count, trial0, p0, m_rows, wd,
+                           d_status, st);
+}
+
+ffa_status launch_score2_group(const void* d_plane, int32_t precision, int n, const int64_t* p0, const int64_t* off,
+                               int64_t m_rows, const ScoreWidths& wd, ffa_record* const* recs, int32_t* d_status,
+                               cudaStream_t st) {
+    if (n < 1 || n > FOLD_GROUP_MAX) return fail(FFA_ERR_ARG, "score group: 1..FOLD_GROUP_MAX base periods");
+    int64_t p0max = 0;
+    const ScoreGroup sg = score_group(n, p0, off, m_rows, recs, &p0max);
+    return score1_dispatch(d_plane, sg, precision, true, (int64_t)n * m_rows, 0, p0max, m_rows, wd, d_status, st);
+}
+
+}  // namespace ffa
