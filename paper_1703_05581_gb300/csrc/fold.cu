@@ -29,6 +29,7 @@
 #include <mutex>
 #include <tuple>
 #include <type_traits>
+#include <utility>
 
 #include "common.cuh"
 #include "internal.h"
@@ -86,97 +87,48 @@ __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Stage `wt` cyclic columns of a row starting at column `base` (< p0) into
-// shared memory (one warp per row); returns the element offset (0..3) of
-// logical column 0 in rowp (16-byte aligned).  A segment that does not wrap
-// is copied as whole 16-byte chunks from its aligned-down start, so the
-// offset is its misalignment; the chunk holding the segment's last element
-// ends within that element's 16-byte block, so nothing outside it is read.
-// A wrapping segment (or a row shorter than the segment) is copied element
-// by element at offset 0, int8 rows are widened to int32 through registers
-// (whole 4-byte words when the segment does not wrap), and rows at or beyond
-// m_data (live == false) are zero.
+// shared memory at rowp[off ...] (one warp per row), element by element: the
+// rows that wrap past p0, that do not start at alignment `off`, or that are
+// shorter than the segment.
 template <class T, class S>
-__device__ __forceinline__ int stage_row(T* __restrict__ rowp, const S* __restrict__ src, int64_t base,
-                                         int64_t p0, int wt, bool live, int lane) {
-    if (!live) {
-        for (int x = 4 * lane; x < wt; x += 128) *reinterpret_cast<int4*>(rowp + x) = make_int4(0, 0, 0, 0);
-        return 0;
-    }
-    if constexpr (sizeof(T) == sizeof(S)) {
-        if (base + wt <= p0) {
-            const S* g = src + base;
-            const int a = (int)(((uintptr_t)g >> 2) & 3);
-            const S* g0 = g - a;
-            const int nc = (wt + a + 3) >> 2;
-            for (int k = lane; k < nc; k += 32) cp_async16(rowp + 4 * k, g0 + 4 * k);
-            return a;
-        }
-        if (wt <= p0) {
-            const int n1 = (int)(p0 - base);  // columns before the wrap
-            const S* a = src + base;
-            for (int x = lane; x < n1; x += 32) cp_async4(rowp + x, a + x);
-            for (int x = n1 + lane; x < wt; x += 32) cp_async4(rowp + x, src + (x - n1));
-            return 0;
-        }
-        int64_t col = base + lane;
+__device__ __forceinline__ void stage_elements(T* __restrict__ rowp, const S* __restrict__ row, int64_t base,
+                                               int64_t p0, int wt, int lane) {
+    int64_t col = base + lane;
+    while (col >= p0) col -= p0;
+    for (int x = lane; x < wt; x += 32) {
+        if constexpr (sizeof(T) == sizeof(S)) cp_async4(rowp + x, row + col);
+        else rowp[x] = (T)row[col];
+        col += 32;
         while (col >= p0) col -= p0;
-        for (int x = lane; x < wt; x += 32) {
-            cp_async4(rowp + x, src + col);
-            col += 32;
-            while (col >= p0) col -= p0;
-        }
-        return 0;
-    } else {
-        if (base + wt <= p0) {
-            // int8 series widened to int32: whole aligned 4-byte words of the
-            // segment, one load per lane per word, each byte sign-extended into
-            // one 128-bit shared store; logical column 0 sits at the segment's
-            // misalignment, as for the copied rows (little-endian bytes)
-            const S* g = src + base;
-            const int a = (int)((uintptr_t)g & 3);
-            const uint32_t* w0 = reinterpret_cast<const uint32_t*>(g - a);
-            const int nw = (wt + a + 3) >> 2;
-            for (int k = lane; k < nw; k += 32) {
-                const uint32_t v = __ldg(w0 + k);
-                *reinterpret_cast<int4*>(rowp + 4 * k) =
-                    make_int4((int)(v << 24) >> 24, (int)(v << 16) >> 24, (int)(v << 8) >> 24, (int)v >> 24);
-            }
-            return a;
-        }
-        int64_t col = base + lane;
-        while (col >= p0) col -= p0;
-        for (int x = lane; x < wt; x += 32) {
-            rowp[x] = (T)src[col];
-            col += 32;
-            while (col >= p0) col -= p0;
-        }
-        return 0;
     }
 }
 
 // ---------------------------------------------------------------------------
 // The FFA of R = 2^QQ rows on W = 4 + R - 1 consecutive columns held in
 // registers (compile-time shifts): out[v][0..3] is trial v at the first four
-// columns.  load() reads a row's W values starting at element offset `off`
-// (0..3) of a 16-byte aligned pointer: 128-bit loads, then two branch-free
-// selects per value (a warp-uniform branch on the offset measured slower).
+// columns.  load() reads a row's W values starting at the compile-time
+// element offset OFF of a 16-byte aligned pointer, in 128-bit loads.
 // ---------------------------------------------------------------------------
 template <class T, int QQ>
 struct RegFFA {
     static constexpr int R = 1 << QQ;
     static constexpr int W = 4 + R - 1;
-    static constexpr int NV = (W + 6) / 4;  // 128-bit loads covering W values at any offset
-    static __device__ __forceinline__ void load(const T* p, int off, T (&a)[W]) {
+    template <int OFF>
+    static __device__ __forceinline__ void load(const T* p, T (&a)[W]) {
+        constexpr int NV = (OFF + W + 3) / 4;
         T r[4 * NV];
 #pragma unroll
         for (int k = 0; k < NV; ++k)
             *reinterpret_cast<int4*>(&r[4 * k]) = *reinterpret_cast<const int4*>(p + 4 * k);
-        const bool b0 = (off & 1) != 0, b1 = (off & 2) != 0;
-        T t[W + 2];
 #pragma unroll
-        for (int k = 0; k < W + 2; ++k) t[k] = b0 ? r[k + 1] : r[k];
-#pragma unroll
-        for (int k = 0; k < W; ++k) a[k] = b1 ? t[k + 2] : t[k];
+        for (int k = 0; k < W; ++k) a[k] = r[k + OFF];
+    }
+    // rows u = 0 .. R-1, row u at p + u * pitch + (k * u & ~3), its values at
+    // offset (TT * u) & 3 (TT = k & 3)
+    template <int TT, size_t... U>
+    static __device__ __forceinline__ void load_rows(const T* p, int pitch, int k, T (&a)[R][W],
+                                                     std::index_sequence<U...>) {
+        (load<(TT * (int)U) & 3>(p + (int)U * pitch + ((k * (int)U) & ~3), a[U]), ...);
     }
     static __device__ __forceinline__ void run(T (&a)[R][W], T (&out)[R][4]) {
 #pragma unroll
@@ -212,7 +164,7 @@ __device__ __forceinline__ int as_bits(T v) {
 // Four consecutive outputs to global memory: one 128-bit store when the row
 // is 16-byte aligned (vec), else element stores up to `left` columns.
 template <class T>
-__device__ __forceinline__ void store4(T* d, const T (&v)[4], int64_t left, bool vec) {
+__device__ __forceinline__ void store4(T* d, const T (&v)[4], int left, bool vec) {
     if (vec) {
         *reinterpret_cast<int4*>(d) = make_int4(as_bits(v[0]), as_bits(v[1]), as_bits(v[2]), as_bits(v[3]));
     } else {
@@ -223,8 +175,8 @@ __device__ __forceinline__ void store4(T* d, const T (&v)[4], int64_t left, bool
 }
 
 // ---------------------------------------------------------------------------
-// One pass of q = Q1 + Q2 <= 6 stages.  A CTA owns (block, kappa, column
-// tile of B columns): it stages 2^q input rows of B + 2^q - 1 columns, row u
+// One pass of q = Q1 + Q2 <= 6 stages.  A CTA takes a (block, kappa, column
+// tile of B columns) -- or, persistent, one after another: it stages 2^q input rows of B + 2^q - 1 columns, row u
 // starting at column c + kappa*u (cyclically), in shared memory.  Sub-pass 1:
 // each thread takes 4 consecutive columns of a group of 2^Q1 rows, applies
 // Q1 stages in registers and stores the group's 2^Q1 partial trials,
@@ -232,10 +184,27 @@ __device__ __forceinline__ void store4(T* d, const T (&v)[4], int64_t left, bool
 // input row u2 of the last Q2 stages is read at column offset k1*u2 (the
 // shift that the unrolled recursion assigns it), Q2 stages in registers, and
 // the tile's output rows go to global memory (128-bit stores on a padded
-// pitch).  Tiles are B = 256 columns up to 5 stages and 128 for 6 (64 rows),
-// so two CTAs fit an SM.
+// pitch).  The staging buffer is free once sub-pass 1 is done, so a persistent
+// CTA issues the next tile's copies before sub-pass 2, to arrive under it.  Tiles are
+// B = 256 columns up to 5 stages and 128 for 6 (64 rows), so two CTAs fit an
+// SM.
+//
+// Alignment.  The staging copies are 16 bytes wide, so a row's columns keep
+// the misalignment 0..3 of their address.  It is (t * u) & 3 in row u for one
+// t per CTA -- the rows of the first pass are p0 elements apart (t = p0 & 3),
+// row u of a later pass starts kappa * u columns on (t = kappa & 3) -- and so
+// is the offset k1*u2 of sub-pass 2 (t = k1 & 3, one per warp): both
+// sub-passes are compiled for each t, with every row's offset known, and need
+// no select on it.  Rows off that pattern (they wrapped past p0, or the plane
+// is not 16-byte aligned) are staged element by element onto it.
 // ---------------------------------------------------------------------------
-constexpr int FK_THREADS = 256;
+// Threads of a CTA: 64-row tiles of 256 columns leave room for one CTA an SM.
+__host__ __device__ constexpr int fk_threads(int q, int b) { return q == 6 && b == 256 ? 512 : 256; }
+// Persistent CTAs, the next tile staged under sub-pass 2, where shared memory
+// holds the SM to two CTAs or one (64 rows of four-byte elements); elsewhere
+// more CTAs in flight hide the staging better than the registers that a
+// pipelined tile takes.
+__host__ __device__ constexpr bool fk_persistent(int q, bool widen) { return q == 6 && !widen; }
 __host__ __device__ constexpr int fk_r4(int x) { return (x + 3) & ~3; }
 __host__ __device__ constexpr int fk_max(int a, int b) { return a > b ? a : b; }
 __host__ __device__ constexpr int fk_wt(int q, int b) { return b + (1 << q) - 1; }                  // staged columns
@@ -251,159 +220,212 @@ __host__ __device__ constexpr int fk_wb(int q, int q1, int b) {
 }
 
 template <class T, bool FIRST, int Q1, int Q2, int B>
-__global__ void __launch_bounds__(FK_THREADS, 2) k_fold(const void* __restrict__ src_v, T* __restrict__ dst_all,
+__global__ void __launch_bounds__(fk_threads(Q1 + Q2, B), fk_threads(Q1 + Q2, B) == 512 ? 1 : 2) k_fold(const void* __restrict__ src_v, T* __restrict__ dst_all,
                                                        const FoldGroup fg, int s) {
     constexpr int q = Q1 + Q2;
+    constexpr int FK_THREADS = fk_threads(q, B);
     constexpr int rows = 1 << q;
     constexpr int R1 = 1 << Q1, R2 = 1 << Q2;
     constexpr int WT = fk_wt(q, B), W1 = fk_w1(q, Q1, B);
     constexpr int WA = fk_wa(q, Q1, B), WB = fk_wb(q, Q1, B);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int off_a[rows];
     T* bufA = reinterpret_cast<T*>(smem_raw);
     T* bufB = bufA + rows * WA;
 
-    const int ei = group_entry(fg, blockIdx.x);
-    const int64_t p0 = fg.p0[ei], m_data = fg.m_data[ei], ld = fg.ld[ei];
-    const int64_t n_ct = (p0 + B - 1) / B;
-    T* __restrict__ dst = dst_all + fg.off[ei];
-    const int64_t unit = blockIdx.x - fg.unit0[ei];
-    const int64_t ct = unit % n_ct;
-    const int64_t rest = unit / n_ct;
-    const int64_t kappa = rest & ((1ll << s) - 1);
-    const int64_t blk = rest >> s;
-    const int64_t c = ct * B;
+    using S = typename std::conditional<FIRST, typename FoldIn<T>::type, T>::type;
+    constexpr bool WIDEN = sizeof(S) == 1;  // int8 series
+    constexpr bool PERSIST = fk_persistent(q, WIDEN);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int NW = FK_THREADS / 32;
+    constexpr int RPW = (rows + NW - 1) / NW;            // rows staged by a warp
+    constexpr int KPL = ((WT + 6) / 4 + 31) / 32;        // aligned words per lane and row (WIDEN)
+    const uint32_t units = (uint32_t)fg.unit0[fg.n];     // fits int32
 
-    const int64_t kmod = kappa % p0;
-    auto row_base = [&](int u) -> int64_t {
-        int64_t base = c + (kmod * (u % p0)) % p0;
-        return base >= p0 ? base - p0 : base;
+    struct Tile {
+        int64_t p0, ld, blk, c;
+        uint32_t kappa;
+        int ei, t;
     };
-    if constexpr (FIRST && sizeof(typename FoldIn<T>::type) == 1) {
-        // int8 series: the plain loads of all of this warp's rows are issued
-        // before any is widened and stored, so that their DRAM latencies
-        // overlap (cp.async cannot widen).  Rows that wrap or lie beyond the
-        // data take stage_row's general path.
-        using S = typename FoldIn<T>::type;
-        constexpr int RPW = (rows + NW - 1) / NW;     // rows per warp
-        constexpr int KPL = ((WT + 6) / 4 + 31) / 32;  // aligned words per lane and row
-        const S* srcb = (const S*)fg.src[ei];
-        uint32_t wv[RPW][KPL];
-        int aw[RPW];
-#pragma unroll
-        for (int j = 0; j < RPW; ++j) {
-            const int u = warp + j * NW;
-            aw[j] = -1;
-            if (u < rows) {
-                const int64_t g = blk * rows + u;
-                const int64_t base = row_base(u);
-                if (g < m_data && base + WT <= p0) {
-                    const S* gp = srcb + g * p0 + base;
-                    const int a = (int)((uintptr_t)gp & 3);
-                    const uint32_t* w0 = reinterpret_cast<const uint32_t*>(gp - a);
-                    const int nw = (WT + a + 3) >> 2;  // the word holding the last element ends the copy
-#pragma unroll
-                    for (int t = 0; t < KPL; ++t) {
-                        const int k = lane + 32 * t;
-                        wv[j][t] = k < nw ? __ldg(w0 + k) : 0u;
-                    }
-                    aw[j] = a;
-                }
+    auto locate = [&](uint32_t u) {
+        Tile w;
+        w.ei = group_entry(fg, u);
+        w.p0 = fg.p0[w.ei];
+        w.ld = fg.ld[w.ei];
+        const uint32_t unit = u - (uint32_t)fg.unit0[w.ei];
+        const uint32_t n_ct = (uint32_t)((w.p0 + B - 1) / B);
+        const uint32_t rest = unit / n_ct;
+        w.kappa = rest & ((1u << s) - 1);
+        w.blk = rest >> s;
+        w.c = (int64_t)(unit - rest * n_ct) * B;
+        w.t = (int)((FIRST ? w.p0 : (int64_t)w.kappa) & 3);
+        return w;
+    };
+    uint32_t wv[WIDEN ? RPW : 1][KPL];  // WIDEN: the tile's words between issue and store
+    int64_t my_row = 0, my_base = 0;
+    int my_how = 0;
+    auto row_how = [&](int j) { return __shfl_sync(0xffffffffu, my_how, j); };
+    auto row_base = [&](int j) { return __shfl_sync(0xffffffffu, my_base, j); };
+    // Start staging a tile.  cp.async copies straight into bufA; the words of
+    // an int8 series (cp.async cannot widen) are loaded into registers, every
+    // row's before any is needed.
+    auto stage_issue = [&](const Tile& w) {
+        // lane j: where row warp + j * NW starts, and how it is staged (0:
+        // beyond the data, zeros; 1: 16-byte copies; 2: element by element)
+        const S* __restrict__ src = FIRST ? (const S*)fg.src[w.ei] : (const S*)src_v + fg.off[w.ei];
+        my_how = 0;
+        {
+            const int u = warp + lane * NW;
+            if (lane < RPW && u < rows) {
+                const int64_t g = w.blk * rows + u;
+                if (w.p0 < (1 << 25))
+                    my_base = (uint32_t)((uint32_t)w.c + (w.kappa % (uint32_t)w.p0) * (uint32_t)u) % (uint32_t)w.p0;
+                else
+                    my_base = (w.c + (int64_t)w.kappa * u) % w.p0;
+                my_row = FIRST ? g * w.p0 : ((g << s) + w.kappa) * w.ld;
+                const uintptr_t a = reinterpret_cast<uintptr_t>(src + my_row + my_base) / sizeof(S);
+                if (!FIRST || g < fg.m_data[w.ei]) my_how = my_base + WT <= w.p0 && (a & 3) == ((w.t * u) & 3) ? 1 : 2;
             }
         }
 #pragma unroll
         for (int j = 0; j < RPW; ++j) {
-            const int u = warp + j * NW;
-            if (u >= rows) continue;
+            const int u = warp + j * NW, off = (w.t * u) & 3;
+            if (u >= rows) break;
             T* rowp = bufA + u * WA;
-            int a = aw[j];
-            if (a >= 0) {
-                const int nw = (WT + a + 3) >> 2;
+            const int how = row_how(j);
+            const S* rp = src + __shfl_sync(0xffffffffu, my_row, j);
+            const int64_t base = row_base(j);
+            if (how == 1) {
+                // from the aligned-down start; the chunk (word) holding the
+                // segment's last element ends within that element's 16-byte
+                // (4-byte) block
+                const S* g0 = rp + base - off;
+                const int nc = (WT + off + 3) >> 2;
+                if constexpr (WIDEN) {
 #pragma unroll
-                for (int t = 0; t < KPL; ++t) {
-                    const int k = lane + 32 * t;
-                    const uint32_t v = wv[j][t];
-                    if (k < nw)
-                        *reinterpret_cast<int4*>(rowp + 4 * k) = make_int4(
+                    for (int i = 0; i < KPL; ++i) {
+                        const int k = lane + 32 * i;
+                        wv[j][i] = k < nc ? __ldg(reinterpret_cast<const uint32_t*>(g0) + k) : 0u;
+                    }
+                } else {
+                    for (int k = lane; k < nc; k += 32) cp_async16(rowp + 4 * k, g0 + 4 * k);
+                }
+            } else if (how == 2) {
+                stage_elements(rowp + off, rp, base, w.p0, WT, lane);
+            } else {
+                for (int x = 4 * lane; x < WT + 3; x += 128) *reinterpret_cast<int4*>(rowp + x) = make_int4(0, 0, 0, 0);
+            }
+        }
+    };
+    // Finish it: bufA holds the tile after the next barrier.
+    auto stage_finish = [&](int t) {
+        if constexpr (WIDEN) {
+#pragma unroll
+            for (int j = 0; j < RPW; ++j) {
+                const int u = warp + j * NW, off = (t * u) & 3;
+                if (u >= rows) break;
+                if (row_how(j) != 1) continue;
+                const int nc = (WT + off + 3) >> 2;
+#pragma unroll
+                for (int i = 0; i < KPL; ++i) {
+                    const int k = lane + 32 * i;
+                    const uint32_t v = wv[j][i];
+                    if (k < nc)
+                        *reinterpret_cast<int4*>(bufA + u * WA + 4 * k) = make_int4(
                             (int)(v << 24) >> 24, (int)(v << 16) >> 24, (int)(v << 8) >> 24, (int)v >> 24);
                 }
-            } else {
-                const int64_t g = blk * rows + u;
-                a = stage_row(rowp, srcb + g * p0, row_base(u), p0, WT, g < m_data, lane);
             }
-            if (lane == 0) off_a[u] = a;
+        } else {
+            cp_async_wait();
         }
-    } else {
-        for (int u = warp; u < rows; u += NW) {
-            const int64_t g = blk * rows + u;
-            const int64_t base = row_base(u);
-            int a;
-            if (FIRST)
-                a = stage_row(bufA + u * WA, (const typename FoldIn<T>::type*)fg.src[ei] + g * p0, base, p0, WT,
-                              g < m_data, lane);
-            else
-                a = stage_row(bufA + u * WA, (const T*)src_v + fg.off[ei] + ((g << s) + kappa) * ld, base, p0, WT,
-                              true, lane);
-            if (lane == 0) off_a[u] = a;
-        }
-    }
-    cp_async_wait();
-    __syncthreads();
-    const int64_t grow0 = (blk << (s + q)) + (kappa << q);
-    const int64_t ncols = (c + B <= p0) ? B : p0 - c;
-    const bool vec = (ld & 3) == 0 && ((uintptr_t)dst & 15) == 0;
+    };
 
-    // sub-pass 1: groups of R1 consecutive rows
-    {
-        constexpr int W = RegFFA<T, Q1>::W;
-        constexpr int nstrips = (W1 + 3) / 4;
-        constexpr int items = (rows / R1) * nstrips;
-        for (int it = threadIdx.x; it < items; it += FK_THREADS) {
-            const int strip = it % nstrips, g = it / nstrips;
-            const int x0 = 4 * strip;
-            T a[R1][W];
-#pragma unroll
-            for (int u = 0; u < R1; ++u) RegFFA<T, Q1>::load(bufA + (g * R1 + u) * WA + x0, off_a[g * R1 + u], a[u]);
-            T out[R1][4];
-            RegFFA<T, Q1>::run(a, out);
-            if (Q2 == 0) {
-                if (x0 < ncols) {
-#pragma unroll
-                    for (int v = 0; v < R1; ++v) store4(dst + (grow0 + v) * ld + c + x0, out[v], ncols - x0, vec);
-                }
-            } else {
-                // group g is input row u2 = g of sub-pass 2
-#pragma unroll
-                for (int v = 0; v < R1; ++v)
-                    *reinterpret_cast<int4*>(bufB + (v * R2 + g) * WB + x0) =
-                        make_int4(as_bits(out[v][0]), as_bits(out[v][1]), as_bits(out[v][2]), as_bits(out[v][3]));
-            }
-        }
-    }
-    if (Q2 > 0) {
+    uint32_t unit = blockIdx.x;
+    Tile w = locate(unit);
+    stage_issue(w);
+    stage_finish(w.t);
+    for (;;) {
         __syncthreads();
-        constexpr int W = RegFFA<T, Q2>::W;
-        constexpr int nstrips = B / 4;
-        constexpr int items = R1 * nstrips;
-        for (int it = threadIdx.x; it < items; it += FK_THREADS) {
-            const int strip = it % nstrips, k1 = it / nstrips;
-            const int x0 = 4 * strip;
-            T a[R2][W];
+        T* __restrict__ dst = dst_all + fg.off[w.ei];
+        const int64_t ld = w.ld;
+        const int ncols = (w.c + B <= w.p0) ? B : (int)(w.p0 - w.c);
+        const bool vec = (ld & 3) == 0 && ((uintptr_t)dst & 15) == 0;
+        T* __restrict__ drow = dst + ((w.blk << (s + q)) + ((int64_t)w.kappa << q)) * ld + w.c;
+
+        // sub-pass 1: groups of R1 consecutive rows
+        auto sub1 = [&](auto tt) {
+            using F = RegFFA<T, Q1>;
+            constexpr int nstrips = (W1 + 3) / 4;
+            constexpr int items = (rows / R1) * nstrips;
+            for (int it = threadIdx.x; it < items; it += FK_THREADS) {
+                const int strip = it % nstrips, g = it / nstrips;
+                const int x0 = 4 * strip;
+                T a[R1][F::W];
+                // rows g * R1 + u: (t * (g * R1 + u)) & 3 = (t * u) & 3 when R1 is a multiple of 4
+                F::template load_rows<decltype(tt)::value>(bufA + g * R1 * WA + x0, WA, 0, a,
+                                                           std::make_index_sequence<R1>{});
+                T out[R1][4];
+                F::run(a, out);
+                if (Q2 == 0) {
+                    if (x0 < ncols) {
 #pragma unroll
-            for (int u = 0; u < R2; ++u) {
-                const int sh = k1 * u;
-                RegFFA<T, Q2>::load(bufB + (k1 * R2 + u) * WB + x0 + (sh & ~3), sh & 3, a[u]);
+                        for (int v = 0; v < R1; ++v) store4(drow + v * ld + x0, out[v], ncols - x0, vec);
+                    }
+                } else {
+                    // group g is input row u2 = g of sub-pass 2
+#pragma unroll
+                    for (int v = 0; v < R1; ++v)
+                        *reinterpret_cast<int4*>(bufB + (v * R2 + g) * WB + x0) =
+                            make_int4(as_bits(out[v][0]), as_bits(out[v][1]), as_bits(out[v][2]), as_bits(out[v][3]));
+                }
             }
-            T out[R2][4];
-            RegFFA<T, Q2>::run(a, out);
-            if (x0 < ncols) {
+        };
+        static_assert(Q2 == 0 || R1 % 4 == 0, "a group's rows start on the pattern");
+        switch (w.t) {
+            case 0: sub1(std::integral_constant<int, 0>{}); break;
+            case 1: sub1(std::integral_constant<int, 1>{}); break;
+            case 2: sub1(std::integral_constant<int, 2>{}); break;
+            default: sub1(std::integral_constant<int, 3>{}); break;
+        }
+        __syncthreads();
+        // bufA is free: the next tile's copies run under sub-pass 2
+        bool more = false;
+        if constexpr (PERSIST) {
+            unit += gridDim.x;
+            more = unit < units;
+        }
+        if (more) {
+            w = locate(unit);
+            stage_issue(w);
+        }
+        if constexpr (Q2 > 0) {
+            constexpr int nstrips = B / 4;
+            constexpr int items = R1 * nstrips;
+            static_assert(nstrips % 32 == 0, "one trial of sub-pass 1 per warp");
+            for (int it = threadIdx.x; it < items; it += FK_THREADS) {
+                const int strip = it % nstrips, k1 = it / nstrips;
+                const int x0 = 4 * strip;
+                if (x0 >= ncols) continue;
+                auto sub2 = [&](auto tt) {
+                    using F = RegFFA<T, Q2>;
+                    T a[R2][F::W];
+                    F::template load_rows<decltype(tt)::value>(bufB + k1 * R2 * WB + x0, WB, k1, a,
+                                                               std::make_index_sequence<R2>{});
+                    T out[R2][4];
+                    F::run(a, out);
+                    T* d = drow + (int64_t)(k1 * R2) * ld + x0;
 #pragma unroll
-                for (int v = 0; v < R2; ++v)
-                    store4(dst + (grow0 + k1 * R2 + v) * ld + c + x0, out[v], ncols - x0, vec);
+                    for (int v = 0; v < R2; ++v) store4(d + v * ld, out[v], ncols - x0, vec);
+                };
+                switch (k1 & 3) {
+                    case 0: sub2(std::integral_constant<int, 0>{}); break;
+                    case 1: sub2(std::integral_constant<int, 1>{}); break;
+                    case 2: sub2(std::integral_constant<int, 2>{}); break;
+                    default: sub2(std::integral_constant<int, 3>{}); break;
+                }
             }
         }
+        if (!more) break;
+        stage_finish(w.t);
     }
 }
 
@@ -438,7 +460,15 @@ static ffa_status launch_k(const void* src, T* dst, FoldGroup& fg, int64_t m_row
     const int64_t units = group_units(fg, m_rows, rows, B);
     if (units <= 0) return FFA_OK;
     if (units > INT32_MAX) return fail(FFA_ERR_UNSUPPORTED, "fold: plane too large for one launch");
-    k_fold<T, FIRST, Q1, Q2, B><<<(unsigned)units, FK_THREADS, smem, st>>>(src, dst, fg, s);
+    constexpr int threads = fk_threads(q, B);
+    int64_t grid = units;
+    if (fk_persistent(q, FIRST && sizeof(typename FoldIn<T>::type) == 1)) {
+        int64_t resident = 0;
+        es = resident_ctas((const void*)k_fold<T, FIRST, Q1, Q2, B>, threads, smem, &resident);
+        if (es != FFA_OK) return es;
+        grid = units < resident ? units : resident;
+    }
+    k_fold<T, FIRST, Q1, Q2, B><<<(unsigned)grid, threads, smem, st>>>(src, dst, fg, s);
     FFA_LAUNCH_CHECK("k_fold");
     count_launch();
     return FFA_OK;

@@ -36,10 +36,6 @@ __device__ __forceinline__ int score_entry(const ScoreGroup& g, int64_t it) {
     return lo;
 }
 
-// Resident CTAs of a kernel for a dynamic shared-memory size, times the SM
-// count, per device: queried once (launches come per base period).
-ffa_status resident_ctas(const void* fn, int threads, size_t smem, int64_t* out);
-
 // One base period (or `count` ready profiles of p0 bins), and a group of n
 // base periods sharing m_rows (*p0max: the longest profile).
 ScoreGroup score_single(int64_t p0, int64_t ld, int64_t count, ffa_record* d_rec);
