@@ -4,18 +4,28 @@
 //   * FP64 normalisation to FP32 z, or to the int8 code q = clip(rint(16 z)).
 //
 // Running median design (exact, tiled).  A CTA owns T consecutive outputs
-// a..l.  Their windows all contain the core C = [s_l, e_a]; window i is C
-// plus |F_i| <= T-1 fringe samples.  The rank-r element of window i lies
-// between C's order statistics (r - |F_i|) and r, so with
-//   rho_lo = min_i (r1_i - |F_i|),  rho_hi = max_i r2_i
-// every median of the tile lies in [C_(rho_lo), C_(rho_hi)].  Two histogram
-// passes over C (on the top 12 and next 12 bits of an order-preserving
-// 64-bit key) find the 24-bit key prefixes P_lo, P_hi of those two order
-// statistics.  The samples of the tile's union whose prefix lies in
-// [P_lo, P_hi] are the only possible medians (about T of them); they are
-// sorted in shared memory and each thread walks the sorted list counting the
-// ones inside its own window, starting from the exact number of window
-// samples below P_lo.  T <= (W+1)/4 keeps rho_lo >= 0 and rho_hi < |C|.
+// a..l at a time.  Their windows all contain the core C = [s_l, e_a]; window
+// i is C plus |F_i| <= T-1 fringe samples left and right of it.  One pass over
+// the tile's union counts the core samples below a value bracket and gathers
+// the samples inside it (keyed by an order-preserving 64-bit integer,
+// classified on its top 32 bits); they are sorted, and output i's order
+// statistic is found by walking the few gathered fringe samples, the only
+// ones whose membership depends on i.  The counts are exact, so a bracket is
+// only a guess that is checked: a median outside it fails the tile's attempt
+// and the next bracket is tried,
+//   1. around the previous tile's medians (a CTA takes consecutive tiles;
+//      a window of W samples changes by T of them from tile to tile),
+//   2. wider, or exactly those medians' range if that bracket held too many
+//      samples (series of few distinct values),
+//   3. quantiles of a sample of the core,
+//   4. the proven bracket: the rank-r element of window i lies between C's
+//      order statistics r - |F_i| and r, so with rho_lo = min_i (r1_i - |F_i|)
+//      and rho_hi = max_i r2_i every median of the tile lies in [C_(rho_lo),
+//      C_(rho_hi)], whose 24-bit key prefixes two histogram passes over C
+//      find (T <= (W+1)/4 keeps rho_lo >= 0 and rho_hi < |C|).
+// Bound by L2: the union is read once per tile, 8 (W + T) bytes for T outputs.
+// 2^24 samples, W = 62501: 2.0 ms; 13.9 ms with the proven bracket alone (three
+// passes, a bitonic sort of about T samples and a walk over all of them).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -214,24 +224,125 @@ __global__ void k_runmed_small(const double* __restrict__ x, int64_t n, int64_t 
 // ---------------------------------------------------------------------------
 // tiled exact running median
 // ---------------------------------------------------------------------------
-constexpr int RM_CAP = 4096;    // candidate capacity (power of two)
+constexpr int RM_CAP = 4096;    // gathered samples (power of two)
 constexpr int RM_MAXT = 1024;   // largest tile
+constexpr int RM_NT = 512;      // threads of the largest tile's CTA
+constexpr int RM_NBK = 1024;    // buckets of the sort over a bracket
 
 struct RmShared {
-    uint32_t hist1[4096];
-    uint32_t hist2a[4096];
-    uint32_t hist2b[4096];
-    uint64_t ckey[RM_CAP];
-    uint32_t coff[RM_CAP];
-    uint32_t lflag[RM_MAXT + 1];
-    uint32_t rflag[RM_MAXT + 1];
+    union {
+        struct {
+            uint32_t hist1[4096], hist2a[4096], hist2b[4096];
+        };
+        struct {
+            uint64_t ckey[RM_CAP];
+            uint32_t coff[RM_CAP];
+        };
+    };
+    uint16_t ord[RM_CAP];  // the gathered samples in key order
+    union {
+        // gathered fringe samples in key order: sorted place | index << 12 | right << 23
+        uint32_t fringe[2 * RM_MAXT];
+        uint16_t place[RM_CAP];  // while sorting: a sample's bucket, then its rank
+    };
+    uint32_t bkt[RM_NBK];
+    uint32_t fbits[RM_CAP / 32];  // sorted places that hold fringe samples
+    // fringe samples below the bracket: bits, and the counts before each word
+    uint32_t lbits[RM_MAXT / 32], rbits[RM_MAXT / 32], lpre[RM_MAXT / 32 + 1], rpre[RM_MAXT / 32 + 1];
+    // the same for the gathered fringe samples that precede every output's median
+    uint32_t l2bits[RM_MAXT / 32], r2bits[RM_MAXT / 32], l2pre[RM_MAXT / 32 + 1], r2pre[RM_MAXT / 32 + 1];
     uint32_t tmp[64];
     int64_t tmp64[64];
-    unsigned long long kmin, kmax;
-    uint32_t ccount;
+    unsigned long long kmin, kmax, blo, bhi;
+    float flo, finv;
+    uint32_t ccount, cbelow, nf, tmin, mmin, mmax, pmin, pmax;
+    int big;
     int bin_a, bin_b;
     uint32_t below_a, below_b;
 };
+
+// Sort the first cc of ckey (and coff) by key: bitonic over the next power of two.
+__device__ void rm_bitonic(RmShared& sh, uint32_t cc) {
+    const int T = blockDim.x, tid = threadIdx.x;
+    uint32_t np2 = 1;
+    while (np2 < cc) np2 <<= 1;
+    for (uint32_t t = cc + tid; t < np2; t += T) {
+        sh.ckey[t] = ~0ull;
+        sh.coff[t] = 0xffffffffu;
+    }
+    __syncthreads();
+    for (uint32_t kk = 2; kk <= np2; kk <<= 1) {
+        for (uint32_t jj = kk >> 1; jj > 0; jj >>= 1) {
+            for (uint32_t p = tid; p < np2 / 2; p += T) {
+                const uint32_t t = ((p & ~(jj - 1)) << 1) | (p & (jj - 1)), u = t | jj;
+                const uint64_t kt = sh.ckey[t], ku = sh.ckey[u];
+                if ((kt > ku) == ((t & kk) == 0)) {
+                    sh.ckey[t] = ku;
+                    sh.ckey[u] = kt;
+                    const uint32_t o = sh.coff[t];
+                    sh.coff[t] = sh.coff[u];
+                    sh.coff[u] = o;
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// ord = the gathered samples 0 .. cc-1 in key order: by buckets linear in the
+// value across the bracket (flo, finv; a monotone map, so buckets are in
+// order), then by counting inside a bucket -- one or two samples each, where
+// a bitonic sort takes 55 barriers for a thousand samples.  Many equal values
+// in one bucket take the bitonic sort.
+__device__ void rm_sort(RmShared& sh, uint32_t cc) {
+    const int T = blockDim.x, tid = threadIdx.x;
+    for (int b = tid; b < RM_NBK; b += T) sh.bkt[b] = 0;
+    if (tid == 0) sh.big = 0;
+    __syncthreads();
+    const float flo = sh.flo, finv = sh.finv;
+    for (uint32_t i = tid; i < cc; i += T) {
+        const float f = __fmul_rn(__fsub_rn(__double2float_rn(dkey_inv(sh.ckey[i])), flo), finv);
+        const int b = min(max((int)f, 0), RM_NBK - 1);
+        sh.place[i] = (uint16_t)b;
+        if (atomicAdd(&sh.bkt[b], 1u) >= 64) sh.big = 1;
+    }
+    __syncthreads();
+    if (sh.big) {
+        rm_bitonic(sh, cc);
+        for (uint32_t i = tid; i < cc; i += T) sh.ord[i] = (uint16_t)i;
+        __syncthreads();
+        return;
+    }
+    {
+        const int per = RM_NBK / T, b0 = tid * per;
+        uint32_t s = 0;
+        for (int t = 0; t < per; ++t) s += sh.bkt[b0 + t];
+        uint32_t c = block_exscan(s, sh.tmp, nullptr);
+        for (int t = 0; t < per; ++t) {
+            const uint32_t hc = sh.bkt[b0 + t];
+            sh.bkt[b0 + t] = c;
+            c += hc;
+        }
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < cc; i += T) sh.ord[atomicAdd(&sh.bkt[sh.place[i]], 1u)] = (uint16_t)i;
+    __syncthreads();  // bkt[b] is now the end of bucket b
+    for (uint32_t i = tid; i < cc; i += T) {
+        const int b = sh.place[i];
+        const uint32_t e0 = b ? sh.bkt[b - 1] : 0u, e1 = sh.bkt[b];
+        const uint64_t k = sh.ckey[i];
+        uint32_t r = e0;
+        for (uint32_t e = e0; e < e1; ++e) {
+            const uint32_t o = sh.ord[e];
+            const uint64_t ko = sh.ckey[o];
+            r += ko < k || (ko == k && o < i);
+        }
+        sh.place[i] = (uint16_t)r;
+    }
+    __syncthreads();
+    for (uint32_t i = tid; i < cc; i += T) sh.ord[sh.place[i]] = (uint16_t)i;
+    __syncthreads();
+}
 
 // Exact rank-`rank` key of x[s..e] by an 8-pass, 8-bit radix select over the
 // whole CTA (slow path for tiles whose candidate set overflows).
@@ -267,189 +378,401 @@ __device__ uint64_t cta_select_key(const double* __restrict__ x, int64_t s, int6
     return prefix;
 }
 
-__global__ void __launch_bounds__(1024) k_runmed_tile(const double* __restrict__ x, int64_t n,
-                                                      int64_t w, double* __restrict__ resid,
-                                                      int32_t* d_status) {
+__device__ __forceinline__ uint32_t hi_key(uint64_t bits) {  // top 32 bits of dkey
+    const uint32_t u = (uint32_t)(bits >> 32);
+    return u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);
+}
+
+// One warp: the counts of set bits before each of 32 words (pre[32]: all).
+__device__ __forceinline__ void rm_word_prefix(const uint32_t* bits, uint32_t* pre) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t v = __popc(bits[lane]);
+    uint32_t c = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, c, o);
+        if (lane >= o) c += u;
+    }
+    pre[lane] = c - v;
+    if (lane == 31) pre[32] = c;
+}
+// set bits below position q (<= RM_MAXT)
+__device__ __forceinline__ uint32_t rm_bits_before(const uint32_t* bits, const uint32_t* pre, uint32_t q) {
+    return pre[q >> 5] + ((q & 31) ? __popc(bits[q >> 5] & ((1u << (q & 31)) - 1)) : 0u);
+}
+
+// T outputs per tile, blockDim threads.  The CTAs take runs of `run`
+// consecutive tiles in turn: long enough for one tile to predict the next,
+// short enough that the CTAs' windows lie together in L2.
+__global__ void __launch_bounds__(RM_NT, 3) k_runmed_tile(const double* __restrict__ x, int64_t n, int64_t w, int T,
+                                                          int64_t tiles, int64_t run, double* __restrict__ resid,
+                                                          int32_t* d_status) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     RmShared& sh = *reinterpret_cast<RmShared*>(smem_raw);
-    const int T = blockDim.x;
-    const int tid = threadIdx.x;
+    const int NT = blockDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t h = w / 2;
-    const int64_t a = (int64_t)blockIdx.x * T;
-    const int64_t l = (a + T < n ? a + T : n) - 1;
-    const int64_t i = a + tid;
-    const bool active = i <= l;
     auto win_s = [&](int64_t q) { return q - h < 0 ? (int64_t)0 : q - h; };
     auto win_e = [&](int64_t q) { return q + h > n - 1 ? n - 1 : q + h; };
-    const int64_t s_a = win_s(a), e_a = win_e(a), s_l = win_s(l), e_l = win_e(l);
-    const int64_t c0 = s_l, c1 = e_a;
-    const int64_t csize = c1 - c0 + 1;
-    const int64_t s_i = win_s(active ? i : l), e_i = win_e(active ? i : l);
-    const int64_t n_i = e_i - s_i + 1;
-    const int64_t f_i = n_i - csize;
-    const int64_t r1 = (n_i - 1) / 2, r2 = n_i / 2;
-
-    int64_t lo_need = block_reduce_min<int64_t>(active ? r1 - f_i : INT64_MAX, sh.tmp64);
-    int64_t hi_need = block_reduce_max<int64_t>(active ? r2 : INT64_MIN, sh.tmp64);
-    bool bracket_ok = csize > 0 && lo_need >= 0 && hi_need < csize;
-
-    bool fast = false;
-    if (bracket_ok) {
-        const uint32_t rho_lo = (uint32_t)lo_need, rho_hi = (uint32_t)hi_need;
-        // pass 1: top 12 key bits over the core
-        for (int b = tid; b < 4096; b += T) {
-            sh.hist1[b] = 0;
-            sh.hist2a[b] = 0;
-            sh.hist2b[b] = 0;
+    bool known = false;         // pmin, pmax: the previous tile's medians (top key words)
+    float wide = 0.0f;          // half-width of the bracket around them (thread 0)
+    int64_t in_run = 0;
+    for (int64_t tile = blockIdx.x * run; tile < tiles;) {
+        const int64_t a = tile * T;
+        const int64_t l = (a + T < n ? a + T : n) - 1;
+        const int no = (int)(l - a + 1);
+        const int64_t s_a = win_s(a), e_a = win_e(a), s_l = win_s(l), e_l = win_e(l);
+        const int64_t c0 = s_l, c1 = e_a, csize = c1 - c0 + 1;
+        const int lsz = (int)(s_l - s_a), rsz = (int)(e_l - e_a);
+        // proven core ranks; they grow with i or fall, by pieces: all outputs
+        int64_t lo_need = INT64_MAX, hi_need = INT64_MIN;
+        for (int o = tid; o < no; o += NT) {
+            const int64_t n_i = win_e(a + o) - win_s(a + o) + 1;
+            const int64_t lo = (n_i - 1) / 2 - (n_i - csize), hi = n_i / 2;
+            lo_need = lo < lo_need ? lo : lo_need;
+            hi_need = hi > hi_need ? hi : hi_need;
         }
-        __syncthreads();
-        for (int64_t p = c0 + tid; p <= c1; p += T) atomicAdd(&sh.hist1[dkey(x[p]) >> 52], 1u);
-        __syncthreads();
-        block_find_rank(sh.hist1, 4096, rho_lo, sh.tmp, &sh.bin_a, &sh.below_a);
-        block_find_rank(sh.hist1, 4096, rho_hi, sh.tmp, &sh.bin_b, &sh.below_b);
-        const uint32_t b1_lo = sh.bin_a, b1_hi = sh.bin_b;
-        const uint32_t below1_lo = sh.below_a, below1_hi = sh.below_b;
-        __syncthreads();
-        // pass 2: next 12 bits inside the two selected top buckets
-        for (int64_t p = c0 + tid; p <= c1; p += T) {
-            uint64_t k = dkey(x[p]);
-            uint32_t top = (uint32_t)(k >> 52), sub = (uint32_t)(k >> 40) & 0xfff;
-            if (top == b1_lo) atomicAdd(&sh.hist2a[sub], 1u);
-            if (top == b1_hi && b1_hi != b1_lo) atomicAdd(&sh.hist2b[sub], 1u);
-        }
-        __syncthreads();
-        block_find_rank(sh.hist2a, 4096, rho_lo - below1_lo, sh.tmp, &sh.bin_a, &sh.below_a);
-        const uint32_t b2_lo = sh.bin_a, below2_lo = sh.below_a;
-        __syncthreads();
-        block_find_rank(b1_hi == b1_lo ? sh.hist2a : sh.hist2b, 4096, rho_hi - below1_hi, sh.tmp,
-                        &sh.bin_b, &sh.below_b);
-        const uint32_t b2_hi = sh.bin_b;
-        const uint64_t p_lo = ((uint64_t)b1_lo << 12) | b2_lo;
-        const uint64_t p_hi = ((uint64_t)b1_hi << 12) | b2_hi;
-        const uint32_t c_below = below1_lo + below2_lo;  // core samples with prefix < p_lo
-        // gather candidates from the union [s_a, e_l]; flag fringe samples below p_lo
-        if (tid == 0) {
-            sh.ccount = 0;
-            sh.kmin = ~0ull;
-            sh.kmax = 0ull;
-        }
-        for (int t = tid; t <= RM_MAXT; t += T) {
-            sh.lflag[t] = 0;
-            sh.rflag[t] = 0;
-        }
-        __syncthreads();
-        for (int64_t p = s_a + tid; p <= e_l; p += T) {
-            uint64_t k = dkey(x[p]);
-            uint64_t pre = k >> 40;
-            if (pre >= p_lo && pre <= p_hi) {
-                uint32_t slot = atomicAdd(&sh.ccount, 1u);
+        lo_need = block_reduce_min<int64_t>(lo_need, sh.tmp64);
+        hi_need = block_reduce_max<int64_t>(hi_need, sh.tmp64);
+        const bool bracket_ok = csize > 0 && lo_need >= 0 && hi_need < csize;
+        bool done = false, over = false;
+        for (int attempt = known ? 0 : 2; bracket_ok && attempt < 4 && !done; ++attempt) {
+            // ---- the bracket, as keys [blo, bhi] and as floats for the sort
+            auto set_bracket = [&](double lo, double hi) {  // thread 0
+                sh.blo = dkey(lo);
+                sh.bhi = dkey(hi);
+                sh.flo = __double2float_rn(lo);
+                sh.finv = (float)RM_NBK / (__double2float_rn(hi) - sh.flo);
+            };
+            if (attempt < 2) {
+                // 1: the tight one if too many were gathered, else a wider one
+                if (tid == 0) {
+                    const double lo = dkey_inv((uint64_t)sh.pmin << 32), hi = dkey_inv(((uint64_t)sh.pmax << 32) | 0xffffffffull);
+                    const double d = attempt == 0 ? (double)wide : (over ? 0.0 : 4.0 * (double)wide);
+                    set_bracket(lo - d, hi + d);
+                }
+            } else if (attempt == 2) {
+                if (csize < 256) continue;
+                int ns = 128;
+                while (ns * 2 <= RM_CAP && ns * 2 <= csize / 2 && (ns < 1024 || (int64_t)ns * 20 < csize)) ns *= 2;
+                const int64_t stride = csize / ns;
+                float* fv = reinterpret_cast<float*>(sh.coff);
+                float mn = INFINITY, mx = -INFINITY;
+                for (int i = tid; i < ns; i += NT) {
+                    const float v = __double2float_rn(x[c0 + i * stride]);
+                    fv[i] = v;
+                    mn = fminf(mn, v);
+                    mx = fmaxf(mx, v);
+                }
+                for (int b = tid; b < RM_NBK; b += NT) sh.bkt[b] = 0;
+                mn = block_reduce_min<float>(mn, reinterpret_cast<float*>(sh.tmp));
+                mx = block_reduce_max<float>(mx, reinterpret_cast<float*>(sh.tmp));
+                const float inv = (float)RM_NBK / (mx - mn);
+                for (int i = tid; i < ns; i += NT)
+                    atomicAdd(&sh.bkt[min(max((int)((fv[i] - mn) * inv), 0), RM_NBK - 1)], 1u);
+                // a quarter of the proven rank range on each side of its
+                // middle, and 2.5 sigma of the sample quantile
+                const float f = (float)ns / (float)csize, mid = 0.5f * (float)(lo_need + hi_need) * f;
+                const float d = 0.25f * (float)(hi_need - lo_need) * f + 1.25f * sqrtf((float)ns) + 1.0f;
+                const int ilo = max((int)floorf(mid - d), 0), ihi = min((int)ceilf(mid + d), ns - 1);
+                __syncthreads();
+                block_find_rank(sh.bkt, RM_NBK, (uint32_t)ilo, sh.tmp, &sh.bin_a, &sh.below_a);
+                block_find_rank(sh.bkt, RM_NBK, (uint32_t)ihi, sh.tmp, &sh.bin_b, &sh.below_b);
+                if (tid == 0)
+                    set_bracket((double)(mn + (float)sh.bin_a / inv), (double)(mn + (float)(sh.bin_b + 1) / inv));
+            } else {
+                const uint32_t rho_lo = (uint32_t)lo_need, rho_hi = (uint32_t)hi_need;
+                // pass 1: top 12 key bits over the core
+                for (int b = tid; b < 4096; b += NT) {
+                    sh.hist1[b] = 0;
+                    sh.hist2a[b] = 0;
+                    sh.hist2b[b] = 0;
+                }
+                __syncthreads();
+                for (int64_t p = c0 + tid; p <= c1; p += NT) atomicAdd(&sh.hist1[dkey(x[p]) >> 52], 1u);
+                __syncthreads();
+                block_find_rank(sh.hist1, 4096, rho_lo, sh.tmp, &sh.bin_a, &sh.below_a);
+                block_find_rank(sh.hist1, 4096, rho_hi, sh.tmp, &sh.bin_b, &sh.below_b);
+                const uint32_t b1_lo = sh.bin_a, b1_hi = sh.bin_b;
+                const uint32_t below1_lo = sh.below_a, below1_hi = sh.below_b;
+                __syncthreads();
+                // pass 2: next 12 bits inside the two selected top buckets
+                for (int64_t p = c0 + tid; p <= c1; p += NT) {
+                    uint64_t k = dkey(x[p]);
+                    uint32_t top = (uint32_t)(k >> 52), sub = (uint32_t)(k >> 40) & 0xfff;
+                    if (top == b1_lo) atomicAdd(&sh.hist2a[sub], 1u);
+                    if (top == b1_hi && b1_hi != b1_lo) atomicAdd(&sh.hist2b[sub], 1u);
+                }
+                __syncthreads();
+                block_find_rank(sh.hist2a, 4096, rho_lo - below1_lo, sh.tmp, &sh.bin_a, &sh.below_a);
+                const uint32_t b2_lo = sh.bin_a;
+                __syncthreads();
+                block_find_rank(b1_hi == b1_lo ? sh.hist2a : sh.hist2b, 4096, rho_hi - below1_hi, sh.tmp, &sh.bin_b,
+                                &sh.below_b);
+                const uint32_t b2_hi = sh.bin_b;
+                if (tid == 0) {
+                    const uint64_t blo = (((uint64_t)b1_lo << 12) | b2_lo) << 40;
+                    const uint64_t bhi = ((((uint64_t)b1_hi << 12) | b2_hi) << 40) | 0xffffffffffull;
+                    set_bracket(dkey_inv(blo), dkey_inv(bhi));
+                    sh.blo = blo;  // exactly, also where a key is no number's
+                    sh.bhi = bhi;
+                }
+            }
+            __syncthreads();  // blo, bhi; the sample and the histograms are done with
+            const uint32_t klo = (uint32_t)(sh.blo >> 32), khi = (uint32_t)(sh.bhi >> 32), span = khi - klo;
+            if (tid == 0) {
+                sh.ccount = 0;
+                sh.cbelow = 0;
+                sh.kmin = ~0ull;
+                sh.kmax = 0ull;
+            }
+            __syncthreads();
+            if (khi < klo) continue;
+            // ---- gather the union's samples inside the bracket, count the
+            // core's below it, flag the fringe's
+            const unsigned long long* __restrict__ xb = reinterpret_cast<const unsigned long long*>(x);
+            auto keep = [&](uint64_t bits, int64_t p) {
+                const uint64_t k = (bits >> 63) ? ~bits : (bits | 0x8000000000000000ull);
+                const uint32_t slot = atomicAdd(&sh.ccount, 1u);
                 if (slot < RM_CAP) {
                     sh.ckey[slot] = k;
                     sh.coff[slot] = (uint32_t)(p - s_a);
                 }
-                atomicMin(&sh.kmin, (unsigned long long)k);
-                atomicMax(&sh.kmax, (unsigned long long)k);
-            }
-            if (p < s_l) sh.lflag[p - s_a] = pre < p_lo;
-            if (p > e_a) sh.rflag[p - e_a - 1] = pre < p_lo;
-        }
-        __syncthreads();
-        const uint32_t cc = sh.ccount;
-        if (cc > RM_CAP && sh.kmin == sh.kmax) {
-            // every possible median has the same value
-            if (active) resid[i] = x[i] - dkey_inv(sh.kmin);
-            return;
-        }
-        if (cc <= RM_CAP) {
-            fast = true;
-            // fringe counts: left suffix sums, right prefix sums
-            uint32_t lsz = (uint32_t)(s_l - s_a), rsz = (uint32_t)(e_l - e_a);
-            uint32_t lv = (uint32_t)tid < lsz ? sh.lflag[tid] : 0u;
-            uint32_t rv = (uint32_t)tid < rsz ? sh.rflag[tid] : 0u;
-            uint32_t ltot, rtot;
-            uint32_t lex = block_exscan(lv, sh.tmp, &ltot);
-            uint32_t rex = block_exscan(rv, sh.tmp, &rtot);
-            // lflag[t] <- number flagged in [t, lsz); rflag[t] <- number flagged in [0, t]
-            __syncthreads();
-            if ((uint32_t)tid < lsz) sh.lflag[tid] = ltot - lex;
-            if ((uint32_t)tid == lsz) sh.lflag[tid] = 0;
-            if ((uint32_t)tid < rsz) sh.rflag[tid] = rex + rv;
-            // bitonic sort of the candidates by key
-            uint32_t np2 = 1;
-            while (np2 < cc) np2 <<= 1;
-            for (uint32_t t = cc + tid; t < np2; t += T) {
-                sh.ckey[t] = ~0ull;
-                sh.coff[t] = 0xffffffffu;
-            }
-            __syncthreads();
-            for (uint32_t kk = 2; kk <= np2; kk <<= 1) {
-                for (uint32_t jj = kk >> 1; jj > 0; jj >>= 1) {
-                    for (uint32_t t = tid; t < np2; t += T) {
-                        uint32_t u = t ^ jj;
-                        if (u > t) {
-                            bool up = (t & kk) == 0;
-                            uint64_t kt = sh.ckey[t], ku = sh.ckey[u];
-                            if ((kt > ku) == up) {
-                                sh.ckey[t] = ku;
-                                sh.ckey[u] = kt;
-                                uint32_t o = sh.coff[t];
-                                sh.coff[t] = sh.coff[u];
-                                sh.coff[u] = o;
-                            }
-                        }
+                if (attempt == 3) {
+                    atomicMin(&sh.kmin, (unsigned long long)k);
+                    atomicMax(&sh.kmax, (unsigned long long)k);
+                }
+            };
+            uint32_t below = 0;
+            {
+                const int64_t step = NT;
+                int64_t p = c0 + tid;
+                for (; p + 7 * step <= c1; p += 8 * step) {
+                    unsigned long long v[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) v[i] = xb[p + i * step];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const uint32_t k = hi_key(v[i]);
+                        below += k < klo;
+                        if (k - klo <= span) keep(v[i], p + i * step);
                     }
-                    __syncthreads();
+                }
+                for (; p <= c1; p += step) {
+                    const unsigned long long v = xb[p];
+                    const uint32_t k = hi_key(v);
+                    below += k < klo;
+                    if (k - klo <= span) keep(v, p);
                 }
             }
-            if (active) {
-                uint32_t lcnt = (s_i < s_l) ? sh.lflag[(uint32_t)(s_i - s_a)] : 0u;
-                uint32_t rcnt = (e_i > e_a) ? sh.rflag[(uint32_t)(e_i - e_a - 1)] : 0u;
-                int64_t below = (int64_t)c_below + lcnt + rcnt;
-                int64_t t1 = r1 - below, t2 = r2 - below;
-                uint32_t so = (uint32_t)(s_i - s_a), eo = (uint32_t)(e_i - s_a);
-                int64_t c = 0;
-                uint64_t k1 = 0, k2 = 0;
-                bool got2 = false;
-                if (t1 >= 0) {
-                    for (uint32_t j = 0; j < cc; ++j) {
-                        uint32_t off = sh.coff[j];
-                        if (off >= so && off <= eo) {
-                            if (c == t1) k1 = sh.ckey[j];
-                            if (c == t2) {
-                                k2 = sh.ckey[j];
-                                got2 = true;
+            for (int side = 0; side < 2; ++side) {
+                const int64_t p0 = side ? e_a + 1 : s_a;
+                const int sz = side ? rsz : lsz;
+                for (int q0 = warp * 32; q0 < RM_MAXT; q0 += NT) {
+                    const int q = q0 + lane;
+                    bool lt = false;
+                    if (q < sz) {
+                        const unsigned long long v = xb[p0 + q];
+                        const uint32_t k = hi_key(v);
+                        lt = k < klo;
+                        if (k - klo <= span) keep(v, p0 + q);
+                    }
+                    const unsigned m = __ballot_sync(0xffffffffu, lt);
+                    if (lane == 0) (side ? sh.rbits : sh.lbits)[q0 >> 5] = m;
+                }
+            }
+            below = __reduce_add_sync(0xffffffffu, below);
+            if (lane == 0) atomicAdd(&sh.cbelow, below);
+            __syncthreads();
+            const uint32_t cc = sh.ccount;
+            if (cc > RM_CAP && attempt == 3 && sh.kmin == sh.kmax) {
+                // every possible median has the same value
+                for (int o = tid; o < no; o += NT) resid[a + o] = x[a + o] - dkey_inv(sh.kmin);
+                done = true;
+                known = false;
+                continue;
+            }
+            over = cc > RM_CAP;
+            if (over) {
+                __syncthreads();
+                continue;
+            }
+            for (int b = tid; b < RM_CAP / 32; b += NT) sh.fbits[b] = 0;
+            rm_sort(sh, cc);
+            for (uint32_t j = tid; j < cc; j += NT) {
+                const uint32_t off = sh.coff[sh.ord[j]];
+                if (off < (uint32_t)lsz || off > (uint32_t)(e_a - s_a)) atomicOr(&sh.fbits[j >> 5], 1u << (j & 31));
+            }
+            __syncthreads();
+            if (warp == 0) {
+                rm_word_prefix(sh.lbits, sh.lpre);
+                rm_word_prefix(sh.rbits, sh.rpre);
+                sh.l2bits[lane] = 0;
+                sh.r2bits[lane] = 0;
+                // the gathered fringe samples, in key order
+                const uint32_t cl = (uint32_t)lsz, cr = (uint32_t)(e_a - s_a);
+                uint32_t fb[RM_CAP / 1024], cnt = 0;
+#pragma unroll
+                for (int i = 0; i < RM_CAP / 1024; ++i) {
+                    fb[i] = sh.fbits[lane * (RM_CAP / 1024) + i];
+                    cnt += __popc(fb[i]);
+                }
+                uint32_t at = cnt;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t u = __shfl_up_sync(0xffffffffu, at, o);
+                    if (lane >= o) at += u;
+                }
+                if (lane == 31) sh.nf = at;
+                at -= cnt;
+#pragma unroll
+                for (int i = 0; i < RM_CAP / 1024; ++i) {
+                    while (fb[i]) {
+                        const uint32_t j = (uint32_t)(lane * (RM_CAP / 1024) + i) * 32 + __ffs(fb[i]) - 1;
+                        fb[i] &= fb[i] - 1;
+                        const uint32_t off = sh.coff[sh.ord[j]];
+                        sh.fringe[at++] = j | (off < cl ? off << 12 : ((off - cr - 1) << 12) | (1u << 23));
+                    }
+                }
+                if (lane == 0) {
+                    sh.mmin = 0xffffffffu;
+                    sh.mmax = 0u;
+                    sh.tmin = 0xffffffffu;
+                }
+            }
+            __syncthreads();
+            // ---- every output's order statistics
+            const uint32_t nf = sh.nf, cb = sh.cbelow;
+            // output o's windows: left fringe from q on, right fringe up to m;
+            // the first wanted rank among the gathered samples (< 0: below
+            // the bracket)
+            auto place = [&](int o, uint32_t& q, uint32_t& m, int64_t& t2) -> int64_t {
+                const int64_t s_i = win_s(a + o), e_i = win_e(a + o), n_i = e_i - s_i + 1;
+                q = (uint32_t)(s_i - s_a);
+                m = (uint32_t)(e_i - e_a);
+                const int64_t below_i = (int64_t)cb + sh.lpre[32] - rm_bits_before(sh.lbits, sh.lpre, q) +
+                                        rm_bits_before(sh.rbits, sh.rpre, m);
+                t2 = n_i / 2 - below_i;
+                return (n_i - 1) / 2 - below_i;
+            };
+            // Fringe samples sorted below every output's rank only count: how
+            // many are in the output's window comes from bit counts again, and
+            // the walk starts behind them.
+            {
+                uint32_t tm = 0xffffffffu;
+                for (int o = tid; o < no; o += NT) {
+                    uint32_t q, m;
+                    int64_t t2;
+                    const int64_t t1 = place(o, q, m, t2);
+                    tm = min(tm, (uint32_t)(t1 < 0 ? 0 : (t1 > RM_CAP ? RM_CAP : t1)));
+                }
+                tm = __reduce_min_sync(0xffffffffu, tm);
+                if (lane == 0) atomicMin(&sh.tmin, tm);
+            }
+            __syncthreads();
+            {
+                const uint32_t tmin = sh.tmin;
+                for (uint32_t j = tid; j < nf; j += NT) {
+                    const uint32_t e = sh.fringe[j], idx = (e >> 12) & 0x7ffu;
+                    if ((e & 0xfffu) < tmin) atomicOr((e >> 23) ? &sh.r2bits[idx >> 5] : &sh.l2bits[idx >> 5], 1u << (idx & 31));
+                }
+            }
+            __syncthreads();
+            if (warp == 0) {
+                rm_word_prefix(sh.l2bits, sh.l2pre);
+                rm_word_prefix(sh.r2bits, sh.r2pre);
+            }
+            __syncthreads();
+            const uint32_t nskip = sh.l2pre[32] + sh.r2pre[32];
+            uint32_t lo32 = 0xffffffffu, hi32 = 0u;
+            bool bad = false;
+            for (int o = tid; o < no; o += NT) {
+                uint32_t q, m;
+                int64_t t2;
+                const int64_t t1 = place(o, q, m, t2);
+                if (t1 < 0 || t2 >= (int64_t)cc) {
+                    bad = true;
+                    continue;
+                }
+                uint32_t t = (uint32_t)t1, j = nskip, at = 0;
+                uint32_t f = sh.l2pre[32] - rm_bits_before(sh.l2bits, sh.l2pre, q) + rm_bits_before(sh.r2bits, sh.r2pre, m);
+                uint64_t k1 = 0;
+                for (int want = 0; want < 2; ++want) {
+                    bool hit = false;
+                    for (; j < nf; ++j) {
+                        const uint32_t e = sh.fringe[j], sp = e & 0xfffu, idx = (e >> 12) & 0x7ffu;
+                        if (sp - j + f > t) break;  // a core sample comes first
+                        if ((e >> 23) ? idx < m : idx >= q) {
+                            if (sp - j + f == t) {
+                                hit = true;
+                                at = sp;
                                 break;
                             }
-                            ++c;
+                            ++f;
+                        }
+                    }
+                    if (!hit) at = t - f + j;
+                    if (at >= cc) {
+                        bad = true;
+                        break;
+                    }
+                    if (want == 0) k1 = sh.ckey[sh.ord[at]];
+                    if (t2 == t1) break;
+                    if (want == 0) {
+                        ++t;
+                        if (hit) {
+                            ++f;
+                            ++j;
                         }
                     }
                 }
-                if (!got2) {
-                    dev_fail(d_status, FFA_ERR_DEVICE);
-                    resid[i] = __longlong_as_double(0x7ff8000000000000ll);
-                } else {
-                    double v1 = dkey_inv(k1), v2 = dkey_inv(k2);
-                    double med = (t1 == t2) ? v1 : (v1 + v2) / 2;
-                    resid[i] = x[i] - med;
-                }
+                if (bad) continue;
+                const uint64_t k2 = sh.ckey[sh.ord[at]];
+                const double v1 = dkey_inv(k1), v2 = dkey_inv(k2);
+                const double med = (t1 == t2) ? v1 : (v1 + v2) / 2;
+                resid[a + o] = x[a + o] - med;
+                lo32 = min(lo32, (uint32_t)(k1 >> 32));
+                hi32 = max(hi32, (uint32_t)(k2 >> 32));
             }
-            return;
+            lo32 = __reduce_min_sync(0xffffffffu, lo32);
+            hi32 = __reduce_max_sync(0xffffffffu, hi32);
+            if (lane == 0) {
+                atomicMin(&sh.mmin, lo32);
+                atomicMax(&sh.mmax, hi32);
+            }
+            done = !__syncthreads_or(bad);
+            known = done;
+            if (done && tid == 0) {
+                // next tile: two ranges of this tile's medians to each side
+                const float r = (float)(dkey_inv(((uint64_t)sh.mmax << 32) | 0xffffffffull) - dkey_inv((uint64_t)sh.mmin << 32));
+                wide = fmaxf(2.0f * r, 0.7f * wide);
+                sh.pmin = sh.mmin;
+                sh.pmax = sh.mmax;
+            }
         }
-    }
-    if (!fast) {
-        if (!bracket_ok) dev_fail(d_status, FFA_ERR_DEVICE);
-        // slow exact path: per output, radix select over its own window
-        for (int64_t q = a; q <= l; ++q) {
-            int64_t s = win_s(q), e = win_e(q);
-            int64_t cnt = e - s + 1;
-            uint64_t k1 = cta_select_key(x, s, e, (uint32_t)((cnt - 1) / 2), sh);
-            uint64_t k2 = (cnt % 2 == 1) ? k1 : cta_select_key(x, s, e, (uint32_t)(cnt / 2), sh);
-            if (tid == 0) {
-                double v1 = dkey_inv(k1), v2 = dkey_inv(k2);
-                double med = (cnt % 2 == 1) ? v1 : (v1 + v2) / 2;
-                resid[q] = x[q] - med;
+        if (!done) {
+            known = false;
+            if (!bracket_ok) dev_fail(d_status, FFA_ERR_DEVICE);
+            // slow exact path: per output, radix select over its own window
+            for (int64_t q = a; q <= l; ++q) {
+                int64_t s = win_s(q), e = win_e(q);
+                int64_t cnt = e - s + 1;
+                uint64_t k1 = cta_select_key(x, s, e, (uint32_t)((cnt - 1) / 2), sh);
+                uint64_t k2 = (cnt % 2 == 1) ? k1 : cta_select_key(x, s, e, (uint32_t)(cnt / 2), sh);
+                if (tid == 0) {
+                    double v1 = dkey_inv(k1), v2 = dkey_inv(k2);
+                    double med = (cnt % 2 == 1) ? v1 : (v1 + v2) / 2;
+                    resid[q] = x[q] - med;
+                }
+                __syncthreads();
             }
-            __syncthreads();
+        }
+        __syncthreads();
+        ++tile;
+        if (++in_run == run) {
+            in_run = 0;
+            known = false;
+            tile += (int64_t)(gridDim.x - 1) * run;
         }
     }
 }
@@ -469,8 +792,18 @@ ffa_status launch_detrend(const double* d_raw, int64_t n, int32_t window, double
     size_t smem = sizeof(RmShared);
     ffa_status es = ensure_smem((const void*)k_runmed_tile, smem);
     if (es != FFA_OK) return es;
-    int64_t tiles = (n + T - 1) / T;
-    k_runmed_tile<<<(unsigned)tiles, T, smem, st>>>(d_raw, n, w, d_resid, d_status);
+    const int threads = T > 32 ? T / 2 : 32;
+    const int64_t tiles = (n + T - 1) / T;
+    // persistent: consecutive tiles in one CTA predict each other's bracket
+    int64_t grid = 0;
+    es = resident_ctas((const void*)k_runmed_tile, threads, smem, &grid);
+    if (es != FFA_OK) return es;
+    if (grid > tiles) grid = tiles;
+    // runs of at most 16 tiles, as many for every CTA: 456 CTAs' runs of 1024
+    // outputs cover 60 MB of the series, which L2 holds
+    const int64_t rounds = (tiles + grid * 16 - 1) / (grid * 16);
+    const int64_t run = (tiles + grid * rounds - 1) / (grid * rounds);
+    k_runmed_tile<<<(unsigned)grid, threads, smem, st>>>(d_raw, n, w, T, tiles, run, d_resid, d_status);
     FFA_LAUNCH_CHECK("k_runmed_tile");
     count_launch();
     return FFA_OK;
