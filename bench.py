@@ -527,10 +527,10 @@ def run_gpu(args):
                 "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
                 "kernel": ("fold passes (k_fold) + Algorithm 1 scorer with the last FFA stage fused "
-                           f"(k_score2) of one base period; {n_s} sampled base periods"),
+                           f"(k_score1) of one base period; {n_s} sampled base periods"),
                 "bytes": "algorithmic per base period: 4*M_data*P0 (series read once) + 16*M (records)",
                 "search_frac": search_gbs / peak, "search_gbs": search_gbs, "search_bytes": s_bytes,
-                "alu": {"kernel": "k_score2", "achieved_tops": alu_achieved, "peak_tops": alu_pk,
+                "alu": {"kernel": "k_score1", "achieved_tops": alu_achieved, "peak_tops": alu_pk,
                         "frac": alu_achieved / alu_pk, "unit": "T int/FP32 ops/s",
                         "ops": "per bin: last-stage add + 2 per width + 3 (selections, deviation)",
                         "peak_from": "SMs x 128 FP32/INT32 lanes x 2070 MHz",

@@ -89,14 +89,14 @@ ffa_status tune_fold(const void* d_z, int32_t precision, int64_t p0, int64_t m_d
 // plane after all but the last FFA stage (m_rows rows); the kernel applies the
 // last stage while loading.  Otherwise d_prof holds ready profiles.  Rows
 // (profiles) are `ld` elements apart.
-ffa_status launch_score2(const void* d_prof, int32_t precision, bool fused, int64_t count,
+ffa_status launch_score_alg1(const void* d_prof, int32_t precision, bool fused, int64_t count,
                          int64_t trial0, int64_t p0, int64_t ld, int64_t m_rows, const ScoreWidths& wd,
                          ffa_record* d_rec, int32_t* d_status, cudaStream_t st);
 // The fused scorers over a group of n base periods sharing m_rows and the
 // widths: planes at element offsets off[i] of d_plane (rows
 // plane_pitch(p0[i]) apart), the m_rows records of entry i at recs[i] (host
 // array of device pointers; entries may belong to different series).
-ffa_status launch_score2_group(const void* d_plane, int32_t precision, int n, const int64_t* p0, const int64_t* off,
+ffa_status launch_score_alg1_group(const void* d_plane, int32_t precision, int n, const int64_t* p0, const int64_t* off,
                                int64_t m_rows, const ScoreWidths& wd, ffa_record* const* recs, int32_t* d_status,
                                cudaStream_t st);
 ffa_status launch_score_alg2_group(const void* d_plane, int32_t precision, int n, const int64_t* p0,

@@ -4,7 +4,10 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "internal.h"
@@ -99,6 +102,318 @@ template <int R>
 __device__ __forceinline__ uint32_t bin_addr(uint32_t j) {  // byte address of bin j
     constexpr uint32_t QB = R / 4;
     return (((j << 2) & ~15u) ^ (((j >> 5) & (QB - 1)) << 4)) | ((j & 3) << 2);
+}
+
+// The block offsets' element: float-float (a float2) or wrapping int32.
+template <class V>
+struct Offset {
+    using type = float2;
+};
+template <>
+struct Offset<int32_t> {
+    using type = int32_t;
+};
+// Difference of two block offsets, box sums of prefixes: wrapping for int
+// profiles (exact for box sums below 2^31), rounded to nearest for float.
+__device__ __forceinline__ float off_diff(float2 b, float2 a) {
+    return __fadd_rn(__fsub_rn(b.x, a.x), __fsub_rn(b.y, a.y));
+}
+__device__ __forceinline__ int32_t off_diff(int32_t b, int32_t a) { return (int32_t)((uint32_t)b - (uint32_t)a); }
+__device__ __forceinline__ float box_sub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ int32_t box_sub(int32_t a, int32_t b) { return (int32_t)((uint32_t)a - (uint32_t)b); }
+__device__ __forceinline__ float box_add(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ int32_t box_add(int32_t a, int32_t b) { return (int32_t)((uint32_t)a + (uint32_t)b); }
+__device__ __forceinline__ float box_lowest(float) { return -INFINITY; }
+__device__ __forceinline__ int32_t box_lowest(int32_t) { return INT32_MIN; }
+
+template <bool ONE>
+__device__ __forceinline__ void cta_sync() {
+    if (ONE) __syncwarp();
+    else __syncthreads();
+}
+
+template <class V>
+__device__ __forceinline__ void load_quad(const unsigned char* smem, uint32_t a, V (&v)[4]) {
+    *reinterpret_cast<int4*>(v) = *reinterpret_cast<const int4*>(smem + a);
+}
+template <class V, int R>
+__device__ __forceinline__ V load_bin(const unsigned char* smem, uint32_t j) {
+    return *reinterpret_cast<const V*>(smem + bin_addr<R>(j));
+}
+
+// Load a profile into shared memory: hrow's p0 bins, plus (two) trow's read
+// sft bins further on, four bins at a time; acc(v) sees every bin once.
+template <class V, int R, class Acc>
+__device__ __forceinline__ void load_profile(unsigned char* smem, const V* __restrict__ hrow, const V* __restrict__ trow,
+                                             int sft, bool two, int p0, int tid, int T, Acc acc) {
+    auto store_quad = [&](int q, const V (&v)[4]) {
+        *reinterpret_cast<int4*>(smem + (((uint32_t)q ^ (((uint32_t)q >> 3) & (R / 4 - 1))) << 4)) =
+            *reinterpret_cast<const int4*>(v);
+    };
+    const bool al = (reinterpret_cast<uintptr_t>(hrow) & 15) == 0;
+    const int nq4 = p0 >> 2;
+    auto load_head = [&](int q, V (&h)[4]) {
+        if (al) {
+            *reinterpret_cast<int4*>(h) = *reinterpret_cast<const int4*>(hrow + 4 * q);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) h[i] = hrow[4 * q + i];
+        }
+    };
+    if (two) {
+#pragma unroll 4
+        for (int q = tid; q < nq4; q += T) {
+            V h[4], t[4];
+            load_head(q, h);
+            int o = 4 * q + sft;
+            if (o >= p0) o -= p0;
+            if (o + 3 < p0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) t[i] = trow[o + i];
+            } else {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) t[i] = trow[o + i < p0 ? o + i : o + i - p0];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                h[i] = h[i] + t[i];
+                acc(h[i]);
+            }
+            store_quad(q, h);
+        }
+    } else {
+#pragma unroll 4
+        for (int q = tid; q < nq4; q += T) {
+            V h[4];
+            load_head(q, h);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) acc(h[i]);
+            store_quad(q, h);
+        }
+    }
+    if (tid < (p0 & 3)) {
+        const int j = 4 * nq4 + tid;
+        V v = hrow[j];
+        if (two) v = v + trow[j + sft < p0 ? j + sft : j + sft - p0];
+        *reinterpret_cast<V*>(smem + bin_addr<R>(j)) = v;
+        acc(v);
+    }
+}
+
+// Cyclic extension: bins p0 .. nbx * R - 1 repeat the profile.
+template <class V, int R>
+__device__ __forceinline__ void extend_profile(unsigned char* smem, int p0, int nbx, int first, int step) {
+    const int ext = nbx * R - p0;
+    for (int j = first; j < ext; j += step) {
+        int s = j;
+        while (s >= p0) s -= p0;  // at most once for profiles longer than the extension
+        *reinterpret_cast<V*>(smem + bin_addr<R>(p0 + j)) = load_bin<V, R>(smem, s);
+    }
+}
+
+// Block offsets: the exclusive scan of the block totals that offs holds (a
+// float2's x), in segments of 128 blocks, four per lane -- the same tree
+// whatever the CTA's size.  Ends with a barrier.
+template <class V, bool ONE>
+__device__ __forceinline__ void scan_offsets(typename Offset<V>::type* offs, float2* seg, int nbx) {
+    constexpr bool INT = !std::is_same<V, float>::value;
+    const int lane = threadIdx.x & 31, warp = ONE ? 0 : threadIdx.x >> 5, NW = ONE ? 1 : blockDim.x >> 5;
+    const int nseg = (nbx + 127) >> 7;
+    float ch = 0.0f, cl = 0.0f;  // ONE: carry
+    uint32_t ci = 0;
+    for (int sgm = warp; sgm < nseg; sgm += NW) {
+        const int b0 = (sgm << 7) + 4 * lane;
+        if constexpr (INT) {
+            uint32_t v[4], s = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = b0 + i < nbx ? (uint32_t)offs[b0 + i] : 0u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t u = v[i];
+                v[i] = s;
+                s += u;
+            }
+            uint32_t x = s;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t u = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += u;
+            }
+            const uint32_t ex = x - s + ci;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (b0 + i < nbx) offs[b0 + i] = (int)(ex + v[i]);
+            const uint32_t tot = __shfl_sync(0xffffffffu, x, 31);
+            if (ONE) ci += tot;
+            else if (lane == 0) seg[sgm].x = __uint_as_float(tot);
+        } else {
+            float v[4], h[4], l[4], sh_ = 0.0f, sl = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = b0 + i < nbx ? offs[b0 + i].x : 0.0f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                h[i] = sh_;
+                l[i] = sl;
+                ff_acc(sh_, sl, v[i], 0.0f);
+            }
+            float xh = sh_, xl = sl;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const float uh = __shfl_up_sync(0xffffffffu, xh, o);
+                const float ul = __shfl_up_sync(0xffffffffu, xl, o);
+                if (lane >= o) ff_acc(xh, xl, uh, ul);
+            }
+            ff_norm(xh, xl);
+            float eh = __shfl_up_sync(0xffffffffu, xh, 1), el = __shfl_up_sync(0xffffffffu, xl, 1);
+            if (lane == 0) eh = el = 0.0f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                ff_acc(h[i], l[i], eh, el);
+                ff_norm(h[i], l[i]);
+                if (ONE) {
+                    ff_acc(h[i], l[i], ch, cl);
+                    ff_norm(h[i], l[i]);
+                }
+                if (b0 + i < nbx) offs[b0 + i] = make_float2(h[i], l[i]);
+            }
+            const float th = __shfl_sync(0xffffffffu, xh, 31), tl = __shfl_sync(0xffffffffu, xl, 31);
+            if (ONE) {
+                ff_acc(ch, cl, th, tl);
+                ff_norm(ch, cl);
+            } else if (lane == 0) {
+                seg[sgm] = make_float2(th, tl);
+            }
+        }
+    }
+    cta_sync<ONE>();
+    if (!ONE && nseg > 1) {
+        // add the earlier segments' totals
+        for (int sgm = warp ? warp : NW; sgm < nseg; sgm += NW) {
+            if constexpr (INT) {
+                uint32_t base = 0;
+                for (int i = 0; i < sgm; ++i) base += __float_as_uint(seg[i].x);
+                for (int b = (sgm << 7) + lane; b < nbx && b < (sgm + 1) << 7; b += 32)
+                    offs[b] = (int)((uint32_t)offs[b] + base);
+            } else {
+                float bh = 0.0f, bl = 0.0f;
+                for (int i = 0; i < sgm; ++i) {
+                    const float2 t = seg[i];
+                    ff_acc(bh, bl, t.x, t.y);
+                    ff_norm(bh, bl);
+                }
+                for (int b = (sgm << 7) + lane; b < nbx && b < (sgm + 1) << 7; b += 32) {
+                    float2 o = offs[b];
+                    ff_acc(o.x, o.y, bh, bl);
+                    ff_norm(o.x, o.y);
+                    offs[b] = o;
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Widths 2^n of wmask: M[n] = the largest box of width 2^n that starts in
+// this thread's items (first, first + step, ... < nitem; an item is min(R, 16)
+// bins of a block).  A block's largest box is its offset difference plus its
+// largest difference of in-block prefixes (rounding is monotone).
+template <class V, int R, int NS>
+__device__ __forceinline__ void width_maxima(const unsigned char* smem, const typename Offset<V>::type* offs,
+                                             uint32_t wmask, int first, int step, int nitem, V (&M)[NS]) {
+    constexpr int P = R < 16 ? R : 16;
+    constexpr int PARTS = R / P;
+    constexpr int LR = R == 8 ? 3 : (R == 16 ? 4 : 5);
+    const V lowest = box_lowest((V)0);
+#pragma unroll
+    for (int n = 0; n < NS; ++n) M[n] = lowest;
+    for (int im = first; im < nitem; im += step) {
+        const int b = im / PARTS, hf = im % PARTS;
+        const uint32_t a = blk_addr<R>((uint32_t)b) ^ (uint32_t)(hf * (P * 4));
+        const auto o1 = offs[b];
+        V c[P];
+#pragma unroll
+        for (int s = 0; s < P / 4; ++s) load_quad(smem, a ^ (s << 4), *reinterpret_cast<V(*)[4]>(&c[4 * s]));
+        // the next part: the same block's (offset 0), or the next block's
+        const bool last = hf == PARTS - 1;
+        const uint32_t an = last ? blk_addr<R>((uint32_t)b + 1) : a ^ (uint32_t)(P * 4);
+        V xd = 0;
+        if (last) xd = off_diff(offs[b + 1], o1);
+        if (wmask & 15u) {
+            V nx[8];
+            load_quad(smem, an, *reinterpret_cast<V(*)[4]>(&nx[0]));
+            if (R > 8) load_quad(smem, an ^ 16, *reinterpret_cast<V(*)[4]>(&nx[4]));
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                if ((1 << n) >= R || !(wmask >> n & 1u)) continue;
+                const int w = 1 << n;
+                V m = lowest, mx = lowest;
+#pragma unroll
+                for (int r = 0; r + w < P; r += 2) {
+                    if (r + 1 + w < P) m = max3(m, box_sub(c[r + w], c[r]), box_sub(c[r + 1 + w], c[r + 1]));
+                    else m = max3(m, m, box_sub(c[r + w], c[r]));
+                }
+#pragma unroll
+                for (int i = 0; i < w; i += 2) {
+                    if (i + 1 < w) mx = max3(mx, box_sub(nx[i], c[P - w + i]), box_sub(nx[i + 1], c[P - w + i + 1]));
+                    else mx = max3(mx, mx, box_sub(nx[i], c[P - w + i]));
+                }
+                M[n] = max3(M[n], m, box_add(xd, mx));
+            }
+        }
+        if (R == 32 && (wmask >> 4 & 1u)) {  // width 16 = one part further on
+            V m = lowest;
+#pragma unroll
+            for (int s = 0; s < P / 4; ++s) {
+                V v[4];
+                load_quad(smem, an ^ (s << 4), v);
+                m = max3(m, box_sub(v[0], c[4 * s]), box_sub(v[1], c[4 * s + 1]));
+                m = max3(m, box_sub(v[2], c[4 * s + 2]), box_sub(v[3], c[4 * s + 3]));
+            }
+            M[4] = max3(M[4], M[4], box_add(xd, m));
+        }
+#pragma unroll
+        for (int n = LR; n < NS; ++n) {
+            if (!(wmask >> n & 1u)) continue;
+            const int d = 1 << (n - LR);
+            // eight or more blocks on, the swizzle is the same
+            const uint32_t a2 =
+                d >= 8 ? a + (uint32_t)(d * R * 4) : blk_addr<R>((uint32_t)(b + d)) ^ (uint32_t)(hf * (P * 4));
+            const V D = off_diff(offs[b + d], o1);
+            V m = lowest;
+#pragma unroll
+            for (int s = 0; s < P / 4; ++s) {
+                V v[4];
+                load_quad(smem, d >= 8 ? (a ^ (s << 4)) + (uint32_t)(d * R * 4) : a2 ^ (s << 4), v);
+                if constexpr (!std::is_same<V, float>::value) {
+                    m = max3(m, box_sub(v[0], c[4 * s]), box_sub(v[1], c[4 * s + 1]));
+                    m = max3(m, box_sub(v[2], c[4 * s + 2]), box_sub(v[3], c[4 * s + 3]));
+                } else {
+                    float d0, d1, d2, d3;
+                    asm("{\n\t.reg .b64 x, y, z;\n\t"
+                        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+                        : "=f"(d0), "=f"(d1)
+                        : "f"(v[0]), "f"(v[1]), "f"(c[4 * s]), "f"(c[4 * s + 1]));
+                    asm("{\n\t.reg .b64 x, y, z;\n\t"
+                        "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
+                        : "=f"(d2), "=f"(d3)
+                        : "f"(v[2]), "f"(v[3]), "f"(c[4 * s + 2]), "f"(c[4 * s + 3]));
+                    m = max3(m, d0, d1);
+                    m = max3(m, d2, d3);
+                }
+            }
+            M[n] = max3(M[n], M[n], box_add(D, m));
+        }
+    }
+}
+
+// The box of width w that starts at bin j (of the extension's index space),
+// as width_maxima forms it.
+template <class V, int R>
+__device__ __forceinline__ V box_at(const unsigned char* smem, const typename Offset<V>::type* offs, int j, int w) {
+    const int b = j / R, b2 = (j + w) / R;
+    V bx = box_sub(load_bin<V, R>(smem, j + w), load_bin<V, R>(smem, j));
+    if (b2 != b) bx = box_add(off_diff(offs[b2], offs[b]), bx);
+    return bx;
 }
 
 }  // namespace ffa

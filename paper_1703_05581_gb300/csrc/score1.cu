@@ -101,12 +101,6 @@ __device__ __forceinline__ float sqrt_pow2(int n) {
     return __int_as_float((127 + (n >> 1)) << 23) * ((n & 1) ? 1.41421356237309515f : 1.0f);
 }
 
-template <bool ONE>
-__device__ __forceinline__ void cta_sync() {
-    if (ONE) __syncwarp();
-    else __syncthreads();
-}
-
 // Warp 0: the buckets of hist[0, n) (n a multiple of 128) that hold ranks
 // ta <= tb (both below the total), and the count before the first one.
 template <bool ONE>
@@ -155,7 +149,7 @@ __device__ __noinline__ unsigned long long radix_rank(const unsigned char* smem,
         for (int b = tid; b < 256; b += T) hist[b] = 0;
         cta_sync<ONE>();
         for (int j = tid; j < p0; j += T) {
-            const V v = *reinterpret_cast<const V*>(smem + bin_addr<R>((uint32_t)j));
+            const V v = load_bin<V, R>(smem, j);
             unsigned long long kk;
             if constexpr (std::is_integral<V>::value) {
                 const long long e = 2 * (long long)v - s2;
@@ -245,7 +239,6 @@ __global__ void __launch_bounds__(MAXT, MINB)
     constexpr bool INT = IsInt<V>::value;
     constexpr int P = R < 16 ? R : 16;  // bins per item of the width pass
     constexpr int PARTS = R / P;
-    constexpr int LR = R == 8 ? 3 : (R == 16 ? 4 : 5);
     constexpr int NS = R == 8 ? 12 : 16;  // widths 2^0 .. 2^(NS-1)
     constexpr int NB = score_nb(R);
     constexpr int NP = score_pack(R);
@@ -254,15 +247,11 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const int T = ONE ? 32 : (int)blockDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = ONE ? 0 : tid >> 5;
     const int NW = T >> 5;
-    float2* offs = reinterpret_cast<float2*>(smem + lay.offs);
-    int* offi = reinterpret_cast<int*>(smem + lay.offs);
+    using Off = typename Offset<V>::type;
+    Off* offs = reinterpret_cast<Off*>(smem + lay.offs);
     uint32_t* hist = reinterpret_cast<uint32_t*>(smem + lay.aux);
     float* pack = reinterpret_cast<float*>(smem + lay.aux);
     auto sync = [&]() { cta_sync<ONE>(); };
-    auto quad = [&](uint32_t a, V (&v)[4]) {
-        *reinterpret_cast<int4*>(v) = *reinterpret_cast<const int4*>(smem + a);
-    };
-    auto value = [&](uint32_t j) -> V { return *reinterpret_cast<const V*>(smem + bin_addr<R>(j)); };
     // block sums of two counts per thread (one barrier); slot alternates
     auto sum2 = [&](uint32_t a, uint32_t b, int slot) -> uint2 {
         a = __reduce_add_sync(0xffffffffu, a);
@@ -300,7 +289,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
 #pragma unroll
                 for (int s = 0; s < R / 4; ++s) {
                     V v[4], c[4];
-                    quad(a ^ (s << 4), v);
+                    load_quad(smem, a ^ (s << 4), v);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         c[i] = t;
@@ -308,8 +297,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
                     }
                     *reinterpret_cast<int4*>(smem + (a ^ (s << 4))) = *reinterpret_cast<const int4*>(c);
                 }
-                if constexpr (INT) offi[b] = (int)t;
-                else offs[b].x = (float)t;
+                if constexpr (INT) offs[b] = t;
+                else offs[b].x = t;
             }
         };
         bool prefixed = false;
@@ -342,58 +331,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
                 if (FUSED) asm volatile("prefetch.global.L2 [%0];" ::"l"(trow + ld + l * (128 / sizeof(V))));
             }
         }
-        auto store_quad = [&](int q, const V (&v)[4]) {
-            *reinterpret_cast<int4*>(smem + (((uint32_t)q ^ (((uint32_t)q >> 3) & (R / 4 - 1))) << 4)) =
-                *reinterpret_cast<const int4*>(v);
-        };
-        const bool al = ((reinterpret_cast<uintptr_t>(hrow)) & 15) == 0;
-        const int nq4 = p0 >> 2;
-        auto load_head = [&](int q, V (&h)[4]) {
-            if (al) {
-                *reinterpret_cast<int4*>(h) = *reinterpret_cast<const int4*>(hrow + 4 * q);
-            } else {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) h[i] = hrow[4 * q + i];
-            }
-        };
-        if (two) {
-#pragma unroll 4
-            for (int q = tid; q < nq4; q += T) {
-                V h[4], t[4];
-                load_head(q, h);
-                int o = 4 * q + sft;
-                if (o >= p0) o -= p0;
-                if (o + 3 < p0) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) t[i] = trow[o + i];
-                } else {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) t[i] = trow[o + i < p0 ? o + i : o + i - p0];
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    h[i] = h[i] + t[i];
-                    acc(h[i]);
-                }
-                store_quad(q, h);
-            }
-        } else {
-#pragma unroll 4
-            for (int q = tid; q < nq4; q += T) {
-                V h[4];
-                load_head(q, h);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) acc(h[i]);
-                store_quad(q, h);
-            }
-        }
-        if (tid < (p0 & 3)) {
-            const int j = 4 * nq4 + tid;
-            V v = hrow[j];
-            if (two) v = v + trow[j + sft < p0 ? j + sft : j + sft - p0];
-            *reinterpret_cast<V*>(smem + bin_addr<R>(j)) = v;
-            acc(v);
-        }
+        load_profile<V, R>(smem, hrow, trow, sft, two, p0, tid, T, acc);
         if (INT)
             for (int b = 4 * tid; b < NB; b += 4 * T) *reinterpret_cast<int4*>(hist + b) = make_int4(0, 0, 0, 0);
         if (tid < 16) sh.wkey[tid] = 0u;
@@ -430,14 +368,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
         const float rsn = sqrtf(rn) * sig;  // sigma / sqrt(N)
         // cyclic extension: bins past p0 repeat the profile
         bool extended = false;
-        auto extend = [&](int first, int step) {
-            const int ext = nbx * R - p0;
-            for (int j = first; j < ext; j += step) {
-                int s = j;
-                while (s >= p0) s -= p0;  // at most once for profiles longer than the extension
-                *reinterpret_cast<V*>(smem + bin_addr<R>(p0 + j)) = value(s);
-            }
-        };
+        auto extend = [&](int first, int step) { extend_profile<V, R>(smem, p0, nbx, first, step); };
 
         // ---- median and MAD (Eq. 3), exact ----
         const uint32_t r1 = (uint32_t)((p0 - 1) / 2), r2 = (uint32_t)(p0 / 2);
@@ -471,11 +402,11 @@ __global__ void __launch_bounds__(MAXT, MINB)
                     };
                     for (int q = tid; q < nq; q += T) {
                         V v[4];
-                        quad((uint32_t)q << 4, v);
+                        load_quad(smem, (uint32_t)q << 4, v);
 #pragma unroll
                         for (int i = 0; i < 4; ++i) take(v[i]);
                     }
-                    for (int j = jt; j < p0; j += T) take(value(j));
+                    for (int j = jt; j < p0; j += T) take(load_bin<V, R>(smem, j));
                     // pack the threads' lists
                     const uint32_t nl = (ptr - lbase) >> 2;
                     if (nl) {
@@ -637,11 +568,11 @@ __global__ void __launch_bounds__(MAXT, MINB)
                     };
                     for (int q = tid; q < nq; q += T) {
                         V v[4];
-                        quad((uint32_t)q << 4, v);
+                        load_quad(smem, (uint32_t)q << 4, v);
 #pragma unroll
                         for (int i = 0; i < 4; ++i) take((int)v[i]);
                     }
-                    for (int j = jt; j < p0; j += T) take((int)value(j));
+                    for (int j = jt; j < p0; j += T) take((int)load_bin<V, R>(smem, j));
                     const uint2 c = sum2(below, in, a & 1);
                     if (r1 < c.x || r2 >= c.x + c.y) {
                         const int step = MAD ? 2 : 1;
@@ -704,206 +635,12 @@ __global__ void __launch_bounds__(MAXT, MINB)
             prefix(tid, T);
             sync();
         }
-        // block offsets: exclusive scan of the totals, in segments of 128
-        // blocks (four per lane; the same tree whatever the CTA's size)
-        {
-            const int nseg = (nbx + 127) >> 7;
-            float ch = 0.0f, cl = 0.0f;  // ONE: carry
-            uint32_t ci = 0;
-            for (int sgm = warp; sgm < nseg; sgm += NW) {
-                const int b0 = (sgm << 7) + 4 * lane;
-                if constexpr (INT) {
-                    uint32_t v[4], s = 0;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) v[i] = b0 + i < nbx ? (uint32_t)offi[b0 + i] : 0u;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const uint32_t u = v[i];
-                        v[i] = s;
-                        s += u;
-                    }
-                    uint32_t x = s;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const uint32_t u = __shfl_up_sync(0xffffffffu, x, o);
-                        if (lane >= o) x += u;
-                    }
-                    const uint32_t ex = x - s + ci;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        if (b0 + i < nbx) offi[b0 + i] = (int)(ex + v[i]);
-                    const uint32_t tot = __shfl_sync(0xffffffffu, x, 31);
-                    if (ONE) ci += tot;
-                    else if (lane == 0) sh.seg[sgm].x = __uint_as_float(tot);
-                } else {
-                    float v[4], h[4], l[4], sh_ = 0.0f, sl = 0.0f;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) v[i] = b0 + i < nbx ? offs[b0 + i].x : 0.0f;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        h[i] = sh_;
-                        l[i] = sl;
-                        ff_acc(sh_, sl, v[i], 0.0f);
-                    }
-                    float xh = sh_, xl = sl;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const float uh = __shfl_up_sync(0xffffffffu, xh, o);
-                        const float ul = __shfl_up_sync(0xffffffffu, xl, o);
-                        if (lane >= o) ff_acc(xh, xl, uh, ul);
-                    }
-                    ff_norm(xh, xl);
-                    float eh = __shfl_up_sync(0xffffffffu, xh, 1), el = __shfl_up_sync(0xffffffffu, xl, 1);
-                    if (lane == 0) eh = el = 0.0f;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        ff_acc(h[i], l[i], eh, el);
-                        ff_norm(h[i], l[i]);
-                        if (ONE) {
-                            ff_acc(h[i], l[i], ch, cl);
-                            ff_norm(h[i], l[i]);
-                        }
-                        if (b0 + i < nbx) offs[b0 + i] = make_float2(h[i], l[i]);
-                    }
-                    const float th = __shfl_sync(0xffffffffu, xh, 31), tl = __shfl_sync(0xffffffffu, xl, 31);
-                    if (ONE) {
-                        ff_acc(ch, cl, th, tl);
-                        ff_norm(ch, cl);
-                    } else if (lane == 0) {
-                        sh.seg[sgm] = make_float2(th, tl);
-                    }
-                }
-            }
-            sync();
-            if (!ONE && nseg > 1) {
-                // add the earlier segments' totals
-                for (int sgm = warp ? warp : NW; sgm < nseg; sgm += NW) {
-                    if constexpr (INT) {
-                        uint32_t base = 0;
-                        for (int i = 0; i < sgm; ++i) base += __float_as_uint(sh.seg[i].x);
-                        for (int b = (sgm << 7) + lane; b < nbx && b < (sgm + 1) << 7; b += 32)
-                            offi[b] = (int)((uint32_t)offi[b] + base);
-                    } else {
-                        float bh = 0.0f, bl = 0.0f;
-                        for (int i = 0; i < sgm; ++i) {
-                            const float2 t = sh.seg[i];
-                            ff_acc(bh, bl, t.x, t.y);
-                            ff_norm(bh, bl);
-                        }
-                        for (int b = (sgm << 7) + lane; b < nbx && b < (sgm + 1) << 7; b += 32) {
-                            float2 o = offs[b];
-                            ff_acc(o.x, o.y, bh, bl);
-                            ff_norm(o.x, o.y);
-                            offs[b] = o;
-                        }
-                    }
-                }
-                __syncthreads();
-            }
-        }
+        scan_offsets<V, ONE>(offs, sh.seg, nbx);
 
         // ---- widths: the largest box of each, per thread ----
-        auto boff = [&](int b) {
-            if constexpr (INT) return offi[b];
-            else return offs[b];
-        };
-        auto bdiff = [&](auto o2, auto o1) -> V {
-            if constexpr (INT) return (V)((uint32_t)o2 - (uint32_t)o1);
-            else return __fadd_rn(__fsub_rn(o2.x, o1.x), __fsub_rn(o2.y, o1.y));
-        };
-        auto sub = [](V a, V b) -> V {
-            if constexpr (INT) return (V)((uint32_t)a - (uint32_t)b);
-            else return __fsub_rn(a, b);
-        };
-        auto add = [](V a, V b) -> V {
-            if constexpr (INT) return (V)((uint32_t)a + (uint32_t)b);
-            else return __fadd_rn(a, b);
-        };
-        V lowest;
-        if constexpr (INT) lowest = INT32_MIN;
-        else lowest = -INFINITY;
         V M[NS];
-#pragma unroll
-        for (int n = 0; n < NS; ++n) M[n] = lowest;
         const int nitem = nblk * PARTS;
-        for (int im = tid; im < nitem; im += T) {
-            const int b = im / PARTS, hf = im % PARTS;
-            const uint32_t a = blk_addr<R>((uint32_t)b) ^ (uint32_t)(hf * (P * 4));
-            const auto o1 = boff(b);
-            V c[P];
-#pragma unroll
-            for (int s = 0; s < P / 4; ++s) quad(a ^ (s << 4), *reinterpret_cast<V(*)[4]>(&c[4 * s]));
-            // the next part: the same block's (offset 0), or the next block's
-            const bool last = hf == PARTS - 1;
-            const uint32_t an = last ? blk_addr<R>((uint32_t)b + 1) : a ^ (uint32_t)(P * 4);
-            V xd = 0;
-            if (last) xd = bdiff(boff(b + 1), o1);
-            if (wmask & 15u) {
-                V nx[8];
-                quad(an, *reinterpret_cast<V(*)[4]>(&nx[0]));
-                if (R > 8) quad(an ^ 16, *reinterpret_cast<V(*)[4]>(&nx[4]));
-#pragma unroll
-                for (int n = 0; n < 4; ++n) {
-                    if ((1 << n) >= R || !(wmask >> n & 1u)) continue;
-                    const int w = 1 << n;
-                    V m = lowest, mx = lowest;
-#pragma unroll
-                    for (int r = 0; r + w < P; r += 2) {
-                        if (r + 1 + w < P) m = max3(m, sub(c[r + w], c[r]), sub(c[r + 1 + w], c[r + 1]));
-                        else m = max3(m, m, sub(c[r + w], c[r]));
-                    }
-#pragma unroll
-                    for (int i = 0; i < w; i += 2) {
-                        if (i + 1 < w) mx = max3(mx, sub(nx[i], c[P - w + i]), sub(nx[i + 1], c[P - w + i + 1]));
-                        else mx = max3(mx, mx, sub(nx[i], c[P - w + i]));
-                    }
-                    M[n] = max3(M[n], m, add(xd, mx));
-                }
-            }
-            if (R == 32 && (wmask >> 4 & 1u)) {  // width 16 = one part further on
-                V m = lowest;
-#pragma unroll
-                for (int s = 0; s < P / 4; ++s) {
-                    V v[4];
-                    quad(an ^ (s << 4), v);
-                    m = max3(m, sub(v[0], c[4 * s]), sub(v[1], c[4 * s + 1]));
-                    m = max3(m, sub(v[2], c[4 * s + 2]), sub(v[3], c[4 * s + 3]));
-                }
-                M[4] = max3(M[4], M[4], add(xd, m));
-            }
-#pragma unroll
-            for (int n = LR; n < NS; ++n) {
-                if (!(wmask >> n & 1u)) continue;
-                const int d = 1 << (n - LR);
-                // eight or more blocks on, the swizzle is the same
-                const uint32_t a2 = d >= 8 ? a + (uint32_t)(d * R * 4)
-                                           : blk_addr<R>((uint32_t)(b + d)) ^ (uint32_t)(hf * (P * 4));
-                const V D = bdiff(boff(b + d), o1);
-                V m = lowest;
-#pragma unroll
-                for (int s = 0; s < P / 4; ++s) {
-                    V v[4];
-                    quad(d >= 8 ? (a ^ (s << 4)) + (uint32_t)(d * R * 4) : a2 ^ (s << 4), v);
-                    if constexpr (INT) {
-                        m = max3(m, sub(v[0], c[4 * s]), sub(v[1], c[4 * s + 1]));
-                        m = max3(m, sub(v[2], c[4 * s + 2]), sub(v[3], c[4 * s + 3]));
-                    } else {
-                        float d0, d1, d2, d3;
-                        asm("{\n\t.reg .b64 x, y, z;\n\t"
-                            "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
-                            : "=f"(d0), "=f"(d1)
-                            : "f"(v[0]), "f"(v[1]), "f"(c[4 * s]), "f"(c[4 * s + 1]));
-                        asm("{\n\t.reg .b64 x, y, z;\n\t"
-                            "mov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 z, x, y;\n\tmov.b64 {%0, %1}, z;\n\t}"
-                            : "=f"(d2), "=f"(d3)
-                            : "f"(v[2]), "f"(v[3]), "f"(c[4 * s + 2]), "f"(c[4 * s + 3]));
-                        m = max3(m, d0, d1);
-                        m = max3(m, d2, d3);
-                    }
-                }
-                M[n] = max3(M[n], M[n], add(D, m));
-            }
-        }
+        width_maxima<V, R, NS>(smem, offs, wmask, tid, T, nitem, M);
         // lane n of each warp: the warp's maximum of width 2^n; then the CTA's
         uint32_t wk = 0;
 #pragma unroll
@@ -983,7 +720,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
             V target;
             if constexpr (INT) target = (V)(int32_t)(sh.wkey[bw] ^ 0x80000000u);
             else target = (V)fkey_inv(sh.wkey[bw]);
-            V own = lowest;
+            V own = box_lowest((V)0);
 #pragma unroll
             for (int n = 0; n < NS; ++n)
                 if (n == bw) own = M[n];
@@ -997,11 +734,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
                     const int im = src + (i0 + lane / P) * T;
                     uint32_t f = 0x7fffffffu;
                     if (im < nitem) {
-                        const int b = im / PARTS, r = (im % PARTS) * P + lane % P;
-                        const int j = b * R + r, b2 = (j + w) / R;
-                        V bx = sub(value(j + w), value(j));
-                        if (b2 != b) bx = add(bdiff(boff(b2), boff(b)), bx);
-                        if (bx == target) f = (uint32_t)(j < p0 ? j : j % p0);
+                        const int j = (im / PARTS) * R + (im % PARTS) * P + lane % P;
+                        if (box_at<V, R>(smem, offs, j, w) == target) f = (uint32_t)(j < p0 ? j : j % p0);
                     }
                     f = __reduce_min_sync(0xffffffffu, f);
                     if (lane == 0 && f != 0x7fffffffu) atomicMin(&sh.pos, f);
@@ -1135,14 +869,54 @@ ffa_status score1_dispatch(const void* d_prof, const ScoreGroup& sg, int32_t pre
 
 }  // namespace
 
-ffa_status launch_score2(const void* d_prof, int32_t precision, bool fused, int64_t count, int64_t trial0, int64_t p0,
+// The scorers' block length by profile length: 0: 8 bins (up to 2048), 1: 16
+// (up to 8192), 2: 16, 3: 32, -1: too long; the extension by the widest box
+// counts too.  Grouped launches hold one shape only, so that a profile's
+// record does not depend on what it is grouped with.
+int score_shape(int64_t p0, int wmax) {
+    auto fits = [&](int64_t r, int64_t blocks, int64_t ext) {
+        return p0 >= 1 && (p0 + r - 1) / r <= blocks && (p0 + wmax + r) / r + 1 <= ext;
+    };
+    return fits(8, 256, 512) ? 0 : fits(16, 512, 1024) ? 1 : fits(16, 1024, 2048) ? 2 : fits(32, 1024, 2048) ? 3 : -1;
+}
+
+ScoreGroup score_single(int64_t p0, int64_t ld, int64_t count, ffa_record* d_rec) {
+    ScoreGroup sg;
+    sg.n = 1;
+    sg.t0[0] = 0;
+    sg.t0[1] = count;
+    sg.p0[0] = (int32_t)p0;
+    sg.off[0] = 0;
+    sg.ld[0] = ld;
+    sg.rec[0] = d_rec;
+    return sg;
+}
+
+ScoreGroup score_group(int n, const int64_t* p0, const int64_t* off, int64_t m_rows, ffa_record* const* recs,
+                       int64_t* p0max) {
+    ScoreGroup sg;
+    sg.n = n;
+    *p0max = 0;
+    for (int i = 0; i < n; ++i) {
+        sg.t0[i] = (int64_t)i * m_rows;
+        sg.p0[i] = (int32_t)p0[i];
+        sg.off[i] = off[i];
+        sg.ld[i] = plane_pitch(p0[i]);
+        sg.rec[i] = recs[i];
+        *p0max = p0[i] > *p0max ? p0[i] : *p0max;
+    }
+    sg.t0[n] = (int64_t)n * m_rows;
+    return sg;
+}
+
+ffa_status launch_score_alg1(const void* d_prof, int32_t precision, bool fused, int64_t count, int64_t trial0, int64_t p0,
                          int64_t ld, int64_t m_rows, const ScoreWidths& wd, ffa_record* d_rec, int32_t* d_status,
                          cudaStream_t st) {
     return score1_dispatch(d_prof, score_single(p0, ld, count, d_rec), precision, fused, count, trial0, p0, m_rows, wd,
                            d_status, st);
 }
 
-ffa_status launch_score2_group(const void* d_plane, int32_t precision, int n, const int64_t* p0, const int64_t* off,
+ffa_status launch_score_alg1_group(const void* d_plane, int32_t precision, int n, const int64_t* p0, const int64_t* off,
                                int64_t m_rows, const ScoreWidths& wd, ffa_record* const* recs, int32_t* d_status,
                                cudaStream_t st) {
     if (n < 1 || n > FOLD_GROUP_MAX) return fail(FFA_ERR_ARG, "score group: 1..FOLD_GROUP_MAX base periods");

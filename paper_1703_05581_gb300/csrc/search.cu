@@ -14,6 +14,7 @@
 #include <new>
 #include <string>
 #include <thread>
+#include <tuple>
 #include <utility>
 #include <vector>
 
@@ -51,6 +52,32 @@ int sm_count() {
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
     cache[dev] = n;
     return n;
+}
+
+// Resident CTAs of a kernel for a dynamic shared-memory size, times the SM
+// count, per device: queried once (launches come per base period).
+ffa_status resident_ctas(const void* fn, int threads, size_t smem, int64_t* out) {
+    static std::mutex mu;
+    static std::map<std::tuple<const void*, size_t, int>, int64_t> cache;
+    int dev = 0;
+    FFA_CUDA_TRY(cudaGetDevice(&dev));
+    const auto key = std::make_tuple(fn, smem, dev);
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        auto it = cache.find(key);
+        if (it != cache.end()) {
+            *out = it->second;
+            return FFA_OK;
+        }
+    }
+    int nsm = 0, per_sm = 0;
+    FFA_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    FFA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem));
+    const int64_t r = (int64_t)nsm * (per_sm < 1 ? 1 : per_sm);
+    std::lock_guard<std::mutex> lk(mu);
+    cache[key] = r;
+    *out = r;
+    return FFA_OK;
 }
 
 ffa_status ensure_smem(const void* func, size_t bytes) {
@@ -634,7 +661,7 @@ static ffa_status search_range(const ffa_plan* p, const void* d_series, void* d_
                 if (c.scorer == FFA_SCORE_ALG2)
                     s = launch_score_alg2_group(plane0, c.precision, n, p0s, offs, e.m_rows, wd, excl, recs, st);
                 else
-                    s = launch_score2_group(plane0, c.precision, n, p0s, offs, e.m_rows, wd, recs, d_status, st);
+                    s = launch_score_alg1_group(plane0, c.precision, n, p0s, offs, e.m_rows, wd, recs, d_status, st);
                 if (s != FFA_OK) return s;
                 gscore_k.stop();
                 if (d_persist) {
@@ -665,7 +692,7 @@ static ffa_status search_range(const ffa_plan* p, const void* d_series, void* d_
                 s = launch_score_alg2(plane0, c.precision, true, e.m_rows, 0, e.p0, ld, e.m_rows, wd, excl,
                                       d_records + e.first_trial, st);
             else
-                s = launch_score2(plane0, c.precision, true, e.m_rows, 0, e.p0, ld, e.m_rows, wd,
+                s = launch_score_alg1(plane0, c.precision, true, e.m_rows, 0, e.p0, ld, e.m_rows, wd,
                                   d_records + e.first_trial, d_status, st);
             if (s != FFA_OK) return s;
             score_k.stop();
@@ -992,7 +1019,7 @@ ffa_status ffa_search_batch(const ffa_plan* const* plans, const void* const* d_s
             if (c.scorer == FFA_SCORE_ALG2)
                 s = launch_score_alg2_group(plane0, c.precision, n, p0s, offs, e0.m_rows, wd, excl, recs, st);
             else
-                s = launch_score2_group(plane0, c.precision, n, p0s, offs, e0.m_rows, wd, recs, d_status, st);
+                s = launch_score_alg1_group(plane0, c.precision, n, p0s, offs, e0.m_rows, wd, recs, d_status, st);
             if (s != FFA_OK) return s;
             t = j;
         }
@@ -1192,7 +1219,7 @@ ffa_status ffa_score(const void* d_profiles, int32_t precision, int64_t count, i
     }
     if (count > 0 && (!d_profiles || !d_records)) return fail(FFA_ERR_ARG, "score: null buffer");
     if (precision != FFA_FOLD_F32 && precision != FFA_FOLD_I8) return fail(FFA_ERR_ARG, "score: bad precision");
-    return launch_score2(d_profiles, precision, false, count, 0, p0, p0, 1, wd, d_records, d_status,
+    return launch_score_alg1(d_profiles, precision, false, count, 0, p0, p0, 1, wd, d_records, d_status,
                          as_stream(stream));
 }
 

@@ -98,3 +98,25 @@ def test_wide_integers(F, orc):
     ref = np.array([orc.score_alg1(p.astype(np.int64), (1,)) for p in prof])
     ref["snr"] = ref["snr"].astype(np.float32)  # a record holds the rounded quotient
     check_records(got, ref, lambda i: prof[i].astype(np.float64), tol=0.0)
+
+
+@pytest.mark.parametrize("p0", [1, 2, 5, 8, 33, 257, 2047, 2049, 4201, 8193, 16385, 31249])
+@pytest.mark.parametrize("integer", [False, True])
+def test_alg2_block_edges(F, orc, p0, integer):
+    """Algorithm 2 at lengths around blocks, chunks and CTA shapes, with a box
+    that starts in the last, partial block and a flat profile."""
+    import torch
+    rng = np.random.default_rng(p0 * 5 + integer)
+    x = rng.standard_normal((6, p0)) * 37.0
+    x[1, -1] += 900.0
+    x[2, np.arange(p0 - min(p0, 9), p0 + min(p0, 9)) % p0] += 300.0
+    x[3, :] = 4.0
+    prof = np.rint(x).astype(np.int32) if integer else x.astype(np.float32)
+    widths = _widths(p0)
+    rec = F.score_alg2(torch.from_numpy(prof).cuda(), widths)
+    got = F.records_numpy(rec, prof.shape[0])
+    ref = np.array([orc.score_alg2(p.astype(np.float64), widths) for p in prof])
+    # FP32 sums of the profile and of the window: 1e-4 of the score, as for the
+    # other lengths this scorer is compared at
+    tol = 1e-3 + 1e-4 * float(np.abs(ref["snr"]).max())
+    check_records(got, ref, lambda i: prof[i].astype(np.float64), tol=tol, scorer=2)
