@@ -68,8 +68,9 @@ ffa_status launch_persist(const int32_t* d_bplane, int64_t m_rows, int64_t p0, i
 inline int64_t plane_pitch(int64_t p0) { return (p0 + 3) & ~(int64_t)3; }
 
 // Base periods per grouped launch (fold, score): small planes are folded
-// and scored together so that a launch fills the GPU.
-constexpr int FOLD_GROUP_MAX = 32;
+// and scored together so that a launch fills the GPU (their by-value tables
+// take up to 3 KB of the 4 KB of kernel parameters).
+constexpr int FOLD_GROUP_MAX = 64;
 // Fold n base periods sharing m_rows (and their tuned pass depth) in one set
 // of launches: entry i has p0[i] bins, m_data[i] rows of the series z[i]
 // (host array of device pointers, or null: every entry reads d_z), its plane
@@ -109,6 +110,8 @@ ffa_status launch_score_alg2(const void* d_prof, int32_t precision, bool fused, 
 
 // The scorer's CTA shape (0..3) for profiles of p0 bins and widths up to wmax.
 int score_shape(int64_t p0, int wmax);
+// Blocks of one group of a shape's block-offset scan (part of its sums' order).
+int score_scan_group(int shape);
 
 // ffa2best on a plan's records (defined in best.cu); workspace bytes it needs.
 size_t best_workspace_bytes(int64_t n_entries, int64_t n_trials);

@@ -211,19 +211,42 @@ __device__ __forceinline__ void extend_profile(unsigned char* smem, int p0, int 
     }
 }
 
+// Sum of two float-float pairs, as a canonical pair.
+__device__ __forceinline__ void ff_add(float& ah, float& al, float bh, float bl) {
+    float s, e;
+    two_sum(ah, bh, s, e);
+    e = __fadd_rn(e, __fadd_rn(al, bl));
+    ah = __fadd_rn(s, e);
+    al = __fsub_rn(e, __fsub_rn(ah, s));
+}
+// Inclusive scan over the lanes [0, n) of a warp (n <= 32).
+__device__ __forceinline__ void ff_warp_scan(float& h, float& l, int n) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        if (o >= n) break;
+        const float uh = __shfl_up_sync(0xffffffffu, h, o), ul = __shfl_up_sync(0xffffffffu, l, o);
+        if (lane >= o) ff_add(h, l, uh, ul);
+    }
+}
+
+constexpr int SCORE_MAXSEG = 64;  // segments of 32 blocks of the longest profile with its extension
+
 // Block offsets: the exclusive scan of the block totals that offs holds (a
-// float2's x), in segments of 128 blocks, four per lane -- the same tree
-// whatever the CTA's size.  Ends with a barrier.
+// float2's x).  Float sums have one tree whatever the CTA's size: a scan over
+// 32 blocks, a scan over the segments' totals within `group` blocks (1024 /
+// 512 / 256 by profile length), and the groups one after another.  Ends with
+// a barrier.
 template <class V, bool ONE>
-__device__ __forceinline__ void scan_offsets(typename Offset<V>::type* offs, float2* seg, int nbx) {
+__device__ __forceinline__ void scan_offsets(typename Offset<V>::type* offs, float2* seg, int nbx, int group) {
     constexpr bool INT = !std::is_same<V, float>::value;
     const int lane = threadIdx.x & 31, warp = ONE ? 0 : threadIdx.x >> 5, NW = ONE ? 1 : blockDim.x >> 5;
-    const int nseg = (nbx + 127) >> 7;
-    float ch = 0.0f, cl = 0.0f;  // ONE: carry
-    uint32_t ci = 0;
-    for (int sgm = warp; sgm < nseg; sgm += NW) {
-        const int b0 = (sgm << 7) + 4 * lane;
-        if constexpr (INT) {
+    if constexpr (INT) {
+        // wrapping sums have no order: 128 blocks a segment, four per lane
+        const int nseg = (nbx + 127) >> 7;
+        uint32_t ci = 0;  // ONE: carry
+        for (int sgm = warp; sgm < nseg; sgm += NW) {
+            const int b0 = (sgm << 7) + 4 * lane;
             uint32_t v[4], s = 0;
 #pragma unroll
             for (int i = 0; i < 4; ++i) v[i] = b0 + i < nbx ? (uint32_t)offs[b0 + i] : 0u;
@@ -246,70 +269,62 @@ __device__ __forceinline__ void scan_offsets(typename Offset<V>::type* offs, flo
             const uint32_t tot = __shfl_sync(0xffffffffu, x, 31);
             if (ONE) ci += tot;
             else if (lane == 0) seg[sgm].x = __uint_as_float(tot);
-        } else {
-            float v[4], h[4], l[4], sh_ = 0.0f, sl = 0.0f;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v[i] = b0 + i < nbx ? offs[b0 + i].x : 0.0f;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                h[i] = sh_;
-                l[i] = sl;
-                ff_acc(sh_, sl, v[i], 0.0f);
-            }
-            float xh = sh_, xl = sl;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const float uh = __shfl_up_sync(0xffffffffu, xh, o);
-                const float ul = __shfl_up_sync(0xffffffffu, xl, o);
-                if (lane >= o) ff_acc(xh, xl, uh, ul);
-            }
-            ff_norm(xh, xl);
-            float eh = __shfl_up_sync(0xffffffffu, xh, 1), el = __shfl_up_sync(0xffffffffu, xl, 1);
-            if (lane == 0) eh = el = 0.0f;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                ff_acc(h[i], l[i], eh, el);
-                ff_norm(h[i], l[i]);
-                if (ONE) {
-                    ff_acc(h[i], l[i], ch, cl);
-                    ff_norm(h[i], l[i]);
-                }
-                if (b0 + i < nbx) offs[b0 + i] = make_float2(h[i], l[i]);
-            }
-            const float th = __shfl_sync(0xffffffffu, xh, 31), tl = __shfl_sync(0xffffffffu, xl, 31);
-            if (ONE) {
-                ff_acc(ch, cl, th, tl);
-                ff_norm(ch, cl);
-            } else if (lane == 0) {
-                seg[sgm] = make_float2(th, tl);
-            }
         }
-    }
-    cta_sync<ONE>();
-    if (!ONE && nseg > 1) {
-        // add the earlier segments' totals
-        for (int sgm = warp ? warp : NW; sgm < nseg; sgm += NW) {
-            if constexpr (INT) {
+        cta_sync<ONE>();
+        if (!ONE && nseg > 1) {
+            for (int sgm = warp ? warp : NW; sgm < nseg; sgm += NW) {
                 uint32_t base = 0;
                 for (int i = 0; i < sgm; ++i) base += __float_as_uint(seg[i].x);
                 for (int b = (sgm << 7) + lane; b < nbx && b < (sgm + 1) << 7; b += 32)
                     offs[b] = (int)((uint32_t)offs[b] + base);
-            } else {
-                float bh = 0.0f, bl = 0.0f;
-                for (int i = 0; i < sgm; ++i) {
-                    const float2 t = seg[i];
-                    ff_acc(bh, bl, t.x, t.y);
-                    ff_norm(bh, bl);
-                }
-                for (int b = (sgm << 7) + lane; b < nbx && b < (sgm + 1) << 7; b += 32) {
-                    float2 o = offs[b];
-                    ff_acc(o.x, o.y, bh, bl);
-                    ff_norm(o.x, o.y);
-                    offs[b] = o;
+            }
+            __syncthreads();
+        }
+    } else {
+        const int nseg = (nbx + 31) >> 5, per = group >> 5;  // segments, segments a group
+        for (int sgm = warp; sgm < nseg; sgm += NW) {
+            const int b = (sgm << 5) + lane;
+            float h = b < nbx ? offs[b].x : 0.0f, l = 0.0f;
+            ff_warp_scan(h, l, 32);
+            if (lane == 31) seg[sgm] = make_float2(h, l);
+            float ph = __shfl_up_sync(0xffffffffu, h, 1), pl = __shfl_up_sync(0xffffffffu, l, 1);
+            if (lane == 0) ph = pl = 0.0f;
+            if (b < nbx) offs[b] = make_float2(ph, pl);
+        }
+        cta_sync<ONE>();
+        if (nseg == 1) return;
+        float th = 0.0f, tl = 0.0f;  // total of the group before
+        for (int g0 = 0; g0 < nseg; g0 += per) {
+            const int ng = nseg - g0 < per ? nseg - g0 : per;
+            float h = 0.0f, l = 0.0f;
+            if (lane < ng) {
+                const float2 t = seg[g0 + lane];
+                h = t.x;
+                l = t.y;
+            }
+            ff_warp_scan(h, l, ng);
+            // segments of this group dealt out as above
+            const int first = g0 + (warp + NW - g0 % NW) % NW;
+            for (int sgm = first; sgm < g0 + ng; sgm += NW) {
+                float bh = __shfl_sync(0xffffffffu, h, sgm - g0 - 1), bl = __shfl_sync(0xffffffffu, l, sgm - g0 - 1);
+                if (sgm == g0) bh = bl = 0.0f;
+                const int b = (sgm << 5) + lane;
+                if (b < nbx) {
+                    const float2 p = offs[b];
+                    ff_add(bh, bl, p.x, p.y);
+                    if (g0) {
+                        float rh = th, rl = tl;
+                        ff_add(rh, rl, bh, bl);
+                        bh = rh;
+                        bl = rl;
+                    }
+                    offs[b] = make_float2(bh, bl);
                 }
             }
+            th = __shfl_sync(0xffffffffu, h, ng - 1);  // one extension group at most follows
+            tl = __shfl_sync(0xffffffffu, l, ng - 1);
         }
-        __syncthreads();
+        cta_sync<ONE>();
     }
 }
 

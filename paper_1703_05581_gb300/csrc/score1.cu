@@ -59,24 +59,23 @@ struct IsInt {
 struct ScoreLay {
     uint32_t offs, list, aux;
     int32_t cap;
+    int32_t group;  // blocks of one group of the offset scan
 };
 
 constexpr int score_pack(int r) { return r == 8 ? 256 : 768; }  // members a float window may have
 constexpr int score_nb(int r) { return r == 8 ? 256 : 512; }    // buckets of an int window
-constexpr int S1_NC = 64;                                       // near-ties of one pick
-constexpr int S1_MAXSEG = 16;
 
 struct S1Sh {
-    unsigned long long cand[S1_NC], key[2];
+    unsigned long long key[2];
     float fa[32], fb[32], fc[32];
     uint2 wc[2][32];          // per-warp counts of a window pass (two slots, alternating)
-    float2 seg[S1_MAXSEG];    // segment totals of the offset scan
+    float2 seg[SCORE_MAXSEG]; // segment totals of the offset scan
     uint32_t wkey[16];        // per-width maxima as order-preserving keys
-    uint32_t npack, ncand;
+    uint32_t npack;
     int bin_a, bin_b;
     uint32_t below_a;
     int ok;
-    uint32_t pos;
+    uint32_t pos, tail;  // first argmax: in the whole blocks, in the one that runs past p0
     float best;
     int bw;
 };
@@ -174,19 +173,18 @@ __device__ __noinline__ unsigned long long radix_rank(const unsigned char* smem,
 // One warp: the values of ranks t1 <= t2 <= t1 + 1 among the n members of a
 // window at `pack` (padded to a multiple of 128 with +inf), all between lo
 // and hi.  MAD: of |x - mh|.  Counting passes at interpolated pivots; each
-// pass also yields the pivot's neighbours on both sides.
+// pass also yields the pivot's neighbours on both sides, and the interval
+// closes in on members, so that clusters of nearly equal values (folds of
+// quantised series) cost no more passes.
 template <bool MAD>
 __device__ __forceinline__ bool pick2(const float* pack, uint32_t n, uint32_t t1, uint32_t t2, float lo, float hi,
                                       float mh, float& va, float& vb) {
     const int lane = threadIdx.x & 31;
-    uint32_t cl = 0, ch = n;  // members <= lo, <= hi
-    bool exact = false;       // the pivot is the next member above lo
-    float next = 0.0f;
-    for (int a = 0; a < 24; ++a) {
-        float p;
-        if (exact) {
-            p = next;
-        } else {
+    uint32_t cl = 0, ch = n;  // members < lo, <= hi
+    bool step = false;        // next pivot: the first member from lo on
+    for (int a = 0; a < 32; ++a) {
+        float p = lo;
+        if (!step) {
             p = fmaf(__fdividef((float)(2 * (t1 - cl) + 1), (float)(2 * (ch - cl))), hi - lo, lo);
             if (!(p < hi)) p = lo;
         }
@@ -212,23 +210,82 @@ __device__ __forceinline__ bool pick2(const float* pack, uint32_t n, uint32_t t1
                 va = vb = above;
                 return true;
             }
-            // near the rank, or nothing between the pivot and hi: step to the
-            // next member
-            exact = t1 - c <= 1 || above >= hi || p <= lo;
-            lo = p;
+            lo = above;
             cl = c;
-            next = above;
+            step = t1 - c <= 1;
         } else {
-            if (exact || c == t1 + 1) {
+            // fewer than t1 + 1 members are below lo
+            if (p == lo || c == t1 + 1) {
                 va = upto;
                 vb = c > t2 ? upto : above;
                 return true;
             }
             hi = upto;
             ch = c;
+            step = false;
         }
     }
     return false;
+}
+
+// One warp: the exact deviations |x - (mh + ml)| of ranks t1 <= t2 among the
+// m values at `pack` (near-ties of the FP32 deviation), as keys.  Up to 32 by
+// comparison in registers, more by a quickselect.
+__device__ __forceinline__ void rank_deviations(const float* pack, uint32_t m, uint32_t t1, uint32_t t2, float mh,
+                                                float ml, unsigned long long& ka, unsigned long long& kb) {
+    const int lane = threadIdx.x & 31;
+    auto key_of = [&](float x) {
+        float h, l;
+        ff_dev(x, mh, ml, h, l);
+        return ff_key(h, l);
+    };
+    if (m <= 32) {
+        const unsigned long long ki = lane < m ? key_of(pack[lane]) : ~0ull;
+        uint32_t rk = 0;
+        for (uint32_t j = 0; j < m; ++j) {
+            const unsigned long long kj = __shfl_sync(0xffffffffu, ki, j);
+            rk += (kj < ki) || (kj == ki && j < (uint32_t)lane);
+        }
+        ka = __shfl_sync(0xffffffffu, ki, __ffs(__ballot_sync(0xffffffffu, lane < m && rk == t1)) - 1);
+        kb = __shfl_sync(0xffffffffu, ki, __ffs(__ballot_sync(0xffffffffu, lane < m && rk == t2)) - 1);
+        return;
+    }
+    for (int want = 0; want < 2; ++want) {
+        const uint32_t t = want ? t2 : t1;
+        unsigned long long klo = 0, khi = ~0ull, kp = 0;  // the wanted key is in [klo, khi]
+        uint32_t at = 0;
+        for (uint32_t a = 0; a <= m; ++a) {
+            // the next member in the interval is the pivot
+            for (uint32_t scan = 0; scan <= m; scan += 32) {
+                const uint32_t i = at + lane < m ? at + lane : at + lane - m;
+                const unsigned long long k = i < m ? key_of(pack[i]) : 0ull;
+                const unsigned in = __ballot_sync(0xffffffffu, i < m && k >= klo && k <= khi);
+                if (in) {
+                    const int src = __ffs(in) - 1;
+                    kp = __shfl_sync(0xffffffffu, k, src);
+                    at = (at + src + 1) % m;
+                    break;
+                }
+                at = (at + 32) % m;
+            }
+            uint32_t less = 0, upto = 0;
+            for (uint32_t i = lane; i < m; i += 32) {
+                const unsigned long long k = key_of(pack[i]);
+                less += k < kp;
+                upto += k <= kp;
+            }
+            less = __reduce_add_sync(0xffffffffu, less);
+            upto = __reduce_add_sync(0xffffffffu, upto);
+            if (t < less) khi = kp - 1;
+            else if (t >= upto) klo = kp + 1;
+            else break;
+        }
+        (want ? kb : ka) = kp;
+        if (t1 == t2) {
+            kb = kp;
+            break;
+        }
+    }
 }
 
 // R: bins per block.  ONE: the CTA is one warp.
@@ -335,9 +392,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
         if (INT)
             for (int b = 4 * tid; b < NB; b += 4 * T) *reinterpret_cast<int4*>(hist + b) = make_int4(0, 0, 0, 0);
         if (tid < 16) sh.wkey[tid] = 0u;
-        if (tid == 16) sh.pos = 0x7fffffffu;
+        if (tid == 16) sh.pos = sh.tail = 0x7fffffffu;
         if (tid == 17) sh.npack = 0;
-        if (tid == 18) sh.ncand = 0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             fs += __shfl_xor_sync(0xffffffffu, fs, o);
@@ -449,39 +505,32 @@ __global__ void __launch_bounds__(MAXT, MINB)
                             // within 2 E of va, vb; rank those exactly
                             const float E = (hi + fabsf(mh)) * 1.2e-7f;
                             const float ca = va - 3.0f * E, cb = vb + 3.0f * E;
-                            uint32_t less = 0;
-                            for (uint32_t i = lane; i < n; i += 32) {
-                                const float v = pack[i], d = fabsf(__fsub_rn(v, mh));
+                            // (packed in place, every read before the writes it meets)
+                            uint32_t less = 0, m = 0;
+                            for (uint32_t i0 = 0; i0 < n; i0 += 32) {
+                                const uint32_t i = i0 + lane;
+                                const float v = i < n ? pack[i] : INFINITY, d = fabsf(__fsub_rn(v, mh));
                                 less += d < ca;
-                                if (d >= ca && d <= cb) {
-                                    const uint32_t s = atomicAdd(&sh.ncand, 1u);
-                                    float h, l;
-                                    ff_dev(v, mh, ml, h, l);
-                                    if (s < S1_NC) sh.cand[s] = ff_key(h, l);
-                                }
+                                const unsigned near = __ballot_sync(0xffffffffu, d >= ca && d <= cb);
+                                if (d >= ca && d <= cb) pack[m + __popc(near & ((1u << lane) - 1))] = v;
+                                m += __popc(near);
+                                __syncwarp();
                             }
                             less = __reduce_add_sync(0xffffffffu, less);
-                            __syncwarp();
-                            const uint32_t m = sh.ncand;
-                            if (m > S1_NC || ca < lo || cb > hi) {  // too many, or too near the window's edge
+                            if (ca < lo || cb > hi) {  // too near the window's edge
                                 ok = 0;
                             } else {
-                                for (uint32_t i = lane; i < m; i += 32) {
-                                    const unsigned long long ki = sh.cand[i];
-                                    uint32_t rk = 0;
-                                    for (uint32_t j = 0; j < m; ++j) {
-                                        const unsigned long long kj = sh.cand[j];
-                                        rk += (kj < ki) || (kj == ki && j < i);
-                                    }
-                                    if (rk == t1 - less) sh.key[0] = ki;
-                                    if (rk == t2 - less) sh.key[1] = ki;
+                                unsigned long long k1, k2;
+                                rank_deviations(pack, m, t1 - less, t2 - less, mh, ml, k1, k2);
+                                if (lane == 0) {
+                                    sh.key[0] = k1;
+                                    sh.key[1] = k2;
                                 }
                             }
                         }
                         if (lane == 0) {
                             sh.ok = ok;
                             sh.npack = 0;
-                            sh.ncand = 0;
                         }
                     } else if (!ONE) {  // meanwhile
                         if (MAD) prefix(tid - 32, T - 32);
@@ -635,7 +684,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
             prefix(tid, T);
             sync();
         }
-        scan_offsets<V, ONE>(offs, sh.seg, nbx);
+        scan_offsets<V, ONE>(offs, sh.seg, nbx, lay.group);
 
         // ---- widths: the largest box of each, per thread ----
         V M[NS];
@@ -733,12 +782,16 @@ __global__ void __launch_bounds__(MAXT, MINB)
                 for (int i0 = 0; i0 < nk; i0 += 32 / P) {
                     const int im = src + (i0 + lane / P) * T;
                     uint32_t f = 0x7fffffffu;
+                    bool tail = false;
                     if (im < nitem) {
                         const int j = (im / PARTS) * R + (im % PARTS) * P + lane % P;
-                        if (box_at<V, R>(smem, offs, j, w) == target) f = (uint32_t)(j < p0 ? j : j % p0);
+                        tail = (im / PARTS + 1) * R > p0;
+                        if (box_at<V, R>(smem, offs, j, w) == target) f = (uint32_t)j;
                     }
-                    f = __reduce_min_sync(0xffffffffu, f);
-                    if (lane == 0 && f != 0x7fffffffu) atomicMin(&sh.pos, f);
+                    const uint32_t f1 = __reduce_min_sync(0xffffffffu, tail ? 0x7fffffffu : f);
+                    const uint32_t f2 = __reduce_min_sync(0xffffffffu, tail ? f : 0x7fffffffu);
+                    if (lane == 0 && f1 != 0x7fffffffu) atomicMin(&sh.pos, f1);
+                    if (lane == 0 && f2 != 0x7fffffffu) atomicMin(&sh.tail, f2);
                 }
             }
         }
@@ -751,7 +804,10 @@ __global__ void __launch_bounds__(MAXT, MINB)
                 out.phase = 0;
                 out.flags = 1;
             } else {
-                const uint32_t pos = sh.pos;
+                // the last block's first match counts at its cyclic position
+                uint32_t pos = sh.tail;
+                if (pos != 0x7fffffffu && pos >= (uint32_t)p0) pos %= (uint32_t)p0;
+                pos = min(pos, sh.pos);
                 out.snr = sh.best;
                 out.width = 1 << bw;
                 out.phase = pos == 0x7fffffffu ? 0 : (int32_t)pos;
@@ -825,11 +881,13 @@ ffa_status score1_t(const void* d_prof, const ScoreGroup& sg, int64_t count, int
 #define FFA_SCORE1(RR, ONE, MAXT, MINB)                                                                          \
     score1_launch<V, RR, ONE, FF, MAXT, MINB>(d_prof, sg, count, trial0, m_rows, wmask, wtop, threads, lay, smem, \
                                               d_status, st)
+    const int shape = score_shape(p0, wd.w[wd.n - 1]);
+    lay.group = score_scan_group(shape);
     // CTA shapes, measured with ready profiles of 366..30000 bins: threads
     // against registers.  Fewer threads that hold their item in registers
     // beat more threads that spill (20000 bins: 27.7k SM cycles a profile
     // with 448 threads of 72 registers, 35.7k with 640 of 48).
-    switch (score_shape(p0, wd.w[wd.n - 1])) {
+    switch (shape) {
         case 0:
             // one warp a profile up to 1200 bins (1100 bins: 2.1k SM cycles,
             // 2.7k with two warps; 366 bins: 1.2k and 2.2k), two above
@@ -868,6 +926,8 @@ ffa_status score1_dispatch(const void* d_prof, const ScoreGroup& sg, int32_t pre
 }
 
 }  // namespace
+
+int score_scan_group(int shape) { return shape == 0 ? 256 : (shape == 1 ? 512 : 1024); }
 
 // The scorers' block length by profile length: 0: 8 bins (up to 2048), 1: 16
 // (up to 8192), 2: 16, 3: 32, -1: too long; the extension by the widest box

@@ -35,7 +35,7 @@ struct S2Sh {
     float part[3][32];        // per chunk: sum, sum and sum of squares about the mean
     float2 win[16][32];       // per width and chunk: the window's sums
     float2 wtot[16];
-    float2 seg[16];           // segment totals of the offset scan
+    float2 seg[SCORE_MAXSEG]; // segment totals of the offset scan
     uint32_t wkey[16];        // largest box of width 2^n, as an order-preserving key of its float
     uint32_t pos[16];         // its first bin
 };
@@ -49,7 +49,8 @@ __device__ __forceinline__ float warp_sum(float v) {
 template <class V, int R, bool FUSED, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
     k_score_alg2(const V* __restrict__ prof_all, const ScoreGroup sg, int64_t m_rows, int64_t trial0, int64_t count,
-                 const ScoreWidths wd, uint32_t wmask, float excl_frac, uint32_t lay_offs, uint32_t lay_tots) {
+                 const ScoreWidths wd, uint32_t wmask, float excl_frac, uint32_t lay_offs, uint32_t lay_tots,
+                 int group) {
     constexpr int PARTS = R < 16 ? 1 : R / 16;
     constexpr int NS = R == 8 ? 12 : 16;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -147,7 +148,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
             }
         }
         __syncthreads();
-        scan_offsets<V, false>(offs, sh.seg, nbx);
+        scan_offsets<V, false>(offs, sh.seg, nbx, group);
 
         // ---- every width's largest box that starts in the profile (the
         // whole blocks' by items, the last block's bins one by one)
@@ -334,7 +335,8 @@ ffa_status alg2_launch(const void* d_prof, const ScoreGroup& sg, int64_t count, 
     if (es != FFA_OK) return es;
     const unsigned grid = (unsigned)(count < resident ? count : resident);
     k_score_alg2<V, R, FF, MAXT, MINB><<<grid, threads, smem, st>>>((const V*)d_prof, sg, m_rows, trial0, count, wd, wmask,
-                                                                    excl_frac, (uint32_t)offs, (uint32_t)tots);
+                                                                    excl_frac, (uint32_t)offs, (uint32_t)tots,
+                                                                    score_scan_group(score_shape(p0, wmax)));
     FFA_LAUNCH_CHECK("k_score_alg2");
     count_launch();
     return FFA_OK;

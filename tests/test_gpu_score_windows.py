@@ -10,7 +10,7 @@ from parity import check_records
 pytestmark = pytest.mark.gpu
 
 SIZES = [3, 8, 33, 1200, 1201, 2048, 2049, 8193, 16385, 20479, 20481, 31249]
-KINDS = ["normal", "levels", "humps", "skewed", "wave", "offset", "ramp"]
+KINDS = ["normal", "levels", "codes", "humps", "skewed", "wave", "offset", "ramp"]
 
 
 @pytest.fixture(scope="module")
@@ -30,6 +30,8 @@ def _profile(rng, p0, kind):
     x = rng.standard_normal(p0)
     if kind == "levels":     # few distinct values: long runs of ties
         x = np.rint(2.0 * x)
+    elif kind == "codes":    # a quantised series' sums: clusters of tens of equal values
+        x = np.rint(50.0 * x) / 3.0
     elif kind == "humps":    # no samples near the mean
         x = np.where(rng.random(p0) < 0.3, 20.0, 0.0) + 0.1 * x
     elif kind == "skewed":
