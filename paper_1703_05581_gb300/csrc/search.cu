@@ -303,8 +303,11 @@ struct PhaseTimer {
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// grouping of small base periods (see group_end)
-constexpr int64_t GROUP_TRIALS = 1024;
+// Grouping of base periods (see group_end): elements of a group's plane.  Two
+// planes of 64 MB stay in L2 between the fold's passes and the scorer, and a
+// launch holds enough trials to fill the GPU: an 8-bit beam at D0 = 64 (2^20
+// samples, 920 base periods of about 1.5 M elements) takes 31.8 ms with
+// single base periods, 18.1 / 15.6 / 14.6 ms with groups of 2^22 / 2^23 / 2^24.
 constexpr int64_t GROUP_ELEMS = (int64_t)1 << 24;
 // elements a base period's plane takes in a group (256-byte aligned)
 static size_t plane_slot(const ffa_plan_entry& e) {
@@ -449,13 +452,12 @@ ffa_status ffa_plan_create(const ffa_search_config* cfg, int64_t n, ffa_plan** o
     off = align256(off + (cfg->precision == FFA_FOLD_F32 ? 4 : 1) * (size_t)n0);
     p->off_stats = off;
     off = align256(off + sizeof(double) * STATS_DOUBLES);
-    // planes: the largest base period, or a group of small ones (GROUP_ELEMS)
+    // planes: the largest base period, or a group of small ones
     p->plane_elems = std::max<int64_t>(p->max_plane, 1);
-    for (const ffa_plan_entry& e : p->entries)
-        if (e.m_rows < GROUP_TRIALS) {
-            const int64_t want = (GROUP_TRIALS / e.m_rows) * (int64_t)plane_slot(e);
-            p->plane_elems = std::max<int64_t>(p->plane_elems, std::min<int64_t>(want, GROUP_ELEMS));
-        }
+    for (const ffa_plan_entry& e : p->entries) {
+        const int64_t want = (int64_t)FOLD_GROUP_MAX * (int64_t)plane_slot(e);
+        p->plane_elems = std::max<int64_t>(p->plane_elems, std::min<int64_t>(want, GROUP_ELEMS));
+    }
     p->off_plane0 = off;
     off = align256(off + 4 * (size_t)p->plane_elems);
     p->off_plane1 = off;
@@ -520,18 +522,17 @@ ffa_status ffa_plan_periods(const ffa_plan* p, int64_t trial_begin, int64_t coun
 // folded and scored.
 // Consecutive base periods folded and scored by one set of launches: same
 // octave, rows, widths and floor(log2 p0) (so the same tuned pass depth and
-// CTA shape), together fewer than GROUP_TRIALS trials and within the plane
-// buffers.  Base periods of GROUP_TRIALS rows or more go alone.
+// CTA shape), together at most FOLD_GROUP_MAX base periods and GROUP_ELEMS
+// plane elements.  A larger base period goes alone.
 
 static int64_t group_end(const ffa_plan* p, int64_t t, int64_t b) {
     const ffa_plan_entry& e0 = p->entries[(size_t)t];
-    if (e0.m_rows >= GROUP_TRIALS) return t + 1;
     auto lg = [](int64_t v) {
         int r = 0;
         while ((int64_t)2 << r <= v) ++r;
         return r;
     };
-    int64_t j = t, trials = 0;
+    int64_t j = t;
     size_t elems = 0;
     while (j < b && j - t < FOLD_GROUP_MAX) {
         const ffa_plan_entry& e = p->entries[(size_t)j];
@@ -539,9 +540,8 @@ static int64_t group_end(const ffa_plan* p, int64_t t, int64_t b) {
             std::memcmp(e.widths, e0.widths, sizeof(int32_t) * (size_t)e0.n_widths) != 0 ||
             score_shape(e.p0, e.widths[e.n_widths - 1]) != score_shape(e0.p0, e0.widths[e0.n_widths - 1]))
             break;
-        if (elems + plane_slot(e) > (size_t)p->plane_elems || trials + e.m_rows > GROUP_TRIALS) break;
+        if (elems + plane_slot(e) > (size_t)GROUP_ELEMS) break;
         elems += plane_slot(e);
-        trials += e.m_rows;
         ++j;
     }
     return j > t ? j : t + 1;
@@ -826,7 +826,9 @@ ffa_status ffa_search_plane(const ffa_plan* p, const void* d_series, int64_t ent
 // so the records are those of each series searched alone.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr int64_t BATCH_GROUP_ELEMS = (int64_t)1 << 25;  // per plane buffer (32-bit elements)
+// Per plane buffer (32-bit elements).  12 DM trials of 2^19-2^20 samples: 542,
+// 381, 327, 299, 295 ms with 2^21 .. 2^25.
+constexpr int64_t BATCH_GROUP_ELEMS = (int64_t)1 << 25;
 
 struct BatchLayout {
     std::vector<size_t> raw_off, z_off;
@@ -864,7 +866,7 @@ ffa_status batch_layout(const ffa_plan* const* plans, int32_t count, BatchLayout
     off = align256(off + sizeof(double) * (size_t)max_n0);
     L->off_stats = off;
     off = align256(off + sizeof(double) * STATS_DOUBLES);
-    L->plane_elems = std::max<int64_t>(max_slot, std::min<int64_t>(BATCH_GROUP_ELEMS, (int64_t)count * max_slot));
+    L->plane_elems = std::max<int64_t>(max_slot, std::min<int64_t>(BATCH_GROUP_ELEMS, (int64_t)FOLD_GROUP_MAX * max_slot));
     L->off_plane0 = off;
     off = align256(off + 4 * (size_t)L->plane_elems);
     L->off_plane1 = off;
