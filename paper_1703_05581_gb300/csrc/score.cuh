@@ -100,8 +100,7 @@ __device__ __forceinline__ uint32_t blk_addr(uint32_t b) {  // byte address of b
 // quad s of the block at address a is at a ^ (s << 4)
 template <int R>
 __device__ __forceinline__ uint32_t bin_addr(uint32_t j) {  // byte address of bin j
-    constexpr uint32_t QB = R / 4;
-    return (((j << 2) & ~15u) ^ (((j >> 5) & (QB - 1)) << 4)) | ((j & 3) << 2);
+    return (j << 2) ^ ((j >> 1) & ((R / 4 - 1) << 4));
 }
 
 // The block offsets' element: float-float (a float2) or wrapping int32.
@@ -142,72 +141,116 @@ __device__ __forceinline__ V load_bin(const unsigned char* smem, uint32_t j) {
 }
 
 // Load a profile into shared memory: hrow's p0 bins, plus (two) trow's read
-// sft bins further on, four bins at a time; acc(v) sees every bin once.
+// sft bins further on, four bins at a time; acc(v) sees every bin once (and
+// the quad that straddles the wrap a second time, with other tail bins: it
+// only takes statistics that guide a search).  Four quads' loads are issued
+// before any is used, without a branch between them -- one quad in flight per
+// thread took 8.9k of 29.7k SM cycles per profile of 19977 bins.
 template <class V, int R, class Acc>
 __device__ __forceinline__ void load_profile(unsigned char* smem, const V* __restrict__ hrow, const V* __restrict__ trow,
                                              int sft, bool two, int p0, int tid, int T, Acc acc) {
+    constexpr int U = 4;
     auto store_quad = [&](int q, const V (&v)[4]) {
         *reinterpret_cast<int4*>(smem + (((uint32_t)q ^ (((uint32_t)q >> 3) & (R / 4 - 1))) << 4)) =
             *reinterpret_cast<const int4*>(v);
     };
-    const bool al = (reinterpret_cast<uintptr_t>(hrow) & 15) == 0;
     const int nq4 = p0 >> 2;
-    auto load_head = [&](int q, V (&h)[4]) {
-        if (al) {
-            *reinterpret_cast<int4*>(h) = *reinterpret_cast<const int4*>(hrow + 4 * q);
-        } else {
+    auto tail_at = [&](int j) { return trow[j + sft < p0 ? j + sft : j + sft - p0]; };
+    // AL: hrow is 16-byte aligned.  q < nq4; the tail's quad is read from the
+    // last position that lies inside the row if it wraps.
+    auto load_quads = [&](auto al, auto tw, int q0, int n) {
+        constexpr bool AL = decltype(al)::value, TW = decltype(tw)::value;
+        V h[U][4], t[U][4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) h[i] = hrow[4 * q + i];
-        }
-    };
-    if (two) {
-#pragma unroll 4
-        for (int q = tid; q < nq4; q += T) {
-            V h[4], t[4];
-            load_head(q, h);
-            int o = 4 * q + sft;
-            if (o >= p0) o -= p0;
-            if (o + 3 < p0) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) t[i] = trow[o + i];
+        for (int u = 0; u < U; ++u) {
+            if (u >= n) break;
+            const int q = q0 + u * T;
+            if (AL) {
+                *reinterpret_cast<int4*>(h[u]) = *reinterpret_cast<const int4*>(hrow + 4 * q);
             } else {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) t[i] = trow[o + i < p0 ? o + i : o + i - p0];
+                for (int i = 0; i < 4; ++i) h[u][i] = hrow[4 * q + i];
             }
+            if (TW) {
+                int o = 4 * q + sft;
+                o = o >= p0 ? o - p0 : o;
+                o = min(o, p0 - 4);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) t[u][i] = trow[o + i];
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (u >= n) break;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                h[i] = h[i] + t[i];
-                acc(h[i]);
+                if (TW) h[u][i] = h[u][i] + t[u][i];
+                acc(h[u][i]);
             }
-            store_quad(q, h);
+            store_quad(q0 + u * T, h[u]);
+        }
+    };
+    auto load_all = [&](auto al, auto tw) {
+        int q = tid;
+        for (; q + (U - 1) * T < nq4; q += U * T) load_quads(al, tw, q, U);
+        for (; q < nq4; q += T) load_quads(al, tw, q, 1);
+    };
+    const bool al = (reinterpret_cast<uintptr_t>(hrow) & 15) == 0;
+    if (two) {
+        if (al) load_all(std::true_type{}, std::true_type{});
+        else load_all(std::false_type{}, std::true_type{});
+        // the quad whose tail wraps, by the thread that stored it
+        const int qw = (p0 - sft) >> 2;
+        if (sft != 0 && ((p0 - sft) & 3) && qw < nq4 && tid == qw % T) {
+            V v[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                v[i] = hrow[4 * qw + i] + tail_at(4 * qw + i);
+                acc(v[i]);
+            }
+            store_quad(qw, v);
         }
     } else {
-#pragma unroll 4
-        for (int q = tid; q < nq4; q += T) {
-            V h[4];
-            load_head(q, h);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) acc(h[i]);
-            store_quad(q, h);
-        }
+        if (al) load_all(std::true_type{}, std::false_type{});
+        else load_all(std::false_type{}, std::false_type{});
     }
     if (tid < (p0 & 3)) {
         const int j = 4 * nq4 + tid;
         V v = hrow[j];
-        if (two) v = v + trow[j + sft < p0 ? j + sft : j + sft - p0];
+        if (two) v = v + tail_at(j);
         *reinterpret_cast<V*>(smem + bin_addr<R>(j)) = v;
         acc(v);
     }
 }
 
-// Cyclic extension: bins p0 .. nbx * R - 1 repeat the profile.
+// Cyclic extension: bins p0 .. nbx * R - 1 repeat the profile.  A quad of the
+// extension is four consecutive bins of the profile from a start of one
+// residue mod 4: two quads read, one written.
 template <class V, int R>
 __device__ __forceinline__ void extend_profile(unsigned char* smem, int p0, int nbx, int first, int step) {
     const int ext = nbx * R - p0;
-    for (int j = first; j < ext; j += step) {
-        int s = j;
-        while (s >= p0) s -= p0;  // at most once for profiles longer than the extension
-        *reinterpret_cast<V*>(smem + bin_addr<R>(p0 + j)) = load_bin<V, R>(smem, s);
+    if (ext > p0 - 4) {  // wraps again (short profiles): bin by bin
+        for (int j = first; j < ext; j += step) {
+            int s = j;
+            while (s >= p0) s -= p0;
+            *reinterpret_cast<V*>(smem + bin_addr<R>(p0 + j)) = load_bin<V, R>(smem, s);
+        }
+        return;
+    }
+    const int lead = (4 - (p0 & 3)) & 3;  // bins up to the first whole quad
+    if (first < lead) *reinterpret_cast<V*>(smem + bin_addr<R>(p0 + first)) = load_bin<V, R>(smem, first);
+    auto quad_addr = [](uint32_t q) { return (q ^ ((q >> 3) & (R / 4 - 1))) << 4; };
+    const int q0 = (p0 + lead) >> 2, nq = (ext - lead) >> 2;  // nbx * R is a multiple of 4
+    const bool b0 = lead & 1, b1 = lead & 2;
+    for (int q = first; q < nq; q += step) {
+        V r[8], t[6], v[4];
+        load_quad(smem, quad_addr((uint32_t)q), *reinterpret_cast<V(*)[4]>(&r[0]));
+        load_quad(smem, quad_addr((uint32_t)q + 1), *reinterpret_cast<V(*)[4]>(&r[4]));
+#pragma unroll
+        for (int i = 0; i < 6; ++i) t[i] = b0 ? r[i + 1] : r[i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = b1 ? t[i + 2] : t[i];
+        *reinterpret_cast<int4*>(smem + quad_addr((uint32_t)(q0 + q))) = *reinterpret_cast<const int4*>(v);
     }
 }
 
@@ -219,6 +262,30 @@ __device__ __forceinline__ void ff_add(float& ah, float& al, float bh, float bl)
     ah = __fadd_rn(s, e);
     al = __fsub_rn(e, __fsub_rn(ah, s));
 }
+// The same on two pairs at once, in packed FP32 instructions.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tadd.rn.f32x2 z, x, y;\n\t"
+        "mov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    float2 r;
+    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tsub.rn.f32x2 z, x, y;\n\t"
+        "mov.b64 {%0, %1}, z;\n\t}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ void ff_add2(float2& ah, float2& al, float2 bh, float2 bl) {
+    const float2 s = add2(ah, bh), bb = sub2(s, ah);
+    float2 e = add2(sub2(ah, sub2(s, bb)), sub2(bh, bb));
+    e = add2(e, add2(al, bl));
+    ah = add2(s, e);
+    al = sub2(e, sub2(ah, s));
+}
 // Inclusive scan over the lanes [0, n) of a warp (n <= 32).
 __device__ __forceinline__ void ff_warp_scan(float& h, float& l, int n) {
     const int lane = threadIdx.x & 31;
@@ -227,6 +294,21 @@ __device__ __forceinline__ void ff_warp_scan(float& h, float& l, int n) {
         if (o >= n) break;
         const float uh = __shfl_up_sync(0xffffffffu, h, o), ul = __shfl_up_sync(0xffffffffu, l, o);
         if (lane >= o) ff_add(h, l, uh, ul);
+    }
+}
+// Two scans over 32 lanes at once (h and l per scan in x and y).  A lane with
+// no neighbour adds zero, which leaves a canonical pair as it is.
+__device__ __forceinline__ void ff_warp_scan2(float2& h, float2& l) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        float2 uh, ul;
+        uh.x = __shfl_up_sync(0xffffffffu, h.x, o);
+        uh.y = __shfl_up_sync(0xffffffffu, h.y, o);
+        ul.x = __shfl_up_sync(0xffffffffu, l.x, o);
+        ul.y = __shfl_up_sync(0xffffffffu, l.y, o);
+        if (lane < o) uh = ul = make_float2(0.0f, 0.0f);
+        ff_add2(h, l, uh, ul);
     }
 }
 
@@ -282,17 +364,26 @@ __device__ __forceinline__ void scan_offsets(typename Offset<V>::type* offs, flo
         }
     } else {
         const int nseg = (nbx + 31) >> 5, per = group >> 5;  // segments, segments a group
-        for (int sgm = warp; sgm < nseg; sgm += NW) {
-            const int b = (sgm << 5) + lane;
-            float h = b < nbx ? offs[b].x : 0.0f, l = 0.0f;
-            ff_warp_scan(h, l, 32);
-            if (lane == 31) seg[sgm] = make_float2(h, l);
-            float ph = __shfl_up_sync(0xffffffffu, h, 1), pl = __shfl_up_sync(0xffffffffu, l, 1);
-            if (lane == 0) ph = pl = 0.0f;
-            if (b < nbx) offs[b] = make_float2(ph, pl);
+        for (int pair = warp; 2 * pair < nseg; pair += NW) {  // two segments at a time
+            const int b = (pair << 6) + lane;
+            float2 h, l = make_float2(0.0f, 0.0f);
+            h.x = b < nbx ? offs[b].x : 0.0f;
+            h.y = b + 32 < nbx ? offs[b + 32].x : 0.0f;
+            ff_warp_scan2(h, l);
+            if (lane == 31) {
+                seg[2 * pair] = make_float2(h.x, l.x);
+                seg[2 * pair + 1] = make_float2(h.y, l.y);
+            }
+            float2 p, r;
+            p.x = __shfl_up_sync(0xffffffffu, h.x, 1);
+            p.y = __shfl_up_sync(0xffffffffu, l.x, 1);
+            r.x = __shfl_up_sync(0xffffffffu, h.y, 1);
+            r.y = __shfl_up_sync(0xffffffffu, l.y, 1);
+            if (lane == 0) p = r = make_float2(0.0f, 0.0f);
+            if (b < nbx) offs[b] = p;
+            if (b + 32 < nbx) offs[b + 32] = r;
         }
         cta_sync<ONE>();
-        if (nseg == 1) return;
         float th = 0.0f, tl = 0.0f;  // total of the group before
         for (int g0 = 0; g0 < nseg; g0 += per) {
             const int ng = nseg - g0 < per ? nseg - g0 : per;

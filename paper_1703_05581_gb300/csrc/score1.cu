@@ -170,16 +170,15 @@ __device__ __noinline__ unsigned long long radix_rank(const unsigned char* smem,
     return prefix;
 }
 
-// One warp: the values of ranks t1 <= t2 <= t1 + 1 among the n members of a
-// window at `pack` (padded to a multiple of 128 with +inf), all between lo
-// and hi.  MAD: of |x - mh|.  Counting passes at interpolated pivots; each
-// pass also yields the pivot's neighbours on both sides, and the interval
-// closes in on members, so that clusters of nearly equal values (folds of
-// quantised series) cost no more passes.
-template <bool MAD>
-__device__ __forceinline__ bool pick2(const float* pack, uint32_t n, uint32_t t1, uint32_t t2, float lo, float hi,
+// One warp: the values of ranks t1 <= t2 <= t1 + 1 among the n <= 128 KQ
+// members v of a window (in registers, member 128 k + 4 lane + e in v[4 k + e],
+// +inf beyond n), all between lo and hi.  MAD: of |x - mh|.  Counting passes
+// at interpolated pivots; each pass also yields the pivot's neighbours on both
+// sides, and the interval closes in on members, so that clusters of nearly
+// equal values (folds of quantised series) cost no more passes.
+template <bool MAD, int KQ>
+__device__ __forceinline__ bool pick2(const float (&v)[4 * KQ], uint32_t n, uint32_t t1, uint32_t t2, float lo, float hi,
                                       float mh, float& va, float& vb) {
-    const int lane = threadIdx.x & 31;
     uint32_t cl = 0, ch = n;  // members < lo, <= hi
     bool step = false;        // next pivot: the first member from lo on
     for (int a = 0; a < 32; ++a) {
@@ -189,22 +188,27 @@ __device__ __forceinline__ bool pick2(const float* pack, uint32_t n, uint32_t t1
             if (!(p < hi)) p = lo;
         }
         uint32_t c = 0;
-        float above = INFINITY, upto = -INFINITY;
-        for (uint32_t i = 4 * lane; i < n; i += 128) {
-            const float4 q = *reinterpret_cast<const float4*>(pack + i);
-            const float v[4] = {q.x, q.y, q.z, q.w};
+        float ab[4], up[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            ab[e] = INFINITY;
+            up[e] = -INFINITY;
+        }
+#pragma unroll
+        for (int k = 0; k < KQ; ++k) {
+            if (128u * k >= n) break;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float d = MAD ? fabsf(__fsub_rn(v[e], mh)) : v[e];
+                const float d = MAD ? fabsf(__fsub_rn(v[4 * k + e], mh)) : v[4 * k + e];
                 const bool in = d <= p;
                 c += in;
-                upto = fmaxf(upto, in ? d : -INFINITY);
-                above = fminf(above, in ? INFINITY : d);
+                up[e] = fmaxf(up[e], in ? d : -INFINITY);
+                ab[e] = fminf(ab[e], in ? INFINITY : d);
             }
         }
         c = __reduce_add_sync(0xffffffffu, c);
-        above = -warp_max(-above);
-        upto = warp_max(upto);
+        const float above = -warp_max(-fminf(fminf(ab[0], ab[1]), fminf(ab[2], ab[3])));
+        const float upto = warp_max(fmaxf(max3(up[0], up[1], up[2]), up[3]));
         if (c <= t1) {
             if (c == t1 && t2 == t1) {
                 va = vb = above;
@@ -319,6 +323,15 @@ __global__ void __launch_bounds__(MAXT, MINB)
         }
         if (lane == 0) sh.wc[slot][warp] = make_uint2(a, b);
         __syncthreads();
+        if (NW <= 4) {  // few warps: read them all
+            uint2 t = sh.wc[slot][0];
+            for (int i = 1; i < NW; ++i) {
+                const uint2 v = sh.wc[slot][i];
+                t.x += v.x;
+                t.y += v.y;
+            }
+            return t;
+        }
         const uint2 v = lane < NW ? sh.wc[slot][lane] : make_uint2(0u, 0u);
         return make_uint2(__reduce_add_sync(0xffffffffu, v.x), __reduce_add_sync(0xffffffffu, v.y));
     };
@@ -407,13 +420,24 @@ __global__ void __launch_bounds__(MAXT, MINB)
                 if (INT) sh.fc[warp] = fm;
             }
             __syncthreads();
-            fs = lane < NW ? sh.fa[lane] : 0.0f;
-            fq = lane < NW ? sh.fb[lane] : 0.0f;
-            if (INT) fm = warp_max(lane < NW ? sh.fc[lane] : 0.0f);
+            if (NW <= 4) {
+                fs = sh.fa[0];
+                fq = sh.fb[0];
+                if (INT) fm = sh.fc[0];
+                for (int i = 1; i < NW; ++i) {
+                    fs += sh.fa[i];
+                    fq += sh.fb[i];
+                    if (INT) fm = fmaxf(fm, sh.fc[i]);
+                }
+            } else {
+                fs = lane < NW ? sh.fa[lane] : 0.0f;
+                fq = lane < NW ? sh.fb[lane] : 0.0f;
+                if (INT) fm = warp_max(lane < NW ? sh.fc[lane] : 0.0f);
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                fs += __shfl_xor_sync(0xffffffffu, fs, o);
-                fq += __shfl_xor_sync(0xffffffffu, fq, o);
+                for (int o = 16; o > 0; o >>= 1) {
+                    fs += __shfl_xor_sync(0xffffffffu, fs, o);
+                    fq += __shfl_xor_sync(0xffffffffu, fq, o);
+                }
             }
         } else {
             __syncwarp();
@@ -488,12 +512,23 @@ __global__ void __launch_bounds__(MAXT, MINB)
                         continue;
                     }
                     if (warp == 0) {
-                        // pad, pick, then settle near-ties exactly
+                        // pick, then settle near-ties exactly
                         const uint32_t n = c.y, t1 = r1 - cl, t2 = r2 - cl;
-                        for (uint32_t i = n + lane; i < ((n + 127) & ~127u); i += 32) pack[i] = INFINITY;
+                        constexpr int KQ = NP / 128;
+                        float v[4 * KQ];
+#pragma unroll
+                        for (int k = 0; k < KQ; ++k) {
+                            const uint32_t i = 128 * k + 4 * lane;
+                            float4 q = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+                            if (i < n) q = *reinterpret_cast<const float4*>(pack + i);
+                            v[4 * k] = q.x;
+                            v[4 * k + 1] = i + 1 < n ? q.y : INFINITY;
+                            v[4 * k + 2] = i + 2 < n ? q.z : INFINITY;
+                            v[4 * k + 3] = i + 3 < n ? q.w : INFINITY;
+                        }
                         __syncwarp();
                         float va, vb;
-                        int ok = pick2<MAD>(pack, n, t1, t2, lo, hi, mh, va, vb);
+                        int ok = pick2<MAD, KQ>(v, n, t1, t2, lo, hi, mh, va, vb);
                         if constexpr (!MAD) {
                             if (lane == 0) {
                                 sh.key[0] = ff_key(va, 0.0f);
@@ -505,17 +540,20 @@ __global__ void __launch_bounds__(MAXT, MINB)
                             // within 2 E of va, vb; rank those exactly
                             const float E = (hi + fabsf(mh)) * 1.2e-7f;
                             const float ca = va - 3.0f * E, cb = vb + 3.0f * E;
-                            // (packed in place, every read before the writes it meets)
                             uint32_t less = 0, m = 0;
-                            for (uint32_t i0 = 0; i0 < n; i0 += 32) {
-                                const uint32_t i = i0 + lane;
-                                const float v = i < n ? pack[i] : INFINITY, d = fabsf(__fsub_rn(v, mh));
+#pragma unroll
+                            for (int i = 0; i < 4 * KQ; ++i) {
+                                if (32u * (i & ~3) >= n) break;
+                                const float d = fabsf(__fsub_rn(v[i], mh));
                                 less += d < ca;
-                                const unsigned near = __ballot_sync(0xffffffffu, d >= ca && d <= cb);
-                                if (d >= ca && d <= cb) pack[m + __popc(near & ((1u << lane) - 1))] = v;
-                                m += __popc(near);
-                                __syncwarp();
+                                const bool is = d >= ca && d <= cb;
+                                const unsigned near = __ballot_sync(0xffffffffu, is);
+                                if (near) {
+                                    if (is) pack[m + __popc(near & ((1u << lane) - 1))] = v[i];
+                                    m += __popc(near);
+                                }
                             }
+                            __syncwarp();
                             less = __reduce_add_sync(0xffffffffu, less);
                             if (ca < lo || cb > hi) {  // too near the window's edge
                                 ok = 0;
@@ -889,10 +927,11 @@ ffa_status score1_t(const void* d_prof, const ScoreGroup& sg, int64_t count, int
     // with 448 threads of 72 registers, 35.7k with 640 of 48).
     switch (shape) {
         case 0:
-            // one warp a profile up to 1200 bins (1100 bins: 2.1k SM cycles,
-            // 2.7k with two warps; 366 bins: 1.2k and 2.2k), two above
-            // (1900 bins: 3.6k and 3.7k)
-            if (p0 <= 1200) {
+            // One warp a profile up to 1200 bins (1100 bins: 2.3k SM cycles,
+            // 2.8k with two warps; 366 bins: 1.25k and 2.2k); above, two for
+            // ready profiles (1489 bins: 2.8k, 3.0k with one), one in a search
+            // (12 DM trials: 278 ms, 291 ms with two).
+            if (p0 <= 1200 || FF) {
                 score1_shape<V, 8>(p0, wtop, 1, 32, 32, 13, &threads, &lay, &smem);
                 return FFA_SCORE1(8, true, 32, 24);
             }
