@@ -8,6 +8,7 @@
 #include <atomic>
 #include <chrono>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -97,15 +98,10 @@ ffa_status ensure_smem(const void* func, size_t bytes) {
 // ---------------------------------------------------------------------------
 // candidate extraction kernels
 // ---------------------------------------------------------------------------
-struct CandCtl {
-    unsigned long long best_key;
-    uint32_t count;  // records with snr >= snr_min
-    uint32_t n_out;
-    unsigned long long prefix, mask;
-    uint32_t rank;
-    uint32_t take;   // min(top_k, count)
-    uint32_t hist[256];
-};
+constexpr int CAND_MAX = 4096;
+constexpr int CAND_BITS = 11;                                // key bits a pass narrows
+constexpr int CAND_PASSES = (64 + CAND_BITS - 1) / CAND_BITS;
+constexpr int CAND_BINS = 1 << CAND_BITS;
 
 struct CandOut {
     int64_t trial;
@@ -115,7 +111,23 @@ struct CandOut {
     int32_t pad;
 };
 
-constexpr int CAND_MAX = 4096;
+// The head and the outputs are read back together.
+struct CandCtl {
+    unsigned long long best_key;
+    uint32_t n_out;  // min(top_k, records with snr >= snr_min)
+    uint32_t pad;
+    CandOut out[CAND_MAX];
+    unsigned long long keys[CAND_MAX];
+    unsigned long long prefix, mask;  // the wanted key's digits so far
+    uint32_t count;                   // records with snr >= snr_min
+    uint32_t rank;                    // wanted rank among the keys with the prefix
+    uint32_t below;                   // keys below the prefix
+    uint32_t take;
+    uint32_t n_keys;
+    uint32_t done;                    // the keys up to the prefix's end are few enough to sort
+    uint32_t ticket[CAND_PASSES];
+    uint32_t hist[CAND_BINS];
+};
 
 // ascending key = descending snr, then ascending trial index
 __device__ __forceinline__ unsigned long long cand_key(float snr, int64_t idx) {
@@ -123,111 +135,132 @@ __device__ __forceinline__ unsigned long long cand_key(float snr, int64_t idx) {
 }
 
 __global__ void k_cand_init(CandCtl* ctl) {
-    int t = threadIdx.x;
+    const int t = threadIdx.x;
     if (t == 0) {
         ctl->best_key = ~0ull;
-        ctl->count = 0;
         ctl->n_out = 0;
         ctl->prefix = 0;
         ctl->mask = 0;
+        ctl->count = 0;
         ctl->rank = 0;
+        ctl->below = 0;
         ctl->take = 0;
+        ctl->n_keys = 0;
+        ctl->done = 0;
     }
-    for (int b = t; b < 256; b += blockDim.x) ctl->hist[b] = 0;
+    if (t < CAND_PASSES) ctl->ticket[t] = 0;
+    for (int b = t; b < CAND_BINS; b += blockDim.x) ctl->hist[b] = 0;
 }
 
-__global__ void k_cand_count(const ffa_record* __restrict__ rec, int64_t n, float snr_min,
-                             CandCtl* ctl) {
+// One pass narrows the take-th smallest key by CAND_BITS bits: a histogram of
+// the next digit of the keys with the prefix, and the last CTA to finish picks
+// the digit.  Pass 0 also counts the records and finds the best.  The passes
+// end early (done) once the keys up to the prefix's last are few: they are all
+// sorted, which takes less than the remaining passes.
+__global__ void __launch_bounds__(256) k_cand_pass(const ffa_record* __restrict__ rec, int64_t n, float snr_min,
+                                                   int pass, int top_k, CandCtl* ctl) {
+    __shared__ uint32_t h[CAND_BINS];
     __shared__ unsigned long long s_best;
-    __shared__ uint32_t s_cnt;
-    if (threadIdx.x == 0) {
+    __shared__ uint32_t s_cnt, s_last, s_warp[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (pass > 0 && (ctl->done || ctl->take == 0)) return;
+    for (int b = tid; b < CAND_BINS; b += 256) h[b] = 0;
+    if (tid == 0) {
         s_best = ~0ull;
         s_cnt = 0;
     }
     __syncthreads();
+    const unsigned long long prefix = ctl->prefix, mask = ctl->mask;
+    const int shift = 64 - CAND_BITS * (pass + 1) > 0 ? 64 - CAND_BITS * (pass + 1) : 0;
     unsigned long long best = ~0ull;
     uint32_t cnt = 0;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        float s = rec[i].snr;
-        unsigned long long k = cand_key(s, i);
-        best = k < best ? k : best;
-        cnt += (s >= snr_min);
+    const int64_t stride = (int64_t)gridDim.x * 256;
+    for (int64_t i = (int64_t)blockIdx.x * 256 + tid; i < n; i += stride) {
+        const float s = rec[i].snr;
+        const unsigned long long k = cand_key(s, i);
+        if (pass == 0) best = k < best ? k : best;
+        if (!(s >= snr_min)) continue;
+        ++cnt;
+        if ((k & mask) == prefix) atomicAdd(&h[(k >> shift) & (CAND_BINS - 1)], 1u);
     }
-    atomicMin(&s_best, best);
-    atomicAdd(&s_cnt, cnt);
+    if (pass == 0) {
+        atomicMin(&s_best, best);
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0) atomicAdd(&s_cnt, cnt);
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    for (int b = tid; b < CAND_BINS; b += 256)
+        if (h[b]) atomicAdd(&ctl->hist[b], h[b]);
+    if (pass == 0 && tid == 0) {
         atomicMin(&ctl->best_key, s_best);
         atomicAdd(&ctl->count, s_cnt);
     }
-}
-
-__global__ void k_cand_hist(const ffa_record* __restrict__ rec, int64_t n, float snr_min,
-                            int pass, CandCtl* ctl) {
-    __shared__ uint32_t h[256];
-    for (int b = threadIdx.x; b < 256; b += blockDim.x) h[b] = 0;
+    __threadfence();
     __syncthreads();
-    const unsigned long long prefix = ctl->prefix, mask = ctl->mask;
-    const int shift = 56 - 8 * pass;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        float s = rec[i].snr;
-        if (!(s >= snr_min)) continue;
-        unsigned long long k = cand_key(s, i);
-        if ((k & mask) == prefix) atomicAdd(&h[(k >> shift) & 0xff], 1u);
-    }
+    if (tid == 0) s_last = atomicAdd(&ctl->ticket[pass], 1u) == gridDim.x - 1;
     __syncthreads();
-    for (int b = threadIdx.x; b < 256; b += blockDim.x)
-        if (h[b]) atomicAdd(&ctl->hist[b], h[b]);
-}
-
-__global__ void k_cand_pick(int pass, int top_k, CandCtl* ctl) {
-    if (threadIdx.x != 0) return;
-    if (pass == 0) {
-        ctl->take = ctl->count < (uint32_t)top_k ? ctl->count : (uint32_t)top_k;
-        ctl->rank = ctl->take > 0 ? ctl->take - 1 : 0;
+    if (!s_last) return;
+    __threadfence();
+    // ---- the last CTA: the digit that holds the wanted rank
+    constexpr int PER = CAND_BINS / 256;
+    const uint32_t count = *(volatile uint32_t*)&ctl->count;
+    const uint32_t take = pass == 0 ? (count < (uint32_t)top_k ? count : (uint32_t)top_k) : ctl->take;
+    const uint32_t rank = pass == 0 ? (take ? take - 1 : 0) : ctl->rank;
+    uint32_t v[PER], sum = 0;
+    for (int t = 0; t < PER; ++t) {
+        v[t] = *(volatile uint32_t*)&ctl->hist[tid * PER + t];
+        ctl->hist[tid * PER + t] = 0;
+        sum += v[t];
     }
-    if (ctl->take == 0) return;
-    const int shift = 56 - 8 * pass;
-    uint32_t c = 0;
-    for (int b = 0; b < 256; ++b) {
-        uint32_t h = ctl->hist[b];
-        if (ctl->rank < c + h) {
-            ctl->rank -= c;
-            ctl->prefix |= (unsigned long long)b << shift;
-            ctl->mask |= 0xffull << shift;
-            break;
+    uint32_t x = sum;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t u = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += u;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    uint32_t c = x - sum;
+    for (int w = 0; w < warp; ++w) c += s_warp[w];
+    if (pass == 0 && tid == 0) ctl->take = take;
+    if (take > 0) {
+        for (int t = 0; t < PER; ++t) {
+            if (rank >= c && rank < c + v[t]) {
+                const uint32_t upto = ctl->below + c + v[t];  // keys up to this digit's end
+                ctl->rank = rank - c;
+                ctl->below += c;
+                // the last pass holds the bits that are left; its upper bits
+                // are the prefix's own
+                ctl->prefix |= (unsigned long long)(tid * PER + t) << shift;
+                ctl->mask |= (unsigned long long)(CAND_BINS - 1) << shift;
+                const uint32_t few = 2 * take > 512 ? 2 * take : 512;
+                ctl->done = upto <= (few < CAND_MAX ? few : CAND_MAX);
+            }
+            c += v[t];
         }
-        c += h;
     }
-    for (int b = 0; b < 256; ++b) ctl->hist[b] = 0;
 }
 
-__global__ void k_cand_compact(const ffa_record* __restrict__ rec, int64_t n, float snr_min,
-                               CandCtl* ctl, unsigned long long* keys) {
+__global__ void k_cand_compact(const ffa_record* __restrict__ rec, int64_t n, float snr_min, CandCtl* ctl) {
     if (ctl->take == 0) return;
-    const unsigned long long thr = ctl->prefix;  // key of the take-th best
+    const unsigned long long thr = ctl->prefix | ~ctl->mask;  // no key below the take-th best is above this
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         float s = rec[i].snr;
         if (!(s >= snr_min)) continue;
         unsigned long long k = cand_key(s, i);
         if (k <= thr) {
-            uint32_t slot = atomicAdd(&ctl->n_out, 1u);
-            if (slot < CAND_MAX) keys[slot] = k;
+            uint32_t slot = atomicAdd(&ctl->n_keys, 1u);
+            if (slot < CAND_MAX) ctl->keys[slot] = k;
         }
     }
 }
 
-__global__ void __launch_bounds__(1024) k_cand_sort(const ffa_record* __restrict__ rec,
-                                                    CandCtl* ctl, const unsigned long long* keys,
-                                                    CandOut* out) {
+__global__ void __launch_bounds__(1024) k_cand_sort(const ffa_record* __restrict__ rec, CandCtl* ctl) {
     __shared__ unsigned long long sk[CAND_MAX];
-    uint32_t n = ctl->n_out < CAND_MAX ? ctl->n_out : CAND_MAX;
+    const uint32_t n = ctl->n_keys < CAND_MAX ? ctl->n_keys : CAND_MAX;
     uint32_t np2 = 1;
     while (np2 < n) np2 <<= 1;
-    for (uint32_t t = threadIdx.x; t < np2; t += blockDim.x) sk[t] = t < n ? keys[t] : ~0ull;
+    for (uint32_t t = threadIdx.x; t < np2; t += blockDim.x) sk[t] = t < n ? ctl->keys[t] : ~0ull;
     __syncthreads();
     for (uint32_t kk = 2; kk <= np2; kk <<= 1) {
         for (uint32_t jj = kk >> 1; jj > 0; jj >>= 1) {
@@ -245,7 +278,8 @@ __global__ void __launch_bounds__(1024) k_cand_sort(const ffa_record* __restrict
             __syncthreads();
         }
     }
-    for (uint32_t t = threadIdx.x; t < n; t += blockDim.x) {
+    const uint32_t take = ctl->take < n ? ctl->take : n;
+    for (uint32_t t = threadIdx.x; t < take; t += blockDim.x) {
         int64_t idx = (int64_t)(uint32_t)(sk[t] & 0xffffffffull);
         ffa_record r = rec[idx];
         CandOut o;
@@ -254,8 +288,9 @@ __global__ void __launch_bounds__(1024) k_cand_sort(const ffa_record* __restrict
         o.width = r.width;
         o.phase = r.phase;
         o.pad = 0;
-        out[t] = o;
+        ctl->out[t] = o;
     }
+    if (threadIdx.x == 0) ctl->n_out = take;
 }
 
 }  // namespace ffa
@@ -463,8 +498,7 @@ ffa_status ffa_plan_create(const ffa_search_config* cfg, int64_t n, ffa_plan** o
     p->off_plane1 = off;
     off = align256(off + 4 * (size_t)p->plane_elems);
     p->off_cand = off;
-    off = align256(off + sizeof(CandCtl) + 256 + sizeof(unsigned long long) * CAND_MAX +
-                   sizeof(CandOut) * CAND_MAX);
+    off = align256(off + sizeof(CandCtl));
     p->off_best = off;
     off = align256(off + ffa::best_workspace_bytes((int64_t)p->entries.size(), p->n_trials));
     p->off_bits = off;
@@ -1103,34 +1137,33 @@ static ffa_status candidates_range(const ffa_plan* p, int64_t e0, int64_t e1, co
     if (!d_records || !d_ws) return fail(FFA_ERR_ARG, "candidates: null buffer");
     if (ws_bytes < p->ws_bytes) return fail(FFA_ERR_OOM, "candidates: workspace too small");
     cudaStream_t st = as_stream(stream);
-    char* base = (char*)d_ws + p->off_cand;
-    CandCtl* ctl = (CandCtl*)base;
-    unsigned long long* keys = (unsigned long long*)(base + align256(sizeof(CandCtl)));
-    CandOut* cout = (CandOut*)(base + align256(sizeof(CandCtl)) + sizeof(unsigned long long) * CAND_MAX);
+    CandCtl* ctl = (CandCtl*)((char*)d_ws + p->off_cand);
     const int64_t t0 = p->entries[(size_t)e0].first_trial;
     const ffa_plan_entry& el = p->entries[(size_t)(e1 - 1)];
     const int64_t n = el.first_trial + el.m_rows - t0;
     const ffa_record* rec = d_records + t0;
     const float smin = (float)snr_min;
-    const int grid = sm_count() * 8;
+    // CTAs enough for the records, and no more to wait for
+    const int grid = (int)std::min<int64_t>((int64_t)sm_count() * 8, (n + 1023) / 1024);
     k_cand_init<<<1, 256, 0, st>>>(ctl);
-    k_cand_count<<<grid, 256, 0, st>>>(rec, n, smin, ctl);
-    for (int pass = 0; pass < 8; ++pass) {
-        k_cand_hist<<<grid, 256, 0, st>>>(rec, n, smin, pass, ctl);
-        k_cand_pick<<<1, 32, 0, st>>>(pass, top_k, ctl);
-    }
-    k_cand_compact<<<grid, 256, 0, st>>>(rec, n, smin, ctl, keys);
-    k_cand_sort<<<1, 1024, 0, st>>>(rec, ctl, keys, cout);
+    for (int pass = 0; pass < CAND_PASSES; ++pass) k_cand_pass<<<grid, 256, 0, st>>>(rec, n, smin, pass, top_k, ctl);
+    k_cand_compact<<<grid, 256, 0, st>>>(rec, n, smin, ctl);
+    k_cand_sort<<<1, 1024, 0, st>>>(rec, ctl);
     FFA_LAUNCH_CHECK("candidates kernels");
-    count_launch(21);
+    count_launch(CAND_PASSES + 3);
     ffa_status s = ffa_wait(stream, d_status, timeout_ms);
     if (s != FFA_OK) return s;
-    CandCtl h;
-    FFA_CUDA_TRY(cudaMemcpy(&h, ctl, sizeof(CandCtl), cudaMemcpyDeviceToHost));
-    uint32_t m = std::min<uint32_t>(h.n_out, (uint32_t)top_k);
+    // the head and as many outputs as can have been asked for, in one copy
+    std::vector<char> back(offsetof(CandCtl, out) + sizeof(CandOut) * (size_t)top_k);
+    FFA_CUDA_TRY(cudaMemcpy(back.data(), ctl, back.size(), cudaMemcpyDeviceToHost));
+    unsigned long long best_key;
+    uint32_t n_back;
+    std::memcpy(&best_key, back.data() + offsetof(CandCtl, best_key), sizeof(best_key));
+    std::memcpy(&n_back, back.data() + offsetof(CandCtl, n_out), sizeof(n_back));
+    const uint32_t m = std::min<uint32_t>(n_back, (uint32_t)top_k);
     std::vector<CandOut> buf(m);
-    if (m > 0) FFA_CUDA_TRY(cudaMemcpy(buf.data(), cout, sizeof(CandOut) * m, cudaMemcpyDeviceToHost));
-    if (h.best_key != ~0ull) *best = t0 + (int64_t)(uint32_t)(h.best_key & 0xffffffffull);
+    if (m > 0) std::memcpy(buf.data(), back.data() + offsetof(CandCtl, out), sizeof(CandOut) * m);
+    if (best_key != ~0ull) *best = t0 + (int64_t)(uint32_t)(best_key & 0xffffffffull);
     const ffa_search_config& c = p->cfg;
     for (uint32_t t = 0; t < m; ++t) {
         const CandOut& o = buf[t];
