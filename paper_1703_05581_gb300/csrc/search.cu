@@ -1107,10 +1107,12 @@ ffa_status ffa_wait(void* stream, const int32_t* d_status, int32_t timeout_ms) {
         cudaError_t e = cudaStreamQuery(st);
         if (e == cudaSuccess) break;
         if (e != cudaErrorNotReady) return cuda_fail(e, "wait: cudaStreamQuery");
-        auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(
-                      std::chrono::steady_clock::now() - t0).count();
-        if (timeout_ms >= 0 && ms > timeout_ms) return fail(FFA_ERR_TIMEOUT, "wait: stream did not finish in time");
-        std::this_thread::sleep_for(std::chrono::microseconds(200));
+        const auto us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
+        if (timeout_ms >= 0 && us > (int64_t)timeout_ms * 1000) return fail(FFA_ERR_TIMEOUT, "wait: stream did not finish in time");
+        // poll a short wait closely (a short search ends within a millisecond),
+        // then sleep for a sixteenth of the time waited, at most 200 us
+        if (us < 300) std::this_thread::yield();
+        else std::this_thread::sleep_for(std::chrono::microseconds(std::min<int64_t>(us / 16, 200)));
     }
     if (d_status) {
         int32_t h = 0;
