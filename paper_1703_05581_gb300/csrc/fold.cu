@@ -174,6 +174,34 @@ __device__ __forceinline__ void store4(T* d, const T (&v)[4], int left, bool vec
     }
 }
 
+// A warp's 128 consecutive outputs (four per lane) to a row that is not
+// 16-byte aligned, off elements past such a boundary: every lane but the first
+// stores the aligned quad that ends in its own values, with the lane before's
+// last `off` in front, so that a sector is written once and not in four parts
+// (dense int8 8192 x 1489, passes of
+// 5 + 4 + 4 stages: 86 -> 78 us).
+template <class T>
+__device__ __forceinline__ void store_row(T* d, const T (&v)[4], int off) {
+    const int lane = threadIdx.x & 31;
+    const T u1 = __shfl_up_sync(0xffffffffu, v[1], 1);
+    const T u2 = __shfl_up_sync(0xffffffffu, v[2], 1);
+    const T u3 = __shfl_up_sync(0xffffffffu, v[3], 1);
+    const int a = as_bits(off == 1 ? u3 : off == 2 ? u2 : u1), b = as_bits(off == 1 ? v[0] : off == 2 ? u3 : u2);
+    const int c = as_bits(off == 1 ? v[1] : off == 2 ? v[0] : u3), e = as_bits(off == 1 ? v[2] : off == 2 ? v[1] : v[0]);
+    if (lane > 0) {
+        *reinterpret_cast<int4*>(d - off) = make_int4(a, b, c, e);
+    } else {
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+            if (x < 4 - off) d[x] = v[x];
+    }
+    if (lane == 31) {
+#pragma unroll
+        for (int x = 1; x < 4; ++x)
+            if (x >= 4 - off) d[x] = v[x];
+    }
+}
+
 // ---------------------------------------------------------------------------
 // One pass of q = Q1 + Q2 <= 6 stages.  A CTA takes a (block, kappa, column
 // tile of B columns) -- or, persistent, one after another: it stages 2^q input rows of B + 2^q - 1 columns, row u
@@ -404,6 +432,7 @@ __global__ void __launch_bounds__(fk_threads(Q1 + Q2, B), fk_threads(Q1 + Q2, B)
             for (int it = threadIdx.x; it < items; it += FK_THREADS) {
                 const int strip = it % nstrips, k1 = it / nstrips;
                 const int x0 = 4 * strip;
+                const int whole = ncols - (x0 - 4 * lane);  // columns from the warp's first on
                 if (x0 >= ncols) continue;
                 auto sub2 = [&](auto tt) {
                     using F = RegFFA<T, Q2>;
@@ -413,8 +442,17 @@ __global__ void __launch_bounds__(fk_threads(Q1 + Q2, B), fk_threads(Q1 + Q2, B)
                     T out[R2][4];
                     F::run(a, out);
                     T* d = drow + (int64_t)(k1 * R2) * ld + x0;
+                    if (q == 6 || vec || whole < 128) {  // (64-row tiles: bound by instructions, not by sectors)
 #pragma unroll
-                    for (int v = 0; v < R2; ++v) store4(d + v * ld, out[v], ncols - x0, vec);
+                        for (int v = 0; v < R2; ++v) store4(d + v * ld, out[v], ncols - x0, vec);
+                    } else {
+#pragma unroll
+                        for (int v = 0; v < R2; ++v) {
+                            const int off = (int)((uintptr_t)(d + v * ld) >> 2) & 3;  // the same in every lane
+                            if (off == 0) store4(d + v * ld, out[v], 4, true);
+                            else store_row(d + v * ld, out[v], off);
+                        }
+                    }
                 };
                 switch (k1 & 3) {
                     case 0: sub2(std::integral_constant<int, 0>{}); break;
@@ -548,12 +586,17 @@ int log2i(int64_t v) {
     return r;
 }
 
-FoldShape tuned_shape(int precision, int stages, int64_t p0) {
+FoldShape tuned_shape(int precision, int stages, int64_t p0, int64_t ld) {
+    // Untuned, twelve stages on dense rows that are not 16-byte aligned: three
+    // passes of four instead of two of six, whose unaligned rows cost more
+    // than a pass (4096 x 19977: 428 us, 461; 4096 x 4001: 106, 117; 2048 rows,
+    // six and five stages: 293 us, 377 as four, four and three).
+    const FoldShape none = (ld & 3) != 0 && stages == 12 ? FoldShape{5, 0} : SHAPE_DEFAULT;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return SHAPE_DEFAULT;
+    if (cudaGetDevice(&dev) != cudaSuccess) return none;
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune.find(std::make_tuple(dev, precision, stages, log2i(p0)));
-    return it == g_tune.end() ? SHAPE_DEFAULT : it->second;
+    return it == g_tune.end() ? none : it->second;
 }
 }  // namespace
 
@@ -635,7 +678,7 @@ ffa_status launch_fold_group(const void* d_z, int32_t precision, int n, const in
         fg.src[i] = z ? z[i] : d_z;
     }
     return fold_group(d_z, precision, fg, m_rows, stages, d_plane, d_tmp, st,
-                      tuned_shape(precision, stages, p0[n - 1]));
+                      tuned_shape(precision, stages, p0[n - 1], plane_pitch(p0[n - 1])));
 }
 
 // Run the first `stages` FFA stages (all of them when stages < 0).  With
@@ -647,7 +690,7 @@ ffa_status launch_fold(const void* d_z, int32_t precision, int64_t p0, int64_t m
     while ((1ll << m) < m_rows) ++m;
     if (stages < 0 || stages > m) stages = m;
     return fold_with(d_z, precision, p0, m_data, m_rows, stages, ld, d_plane, d_tmp, st,
-                     tuned_shape(precision, stages, p0));
+                     tuned_shape(precision, stages, p0, ld));
 }
 
 }  // namespace ffa
