@@ -945,6 +945,12 @@ ffa_status score1_t(const void* d_prof, const ScoreGroup& sg, int64_t count, int
             // two profiles an SM while their shared memory fits, else one
             score1_shape<V, 32>(p0, wtop, 3, 320, 448, 7, &threads, &lay, &smem);
             if (2 * (smem + sizeof(S1Sh) + 1024) <= 228 * 1024) return FFA_SCORE1(32, false, 448, 2);
+            // (threads of the one, 4096 x 29705: float 618 us with 640, 631
+            // with 768; int 692 and 678)
+            if (std::is_integral<V>::value) {
+                score1_shape<V, 32>(p0, wtop, 2, 512, 768, 9, &threads, &lay, &smem);
+                return FFA_SCORE1(32, false, 768, 1);
+            }
             score1_shape<V, 32>(p0, wtop, 3, 512, 640, 9, &threads, &lay, &smem);
             return FFA_SCORE1(32, false, 640, 1);
     }
