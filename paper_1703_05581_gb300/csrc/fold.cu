@@ -203,8 +203,8 @@ __device__ __forceinline__ void store_row(T* d, const T (&v)[4], int off) {
 }
 
 // ---------------------------------------------------------------------------
-// One pass of q = Q1 + Q2 <= 6 stages.  A CTA takes a (block, kappa, column
-// tile of B columns) -- or, persistent, one after another: it stages 2^q input rows of B + 2^q - 1 columns, row u
+// One pass of q = Q1 + Q2 <= 6 stages.  A CTA owns (block, kappa, column
+// tile of B columns): it stages 2^q input rows of B + 2^q - 1 columns, row u
 // starting at column c + kappa*u (cyclically), in shared memory.  Sub-pass 1:
 // each thread takes 4 consecutive columns of a group of 2^Q1 rows, applies
 // Q1 stages in registers and stores the group's 2^Q1 partial trials,
@@ -212,10 +212,7 @@ __device__ __forceinline__ void store_row(T* d, const T (&v)[4], int off) {
 // input row u2 of the last Q2 stages is read at column offset k1*u2 (the
 // shift that the unrolled recursion assigns it), Q2 stages in registers, and
 // the tile's output rows go to global memory (128-bit stores on a padded
-// pitch).  The staging buffer is free once sub-pass 1 is done, so a persistent
-// CTA issues the next tile's copies before sub-pass 2, to arrive under it.  Tiles are
-// B = 256 columns up to 5 stages and 128 for 6 (64 rows), so two CTAs fit an
-// SM.
+// pitch).  Tiles are B = 256 columns up to 5 stages and 128 for 6 (64 rows).
 //
 // Alignment.  The staging copies are 16 bytes wide, so a row's columns keep
 // the misalignment 0..3 of their address.  It is (t * u) & 3 in row u for one
@@ -226,13 +223,13 @@ __device__ __forceinline__ void store_row(T* d, const T (&v)[4], int off) {
 // no select on it.  Rows off that pattern (they wrapped past p0, or the plane
 // is not 16-byte aligned) are staged element by element onto it.
 // ---------------------------------------------------------------------------
-// Threads of a CTA: 64-row tiles of 256 columns leave room for one CTA an SM.
-__host__ __device__ constexpr int fk_threads(int q, int b) { return q == 6 && b == 256 ? 512 : 256; }
-// Persistent CTAs, the next tile staged under sub-pass 2, where shared memory
-// holds the SM to two CTAs or one (64 rows of four-byte elements); elsewhere
-// more CTAs in flight hide the staging better than the registers that a
-// pipelined tile takes.
-__host__ __device__ constexpr bool fk_persistent(int q, bool widen) { return q == 6 && !widen; }
+constexpr int FK_THREADS = 256;
+// Six stages (3 + 3): sub-pass 1 works in place, a warp on each of the eight
+// groups, so one buffer of 64 rows (50 KB) serves both sub-passes and four
+// CTAs fit an SM, where two buffers left room for two: 4096 x 19977, first
+// pass, 163 us with two CTAs that staged the next tile under sub-pass 2, 153
+// in place with three, 145 with four; int8 4096 x 29 500: 230, 200, 181.
+__host__ __device__ constexpr bool fk_inplace(int q1, int q2) { return q1 == 3 && q2 == 3; }
 __host__ __device__ constexpr int fk_r4(int x) { return (x + 3) & ~3; }
 __host__ __device__ constexpr int fk_max(int a, int b) { return a > b ? a : b; }
 __host__ __device__ constexpr int fk_wt(int q, int b) { return b + (1 << q) - 1; }                  // staged columns
@@ -248,26 +245,24 @@ __host__ __device__ constexpr int fk_wb(int q, int q1, int b) {
 }
 
 template <class T, bool FIRST, int Q1, int Q2, int B>
-__global__ void __launch_bounds__(fk_threads(Q1 + Q2, B), fk_threads(Q1 + Q2, B) == 512 ? 1 : 2) k_fold(const void* __restrict__ src_v, T* __restrict__ dst_all,
+__global__ void __launch_bounds__(FK_THREADS, fk_inplace(Q1, Q2) ? 4 : 2) k_fold(const void* __restrict__ src_v, T* __restrict__ dst_all,
                                                        const FoldGroup fg, int s) {
     constexpr int q = Q1 + Q2;
-    constexpr int FK_THREADS = fk_threads(q, B);
+    constexpr bool INPLACE = fk_inplace(Q1, Q2);
     constexpr int rows = 1 << q;
     constexpr int R1 = 1 << Q1, R2 = 1 << Q2;
     constexpr int WT = fk_wt(q, B), W1 = fk_w1(q, Q1, B);
-    constexpr int WA = fk_wa(q, Q1, B), WB = fk_wb(q, Q1, B);
+    constexpr int WB = fk_wb(q, Q1, B), WA = INPLACE ? fk_max(fk_wa(q, Q1, B), WB) : fk_wa(q, Q1, B);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* bufA = reinterpret_cast<T*>(smem_raw);
     T* bufB = bufA + rows * WA;
 
     using S = typename std::conditional<FIRST, typename FoldIn<T>::type, T>::type;
     constexpr bool WIDEN = sizeof(S) == 1;  // int8 series
-    constexpr bool PERSIST = fk_persistent(q, WIDEN);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     constexpr int NW = FK_THREADS / 32;
     constexpr int RPW = (rows + NW - 1) / NW;            // rows staged by a warp
     constexpr int KPL = ((WT + 6) / 4 + 31) / 32;        // aligned words per lane and row (WIDEN)
-    const uint32_t units = (uint32_t)fg.unit0[fg.n];     // fits int32
 
     struct Tile {
         int64_t p0, ld, blk, c;
@@ -367,11 +362,10 @@ __global__ void __launch_bounds__(fk_threads(Q1 + Q2, B), fk_threads(Q1 + Q2, B)
         }
     };
 
-    uint32_t unit = blockIdx.x;
-    Tile w = locate(unit);
+    const Tile w = locate(blockIdx.x);
     stage_issue(w);
     stage_finish(w.t);
-    for (;;) {
+    {
         __syncthreads();
         T* __restrict__ dst = dst_all + fg.off[w.ei];
         const int64_t ld = w.ld;
@@ -383,27 +377,50 @@ __global__ void __launch_bounds__(fk_threads(Q1 + Q2, B), fk_threads(Q1 + Q2, B)
         auto sub1 = [&](auto tt) {
             using F = RegFFA<T, Q1>;
             constexpr int nstrips = (W1 + 3) / 4;
-            constexpr int items = (rows / R1) * nstrips;
-            for (int it = threadIdx.x; it < items; it += FK_THREADS) {
-                const int strip = it % nstrips, g = it / nstrips;
-                const int x0 = 4 * strip;
-                T a[R1][F::W];
-                // rows g * R1 + u: (t * (g * R1 + u)) & 3 = (t * u) & 3 when R1 is a multiple of 4
-                F::template load_rows<decltype(tt)::value>(bufA + g * R1 * WA + x0, WA, 0, a,
-                                                           std::make_index_sequence<R1>{});
-                T out[R1][4];
-                F::run(a, out);
-                if (Q2 == 0) {
-                    if (x0 < ncols) {
-#pragma unroll
-                        for (int v = 0; v < R1; ++v) store4(drow + v * ld + x0, out[v], ncols - x0, vec);
+            if constexpr (INPLACE) {
+                // 32 strips at a time from the left: a strip's halo lies in
+                // its own wave, read before the wave's stores, or to the right
+                T* grp = bufA + warp * R1 * WA;
+                for (int s0 = 0; s0 < nstrips; s0 += 32) {
+                    const int x0 = 4 * (s0 + lane);
+                    const bool on = s0 + lane < nstrips;
+                    T a[R1][F::W], out[R1][4];
+                    if (on) {
+                        F::template load_rows<decltype(tt)::value>(grp + x0, WA, 0, a, std::make_index_sequence<R1>{});
+                        F::run(a, out);
                     }
-                } else {
-                    // group g is input row u2 = g of sub-pass 2
+                    __syncwarp();
+                    if (on) {
 #pragma unroll
-                    for (int v = 0; v < R1; ++v)
-                        *reinterpret_cast<int4*>(bufB + (v * R2 + g) * WB + x0) =
-                            make_int4(as_bits(out[v][0]), as_bits(out[v][1]), as_bits(out[v][2]), as_bits(out[v][3]));
+                        for (int v = 0; v < R1; ++v)
+                            *reinterpret_cast<int4*>(grp + v * WA + x0) =
+                                make_int4(as_bits(out[v][0]), as_bits(out[v][1]), as_bits(out[v][2]), as_bits(out[v][3]));
+                    }
+                    __syncwarp();
+                }
+            } else {
+                constexpr int items = (rows / R1) * nstrips;
+                for (int it = threadIdx.x; it < items; it += FK_THREADS) {
+                    const int strip = it % nstrips, g = it / nstrips;
+                    const int x0 = 4 * strip;
+                    T a[R1][F::W];
+                    // rows g * R1 + u: (t * (g * R1 + u)) & 3 = (t * u) & 3 when R1 is a multiple of 4
+                    F::template load_rows<decltype(tt)::value>(bufA + g * R1 * WA + x0, WA, 0, a,
+                                                               std::make_index_sequence<R1>{});
+                    T out[R1][4];
+                    F::run(a, out);
+                    if (Q2 == 0) {
+                        if (x0 < ncols) {
+#pragma unroll
+                            for (int v = 0; v < R1; ++v) store4(drow + v * ld + x0, out[v], ncols - x0, vec);
+                        }
+                    } else {
+                        // group g is input row u2 = g of sub-pass 2
+#pragma unroll
+                        for (int v = 0; v < R1; ++v)
+                            *reinterpret_cast<int4*>(bufB + (v * R2 + g) * WB + x0) =
+                                make_int4(as_bits(out[v][0]), as_bits(out[v][1]), as_bits(out[v][2]), as_bits(out[v][3]));
+                    }
                 }
             }
         };
@@ -415,16 +432,6 @@ __global__ void __launch_bounds__(fk_threads(Q1 + Q2, B), fk_threads(Q1 + Q2, B)
             default: sub1(std::integral_constant<int, 3>{}); break;
         }
         __syncthreads();
-        // bufA is free: the next tile's copies run under sub-pass 2
-        bool more = false;
-        if constexpr (PERSIST) {
-            unit += gridDim.x;
-            more = unit < units;
-        }
-        if (more) {
-            w = locate(unit);
-            stage_issue(w);
-        }
         if constexpr (Q2 > 0) {
             constexpr int nstrips = B / 4;
             constexpr int items = R1 * nstrips;
@@ -437,8 +444,13 @@ __global__ void __launch_bounds__(fk_threads(Q1 + Q2, B), fk_threads(Q1 + Q2, B)
                 auto sub2 = [&](auto tt) {
                     using F = RegFFA<T, Q2>;
                     T a[R2][F::W];
-                    F::template load_rows<decltype(tt)::value>(bufB + k1 * R2 * WB + x0, WB, k1, a,
-                                                               std::make_index_sequence<R2>{});
+                    // trial k1 of group u2
+                    if constexpr (INPLACE)
+                        F::template load_rows<decltype(tt)::value>(bufA + k1 * WA + x0, R1 * WA, k1, a,
+                                                                   std::make_index_sequence<R2>{});
+                    else
+                        F::template load_rows<decltype(tt)::value>(bufB + k1 * R2 * WB + x0, WB, k1, a,
+                                                                   std::make_index_sequence<R2>{});
                     T out[R2][4];
                     F::run(a, out);
                     T* d = drow + (int64_t)(k1 * R2) * ld + x0;
@@ -462,8 +474,6 @@ __global__ void __launch_bounds__(fk_threads(Q1 + Q2, B), fk_threads(Q1 + Q2, B)
                 }
             }
         }
-        if (!more) break;
-        stage_finish(w.t);
     }
 }
 
@@ -491,22 +501,14 @@ template <class T, bool FIRST, int Q1, int Q2, int B>
 static ffa_status launch_k(const void* src, T* dst, FoldGroup& fg, int64_t m_rows, int s, cudaStream_t st) {
     constexpr int q = Q1 + Q2;
     constexpr int rows = 1 << q;
-    const size_t smem =
-        sizeof(T) * ((size_t)rows * fk_wa(q, Q1, B) + (Q2 > 0 ? (size_t)rows * fk_wb(q, Q1, B) : 0));
+    constexpr int wa = fk_wa(q, Q1, B), wb = fk_wb(q, Q1, B);
+    const size_t smem = sizeof(T) * (size_t)rows * (fk_inplace(Q1, Q2) ? fk_max(wa, wb) : wa + (Q2 > 0 ? wb : 0));
     ffa_status es = ensure_smem((const void*)k_fold<T, FIRST, Q1, Q2, B>, smem);
     if (es != FFA_OK) return es;
     const int64_t units = group_units(fg, m_rows, rows, B);
     if (units <= 0) return FFA_OK;
     if (units > INT32_MAX) return fail(FFA_ERR_UNSUPPORTED, "fold: plane too large for one launch");
-    constexpr int threads = fk_threads(q, B);
-    int64_t grid = units;
-    if (fk_persistent(q, FIRST && sizeof(typename FoldIn<T>::type) == 1)) {
-        int64_t resident = 0;
-        es = resident_ctas((const void*)k_fold<T, FIRST, Q1, Q2, B>, threads, smem, &resident);
-        if (es != FFA_OK) return es;
-        grid = units < resident ? units : resident;
-    }
-    k_fold<T, FIRST, Q1, Q2, B><<<(unsigned)grid, threads, smem, st>>>(src, dst, fg, s);
+    k_fold<T, FIRST, Q1, Q2, B><<<(unsigned)units, FK_THREADS, smem, st>>>(src, dst, fg, s);
     FFA_LAUNCH_CHECK("k_fold");
     count_launch();
     return FFA_OK;
