@@ -487,12 +487,16 @@ ffa_status ffa_plan_create(const ffa_search_config* cfg, int64_t n, ffa_plan** o
     off = align256(off + (cfg->precision == FFA_FOLD_F32 ? 4 : 1) * (size_t)n0);
     p->off_stats = off;
     off = align256(off + sizeof(double) * STATS_DOUBLES);
-    // planes: the largest base period, or a group of small ones
+    // planes: the largest base period, or a group of small ones (no more than
+    // all of them)
     p->plane_elems = std::max<int64_t>(p->max_plane, 1);
+    int64_t all = 0, widest = 0;
     for (const ffa_plan_entry& e : p->entries) {
-        const int64_t want = (int64_t)FOLD_GROUP_MAX * (int64_t)plane_slot(e);
-        p->plane_elems = std::max<int64_t>(p->plane_elems, std::min<int64_t>(want, GROUP_ELEMS));
+        all += (int64_t)plane_slot(e);
+        widest = std::max<int64_t>(widest, (int64_t)plane_slot(e));
     }
+    p->plane_elems = std::max<int64_t>(
+        p->plane_elems, std::min<int64_t>({(int64_t)FOLD_GROUP_MAX * widest, GROUP_ELEMS, all}));
     p->off_plane0 = off;
     off = align256(off + 4 * (size_t)p->plane_elems);
     p->off_plane1 = off;
@@ -879,14 +883,17 @@ ffa_status batch_layout(const ffa_plan* const* plans, int32_t count, BatchLayout
     }
     if (plans[0]->cfg.persistence) return fail(FFA_ERR_UNSUPPORTED, "batch: persistence plans are searched one by one");
     const size_t esz = plans[0]->cfg.precision == FFA_FOLD_F32 ? 4 : 1;
-    int64_t max_n0 = 1, max_slot = 1;
+    int64_t max_n0 = 1, max_slot = 1, all = 0;
     size_t off = 0;
     L->raw_off.resize((size_t)count);
     L->z_off.resize((size_t)count);
     for (int32_t i = 0; i < count; ++i) {
         const int64_t n0 = std::max<int64_t>(plans[i]->n0, 1);
         max_n0 = std::max(max_n0, n0);
-        for (const ffa_plan_entry& e : plans[i]->entries) max_slot = std::max<int64_t>(max_slot, (int64_t)plane_slot(e));
+        for (const ffa_plan_entry& e : plans[i]->entries) {
+            max_slot = std::max<int64_t>(max_slot, (int64_t)plane_slot(e));
+            all += (int64_t)plane_slot(e);
+        }
         L->raw_off[(size_t)i] = off;
         off = align256(off + sizeof(double) * (size_t)n0);
     }
@@ -900,7 +907,8 @@ ffa_status batch_layout(const ffa_plan* const* plans, int32_t count, BatchLayout
     off = align256(off + sizeof(double) * (size_t)max_n0);
     L->off_stats = off;
     off = align256(off + sizeof(double) * STATS_DOUBLES);
-    L->plane_elems = std::max<int64_t>(max_slot, std::min<int64_t>(BATCH_GROUP_ELEMS, (int64_t)FOLD_GROUP_MAX * max_slot));
+    L->plane_elems = std::max<int64_t>(
+        max_slot, std::min<int64_t>({BATCH_GROUP_ELEMS, (int64_t)FOLD_GROUP_MAX * max_slot, all}));
     L->off_plane0 = off;
     off = align256(off + 4 * (size_t)L->plane_elems);
     L->off_plane1 = off;
