@@ -41,8 +41,9 @@ void count_launch(int64_t n = 1);
 // 1 if the query fails).  Grid sizes are multiples of it.
 int sm_count();
 
-// Resident CTAs of a kernel for a dynamic shared-memory size, times the SM
-// count, per device: queried once (launches come per base period).
+// Resident CTAs of a kernel for a thread count and a dynamic shared-memory
+// size, times the SM count, per device: queried once (launches come per base
+// period).
 ffa_status resident_ctas(const void* fn, int threads, size_t smem, int64_t* out);
 
 // Raise a kernel's dynamic shared memory limit once per (kernel, device).

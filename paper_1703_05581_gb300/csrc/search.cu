@@ -55,14 +55,15 @@ int sm_count() {
     return n;
 }
 
-// Resident CTAs of a kernel for a dynamic shared-memory size, times the SM
-// count, per device: queried once (launches come per base period).
+// Resident CTAs of a kernel for a thread count and a dynamic shared-memory
+// size, times the SM count, per device: queried once (launches come per base
+// period).
 ffa_status resident_ctas(const void* fn, int threads, size_t smem, int64_t* out) {
     static std::mutex mu;
-    static std::map<std::tuple<const void*, size_t, int>, int64_t> cache;
+    static std::map<std::tuple<const void*, int, size_t, int>, int64_t> cache;
     int dev = 0;
     FFA_CUDA_TRY(cudaGetDevice(&dev));
-    const auto key = std::make_tuple(fn, smem, dev);
+    const auto key = std::make_tuple(fn, threads, smem, dev);
     {
         std::lock_guard<std::mutex> lk(mu);
         auto it = cache.find(key);
