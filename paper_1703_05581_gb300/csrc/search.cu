@@ -1117,7 +1117,8 @@ ffa_status ffa_wait(void* stream, const int32_t* d_status, int32_t timeout_ms) {
         if (e == cudaSuccess) break;
         if (e != cudaErrorNotReady) return cuda_fail(e, "wait: cudaStreamQuery");
         const auto us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
-        if (timeout_ms >= 0 && us > (int64_t)timeout_ms * 1000) return fail(FFA_ERR_TIMEOUT, "wait: stream did not finish in time");
+        // whole milliseconds: a limit of 0 still allows the first one
+        if (timeout_ms >= 0 && us / 1000 > timeout_ms) return fail(FFA_ERR_TIMEOUT, "wait: stream did not finish in time");
         // poll a short wait closely (a short search ends within a millisecond),
         // then sleep for a sixteenth of the time waited, at most 200 us
         if (us < 300) std::this_thread::yield();
