@@ -484,7 +484,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
                             "@q add.u32 %0, %0, 4;\n\t"
                             "@q min.u32 %0, %0, %6;\n\t}"
                             : "+r"(ptr), "+r"(below)
-                            : "f"(d), "f"(lo), "f"(hi), "f"(v), "r"(lim));
+                            : "f"(d), "f"(lo), "f"(hi), "f"(v), "r"(lim)
+                            : "memory");
                     };
                     for (int q = tid; q < nq; q += T) {
                         V v[4];
