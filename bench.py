@@ -57,8 +57,9 @@ PEAKS_PATH = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK_HBM_GBS = 6800.0
 METRIC = "FFA search rate (input samples*trials/s)"
 UNIT = "samples*trials/s"
-# groups of short base periods (fewer rows than this) are folded and scored together
-GROUP_TRIALS = 1024
+# base periods folded and scored together: at most this many, of this many plane elements
+GROUP_MAX = 64
+GROUP_ELEMS = 1 << 24
 
 
 def parse_args():
@@ -159,12 +160,43 @@ def score_ops(entries) -> np.ndarray:
     return e["m_rows"].astype(np.float64) * e["p0"] * (1.0 + 2.0 * e["n_widths"] + 3.0)
 
 
+def scorer_shape(p0: int, wmax: int) -> int:
+    """The scorers' block length class of a base period (the library's score_shape)."""
+    for i, (r, blocks, ext) in enumerate(((8, 256, 512), (16, 512, 1024), (16, 1024, 2048), (32, 1024, 2048))):
+        if (p0 + r - 1) // r <= blocks and (p0 + wmax + r) // r + 1 <= ext:
+            return i
+    return -1
+
+
+def group_starts(entries) -> np.ndarray:
+    """First base period of each group that a search folds and scores together
+    (the library's group_end): consecutive ones of one octave, row count,
+    floor(log2 P0), widths and scorer shape, up to GROUP_MAX of them and
+    GROUP_ELEMS plane elements; a larger one goes alone."""
+    e = entries
+    ints = {k: e[k].tolist() for k in ("octave", "m_rows", "p0", "n_widths")}
+    widths = [tuple(w[:k]) for w, k in zip(e["widths"].tolist(), ints["n_widths"])]
+    starts, key, elems, n = [], None, 0, 0
+    for i in range(len(e)):
+        p0 = ints["p0"][i]
+        k = (ints["octave"][i], ints["m_rows"][i], p0.bit_length(), widths[i], scorer_shape(p0, widths[i][-1]))
+        slot = (ints["m_rows"][i] * ((p0 + 3) // 4 * 4) + 63) // 64 * 64
+        if k != key or n == GROUP_MAX or elems + slot > GROUP_ELEMS:
+            starts.append(i)
+            key, elems, n = k, 0, 0
+        elems += slot
+        n += 1
+    return np.array(starts, np.int64)
+
+
 def sampled_singles(entries, octave, sample):
     """Base periods whose launches the library times one by one: every
     sample-th of the octave, when it is not folded in a group."""
+    starts = group_starts(entries)
+    alone = np.zeros(len(entries), bool)
+    alone[starts[np.diff(np.append(starts, len(entries))) == 1]] = True
     idx = np.flatnonzero(entries["octave"] == octave)[::sample]
-    sub = entries[idx]
-    return sub[sub["m_rows"] >= GROUP_TRIALS]
+    return entries[idx[alone[idx]]]
 
 
 def measured_peaks():
@@ -482,7 +514,7 @@ def run_gpu(args):
             xs.copy_(x_pinned, non_blocking=True)
         step()
         c, b = ffa.candidates(plan, rec, ws, snr_min=8.0, top_k=16, status=status, stream=stream)
-        d2h += 1064 + 24 * len(c)  # control block + candidate entries copied back
+        d2h += 4 + 16 + 24 * 16  # the status word, then the head and top_k candidates in one copy
     torch.cuda.synchronize(dev)
     e2e_s = time.perf_counter() - t0
     te = torch.tensor([e2e_s], dtype=torch.float64, device=dev)
@@ -502,7 +534,9 @@ def run_gpu(args):
             if phase_cnt[3][o] == 0:
                 continue
             sub = sampled_singles(plan.entries, o, ffa.TIMING_SAMPLE)
-            reps = phase_cnt[3][o] / max(len(sub), 1)  # timed steps
+            reps = args.steps
+            if phase_cnt[3][o] != len(sub) * reps:
+                raise RuntimeError(f"octave {o}: {phase_cnt[3][o]} timed launches, {len(sub)} base periods x {reps} steps")
             b_s += float(entry_bytes(sub).sum()) * reps
             ops += float(score_ops(sub).sum()) * reps
             bins += float((sub["m_rows"].astype(np.float64) * sub["p0"]).sum()) * reps

@@ -9,12 +9,13 @@
 #include <string.h>
 #include <time.h>
 
+#define MAXL (1 << 19)
 typedef struct { unsigned x, y, z; } dim3_t;
 typedef struct { char name[256]; unsigned grid, block; uint64_t smem; } launch_t;
 
 static struct { const void* host; char name[256]; } g_fn[512];
 static int g_nfn;
-static launch_t g_launch[65536];
+static launch_t g_launch[MAXL];
 static int g_nlaunch;
 static double g_ready_s;   /* the stream is busy until this monotonic time */
 static float g_elapsed_ms = 1.0f;
@@ -66,7 +67,7 @@ int __cudaGetKernel(void** k, const void* host) { *k = (void*)host; return 0; }
 int cudaLaunchKernel(const void* fn, dim3_t g, dim3_t b, void** args, size_t smem, void* st) {
     (void)args;
     (void)st;
-    if (g_nlaunch < 65536) {
+    if (g_nlaunch < MAXL) {
         launch_t* l = &g_launch[g_nlaunch++];
         strcpy(l->name, "?");
         for (int i = 0; i < g_nfn; ++i)
