@@ -579,13 +579,13 @@ static ffa_status fold_impl(const void* d_z, FoldGroup& fg, int64_t m_rows, int 
 // ---------------------------------------------------------------------------
 // Stages per pass and tile width, tuned.  Any split of the stages into passes,
 // and any tile width, gives the same add tree (bit-identical planes); only the
-// time differs.  The cache maps (device, precision, stages, floor(log2 p0)) to
-// the fastest shape measured by tune_fold; untuned shapes use six stages per
-// pass with the default widths.
+// time differs.  The cache maps (device, precision, stages, floor(log2 p0),
+// rows on 16-byte boundaries) to the fastest shape measured by tune_fold;
+// untuned shapes use six stages per pass with the default widths.
 // ---------------------------------------------------------------------------
 namespace {
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int>, FoldShape> g_tune;
+std::map<std::tuple<int, int, int, int, bool>, FoldShape> g_tune;
 constexpr FoldShape SHAPE_DEFAULT = {6, 0};
 
 int log2i(int64_t v) {
@@ -603,7 +603,7 @@ FoldShape tuned_shape(int precision, int stages, int64_t p0, int64_t ld) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return none;
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tune.find(std::make_tuple(dev, precision, stages, log2i(p0)));
+    auto it = g_tune.find(std::make_tuple(dev, precision, stages, log2i(p0), (ld & 3) == 0));
     return it == g_tune.end() ? none : it->second;
 }
 }  // namespace
@@ -666,7 +666,7 @@ ffa_status tune_fold(const void* d_z, int32_t precision, int64_t p0, int64_t m_d
     FFA_CUDA_TRY(cudaGetDevice(&dev));
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune[std::make_tuple(dev, precision, stages, log2i(p0))] = bs;
+        g_tune[std::make_tuple(dev, precision, stages, log2i(p0), (ld & 3) == 0)] = bs;
     }
     if (best_q) *best_q = bs.qmax * 1000 + bs.tile;
     return FFA_OK;

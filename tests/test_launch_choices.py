@@ -21,3 +21,24 @@ def ctas(kernel, threads, smem):
 emit([ctas(64, t, 20000) for t in (1024, 256, 1024)] + [ctas(128, t, 20000) for t in (256, 1024)])
 """)
     assert got == [2 * 152, 8 * 152, 2 * 152, 8 * 152, 2 * 152]
+
+
+def test_tuned_shape_of_padded_rows_only(fake):
+    """The autotuner times a search's padded planes: a fold of dense rows that
+    are not 16-byte aligned keeps the passes it had."""
+    got = fakecuda.run(fake, """
+def passes(p0):
+    fake.fake_reset()
+    assert lib.ffa_fold(BUF, 0, C.c_int64(p0), C.c_int64(4000), C.c_int64(4096), BUF, BUF, None) == 0
+    return sum("k_fold" in x[0] for x in launches())
+before = [passes(9001), passes(9004)]
+ts = 64e-6
+h = plan(config(tsamp_s=ts, period_min_s=9000 * ts, period_max_s=9010 * ts, detrend_window=-1), 9000 * 8000)
+ws, n = C.c_size_t(), C.c_int32()
+lib.ffa_plan_info(h, None, None, None, None, C.byref(ws))
+assert lib.ffa_autotune(h, BUF, ws, None, C.byref(n)) == 0 and n.value == 1
+emit([before, [passes(9001), passes(9004)]])
+""")
+    before, after = got
+    assert after[0] == before[0]
+    assert before[1] == 2 and after[1] == 4  # tuned to three stages a pass: every shape takes as long here
