@@ -41,9 +41,7 @@
 #include <math.h>
 #include <stdint.h>
 
-#include <map>
-#include <mutex>
-#include <tuple>
+#include <algorithm>
 #include <type_traits>
 
 #include "score.cuh"
@@ -932,8 +930,23 @@ ffa_status score1_t(const void* d_prof, const ScoreGroup& sg, int64_t count, int
     // against registers.  Fewer threads that hold their item in registers
     // beat more threads that spill (20000 bins: 27.7k SM cycles a profile
     // with 448 threads of 72 registers, 35.7k with 640 of 48).
+    //
+    // Few profiles: when no SM gets more than a few CTAs the call takes one
+    // profile's latency, not its share of the SM, so a profile gets the
+    // threads that its items and the SM's registers allow (records do not
+    // depend on it).  `each`: CTAs of the busiest SM.
+    const int64_t each = (count + sm_count() - 1) / sm_count();
     switch (shape) {
-        case 0:
+        case 0: {
+            // Six bins a thread, 768 threads an SM: 150 profiles of 1100 bins
+            // take 9.3 us (one warp each: 13.1), of 700 9.0 (11.2); 800 of
+            // 1100 12 (14.8).  From seven an SM on the shapes below are as
+            // fast (1500 of 1100: 15).
+            const int64_t few = each <= 6 ? std::min<int64_t>({256, (p0 / 6 + 31) & ~31, (768 / each) & ~31}) : 0;
+            if (few >= 64) {
+                score1_shape<V, 8>(p0, wtop, 1, (int)few, (int)few, 10, &threads, &lay, &smem);
+                return FFA_SCORE1(8, false, 256, 4);
+            }
             // One warp a profile up to 1200 bins (1100 bins: 2.3k SM cycles,
             // 2.8k with two warps; 366 bins: 1.25k and 2.2k); above, two for
             // ready profiles (1489 bins: 2.8k, 3.0k with one), one in a search
@@ -944,14 +957,27 @@ ffa_status score1_t(const void* d_prof, const ScoreGroup& sg, int64_t count, int
             }
             score1_shape<V, 8>(p0, wtop, 3, 64, 64, 9, &threads, &lay, &smem);
             return FFA_SCORE1(8, false, 64, 12);
+        }
         case 1:
-        case 2:
+        case 2: {
             score1_shape<V, 16>(p0, wtop, p0 <= 10240 ? 3 : 2, 64, 384, 9, &threads, &lay, &smem);
+            // One item a thread, 512 threads of 128 registers an SM: 150
+            // profiles of 3001 bins take 10.6 us (64 threads: 16.4), of 9001
+            // 13.6 (16.1, 192 threads), 300 of 4201 12.3 (17.5), 500 14.5
+            // of 3001 (20.6).
+            const int64_t few = each <= 4 ? std::min<int64_t>(((p0 + 15) / 16 + 63) & ~63, (512 / each) & ~31) : 0;
+            if (few > threads) {
+                score1_shape<V, 16>(p0, wtop, 1, (int)few, (int)few, 9, &threads, &lay, &smem);
+                return FFA_SCORE1(16, false, 512, 1);
+            }
             return FFA_SCORE1(16, false, 384, 2);
+        }
         default:
-            // two profiles an SM while their shared memory fits, else one
+            // two profiles an SM while their shared memory fits, else one (or
+            // if no SM gets a second: 150 of 20000 bins 21.7 us, 26.2 with
+            // the two's threads)
             score1_shape<V, 32>(p0, wtop, 3, 320, 448, 7, &threads, &lay, &smem);
-            if (2 * (smem + sizeof(S1Sh) + 1024) <= 228 * 1024) return FFA_SCORE1(32, false, 448, 2);
+            if (each > 1 && 2 * (smem + sizeof(S1Sh) + 1024) <= 228 * 1024) return FFA_SCORE1(32, false, 448, 2);
             // (threads of the one, 4096 x 29705: float 618 us with 640, 631
             // with 768; int 692 and 678)
             if (std::is_integral<V>::value) {

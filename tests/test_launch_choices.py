@@ -42,3 +42,31 @@ emit([before, [passes(9001), passes(9004)]])
     before, after = got
     assert after[0] == before[0]
     assert before[1] == 2 and after[1] == 4  # tuned to three stages a pass: every shape takes as long here
+
+
+def test_few_profiles_get_more_threads(fake):
+    """A scoring call that leaves each SM a few profiles takes the latency of
+    one: it gets more threads a profile than a call that fills the GPU, and
+    no more than the SM holds."""
+    got = fakecuda.run(fake, """
+out = {}
+for prec in (0, 1):
+    for p0 in (64, 700, 1100, 1489, 2048, 2049, 3001, 6000, 9001, 16000, 20000, 30001):
+        for n in (1, 152, 153, 304, 500, 900, 8000):
+            fake.fake_reset()
+            w = (C.c_int32 * 3)(1, 2, 4)
+            assert lib.ffa_score(BUF, prec, C.c_int64(n), C.c_int64(p0), w, 3, BUF, BUF, None) == 0
+            (name, grid, block, smem), = launches()
+            out["%d %d %d" % (prec, p0, n)] = (grid, block, smem)
+emit(out)
+""")
+    for key, (grid, block, smem) in got.items():
+        prec, p0, n = map(int, key.split())
+        full = got[f"{prec} {p0} 8000"][1]
+        each = -(-n // 152)
+        assert block % 32 == 0 and grid <= n
+        assert block >= full or each == 1  # (one profile an SM above 16384 bins takes the lone CTA's shape)
+        if each <= 6 and block > full:
+            assert grid == n and each * block <= (768 if p0 <= 2048 else 1024)
+        if p0 in (700, 1100, 2048, 3001, 9001) and each == 1:
+            assert block > full
