@@ -17,8 +17,10 @@
 // interpolated pivots), otherwise the window is moved and the pass repeated,
 // and after a few attempts an exact radix select over the profile takes over.
 // A window's bounds are monotone functions of the value, so the counts are
-// exact whatever the prediction was.  Int profiles need no list: their
-// window holds one bucket per integer.
+// exact whatever the prediction was.  Float profiles with gaps or many equal
+// values, whose windows hold no sample or too many, go on with pivots that are
+// samples themselves.  Int profiles need no list: their window holds one bucket
+// per integer.
 //
 // Box sums.  With the in-block exclusive prefix c_b[o] (blocks of R bins, the
 // cyclic extension included) and the block offsets C[b] = sum of earlier
@@ -73,7 +75,7 @@ struct S1Sh {
     unsigned long long key[2];
     float fa[32], fb[32], fc[32];
     uint2 wc[2][32];          // per-warp counts of a window pass (two slots, alternating)
-    float2 seg[SCORE_MAXSEG]; // segment totals of the offset scan
+    alignas(16) float2 seg[SCORE_MAXSEG];  // segment totals of the offset scan
     uint32_t wkey[16];        // per-width maxima as order-preserving keys
     uint32_t npack;
     int bin_a, bin_b;
@@ -172,6 +174,159 @@ __device__ __noinline__ unsigned long long radix_rank(const unsigned char* smem,
     }
     cta_sync<ONE>();
     return prefix;
+}
+
+__device__ __forceinline__ unsigned long long warp_extreme(unsigned long long k, bool largest) {
+    uint32_t h = (uint32_t)(k >> 32), l = (uint32_t)k;
+    const uint32_t top = largest ? __reduce_max_sync(0xffffffffu, h) : __reduce_min_sync(0xffffffffu, h);
+    if (h != top) l = largest ? 0u : ~0u;
+    l = largest ? __reduce_max_sync(0xffffffffu, l) : __reduce_min_sync(0xffffffffu, l);
+    return ((unsigned long long)top << 32) | l;
+}
+
+// The keys of the two middle ranks of a whole float profile (MAD: of its
+// deviations from mh + ml), for profiles with few distinct values or gaps,
+// where a window holds no sample or too many.  A pass counts the samples below
+// and up to a pivot and finds its neighbours on both sides; the next pivot is
+// the neighbour on the wanted side, then a value interpolated inside the
+// bounds -- two or three passes settle a profile of few levels, which a radix
+// select takes eight or sixteen for (3000 profiles of 1100 bins and 16 levels:
+// 49 us, 144 with windows and a radix select only; 150 of 64 bins and 2 levels:
+// 7.4 and 32).  False if the ranks were not found.
+template <int R, bool ONE, bool MAD>
+__device__ __forceinline__ bool member_ranks(const unsigned char* smem, S1Sh& sh, int p0, float mh, float ml,
+                                             float guess, float sig, unsigned long long& ka,
+                                             unsigned long long& kb) {
+    const uint32_t r1 = (uint32_t)((p0 - 1) / 2), r2 = (uint32_t)(p0 / 2);
+    const int T = ONE ? 32 : (int)blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = T >> 5;
+    uint4* part = reinterpret_cast<uint4*>(sh.seg);  // a warp's neighbours
+    unsigned long long lo = 0, hi = ~0ull;           // the wanted keys are in [lo, hi]
+    uint32_t cl = 0, ch = (uint32_t)p0;              // keys below lo, up to hi
+    unsigned long long p = ff_key(guess, 0.0f);
+    bool member = false;
+    auto found = [&](unsigned long long a, unsigned long long b) {
+        ka = a;
+        kb = b;
+        return true;
+    };
+    auto value = [](unsigned long long k) { return fkey_inv((uint32_t)(k >> 32)); };
+    for (int a = 0; a < 12; ++a) {
+        uint32_t lt = 0, le = 0;
+        unsigned long long dn = 0, up = ~0ull;
+        for (int j = tid; j < p0; j += T) {
+            float h = load_bin<float, R>(smem, j), l = 0.0f;
+            if (MAD) ff_dev(h, mh, ml, h, l);
+            const unsigned long long k = ff_key(h, l);
+            lt += k < p;
+            le += k <= p;
+            if (k < p && k > dn) dn = k;
+            if (k > p && k < up) up = k;
+        }
+        lt = __reduce_add_sync(0xffffffffu, lt);
+        le = __reduce_add_sync(0xffffffffu, le);
+        dn = warp_extreme(dn, true);
+        up = warp_extreme(up, false);
+        if (!ONE) {
+            if (lane == 0) {
+                sh.wc[0][warp] = make_uint2(lt, le);
+                part[warp] = make_uint4((uint32_t)(dn >> 32), (uint32_t)dn, (uint32_t)(up >> 32), (uint32_t)up);
+            }
+            __syncthreads();
+            uint2 c = make_uint2(0u, 0u);
+            uint4 n = make_uint4(0u, 0u, ~0u, ~0u);
+            if (lane < NW) {
+                c = sh.wc[0][lane];
+                n = part[lane];
+            }
+            __syncthreads();
+            lt = __reduce_add_sync(0xffffffffu, c.x);
+            le = __reduce_add_sync(0xffffffffu, c.y);
+            dn = warp_extreme(((unsigned long long)n.x << 32) | n.y, true);
+            up = warp_extreme(((unsigned long long)n.z << 32) | n.w, false);
+        }
+        if (r1 < lt) {
+            if (r2 >= lt) return found(dn, le > lt ? p : up);
+            if (r1 == lt - 1) return found(dn, dn);
+            hi = dn;
+            ch = lt;
+        } else if (r1 < le) {
+            return found(p, r2 < le ? p : up);
+        } else {
+            if (r1 == le && r2 == r1) return found(up, up);
+            lo = up;
+            cl = le;
+        }
+        const bool down = r1 < lt;
+        if (member) {
+            float x;
+            if (lo != 0 && hi != ~0ull)
+                x = fmaf((float)(2 * (r1 - cl) + 1) / (float)(2 * (ch - cl)), value(hi) - value(lo), value(lo));
+            else {
+                // about the ranks' distance near a normal median
+                const float step = sig / (0.3f * (float)p0);
+                x = down ? value(dn) - step * (float)(lt - r1) : value(up) + step * (float)(r1 + 1 - le);
+            }
+            p = ff_key(x, 0.0f);
+            member = !(p > lo && p < hi);
+            if (member) p = down ? dn : up;
+        } else {
+            p = down ? dn : up;
+            member = true;
+        }
+    }
+    return false;
+}
+
+// The median's and the MAD's float pairs from their two middle ranks' keys
+// (the median (a + b) / 2 exactly).
+__device__ __forceinline__ void pair_median(unsigned long long ka, unsigned long long kb, bool two, float& h, float& l) {
+    const float a = fkey_inv((uint32_t)(ka >> 32)), b = fkey_inv((uint32_t)(kb >> 32));
+    h = a;
+    l = 0.0f;
+    if (two) {
+        two_sum(a, b, h, l);
+        h *= 0.5f;
+        l *= 0.5f;
+    }
+}
+__device__ __forceinline__ void pair_mad(unsigned long long ka, unsigned long long kb, bool two, float& h, float& l) {
+    h = fkey_inv((uint32_t)(ka >> 32));
+    l = fkey_inv((uint32_t)ka);
+    if (two) {
+        ff_acc(h, l, fkey_inv((uint32_t)(kb >> 32)), fkey_inv((uint32_t)kb));
+        ff_norm(h, l);
+        h *= 0.5f;
+        l *= 0.5f;
+    }
+}
+
+// Median and MAD of any float profile, as the pairs sh.fa[0..1] and
+// sh.fa[2..3]: by pivots if the profile has a spread (sig; 0: none, or not
+// finite), else, and where they fail, by a radix select.  One call for all of
+// it: the scorer keeps its registers.
+template <int R, bool ONE>
+__device__ __noinline__ void profile_ranks(const unsigned char* smem, uint32_t* hist, S1Sh& sh, int p0, float mean,
+                                           float sig) {
+    const uint32_t r1 = (uint32_t)((p0 - 1) / 2), r2 = (uint32_t)(p0 / 2);
+    float mh = 0.0f, ml = 0.0f, kh, kl;
+    unsigned long long ka, kb;
+    if (!(sig > 0.0f && member_ranks<R, ONE, false>(smem, sh, p0, mh, ml, mean, sig, ka, kb))) {
+        ka = radix_rank<float, R, ONE, false>(smem, hist, sh, p0, r1, mh, ml, 0);
+        kb = r1 == r2 ? ka : radix_rank<float, R, ONE, false>(smem, hist, sh, p0, r2, mh, ml, 0);
+    }
+    pair_median(ka, kb, r1 != r2, mh, ml);
+    if (!(sig > 0.0f && member_ranks<R, ONE, true>(smem, sh, p0, mh, ml, 0.6745f * sig, sig, ka, kb))) {
+        ka = radix_rank<float, R, ONE, true>(smem, hist, sh, p0, r1, mh, ml, 0);
+        kb = r1 == r2 ? ka : radix_rank<float, R, ONE, true>(smem, hist, sh, p0, r2, mh, ml, 0);
+    }
+    pair_mad(ka, kb, r1 != r2, kh, kl);
+    if (threadIdx.x == 0) {
+        sh.fa[0] = mh;
+        sh.fa[1] = ml;
+        sh.fa[2] = kh;
+        sh.fa[3] = kl;
+    }
+    cta_sync<ONE>();
 }
 
 // One warp: the values of ranks t1 <= t2 <= t1 + 1 among the n <= 128 KQ
@@ -458,7 +613,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
         const uint32_t r1 = (uint32_t)((p0 - 1) / 2), r2 = (uint32_t)(p0 / 2);
         // quads entirely inside groups of 32 bins need no bound check
         const int nq = (p0 >> 5) << 3, jt = (p0 & ~31) + tid;
-        bool spread = !redo && sig > 0.0f && sig < 1e30f;  // windows make sense (block-uniform)
+        bool spread = sig > 0.0f && sig < 1e30f;  // a prediction makes sense (block-uniform)
         if (INT) spread = spread && fm < 5e8f;    // 2 |x| and window sums stay in int32
         if constexpr (!INT) {
             mh = ml = 0.0f;
@@ -505,10 +660,17 @@ __global__ void __launch_bounds__(MAXT, MINB)
                         if (tid == 0) sh.npack = 0;
                         r *= 0.5f;
                         sync();
+                        // (one thread's list overflows in every few normal
+                        // profiles; lists half full: equal values, once more)
+                        if (2 * c.y > (uint32_t)(T * (lay.cap - 1))) a += 2;
                         continue;
                     }
+                    if (c.y == 0) {  // a gap
+                        sync();
+                        return false;
+                    }
                     if (r1 < cl || r2 >= cl + c.y) {
-                        const float dens = fmaxf((float)c.y, 1.0f) / (2.0f * r);
+                        const float dens = (float)c.y / (2.0f * r);
                         if (r1 < cl) g -= r + (float)(cl - r1) / dens;
                         else g += r + (float)(r2 + 1 - cl - c.y) / dens;
                         r *= 1.5f;
@@ -589,44 +751,27 @@ __global__ void __launch_bounds__(MAXT, MINB)
             };
             unsigned long long ka = 0, kb = 0;
             bool done = false;
-            if (spread) done = select(std::false_type{}, fmaf(hint_med, sig, mean), 3.2f * rsn, ka, kb);
-            if (!done) {
-                ka = radix_rank<V, R, ONE, false>(smem, hist, sh, p0, r1, 0.0f, 0.0f, 0);
-                kb = r1 == r2 ? ka : radix_rank<V, R, ONE, false>(smem, hist, sh, p0, r2, 0.0f, 0.0f, 0);
-            }
-            // the median as a float pair: (a + b) / 2 exactly
-            {
-                const float a = fkey_inv((uint32_t)(ka >> 32)), b = fkey_inv((uint32_t)(kb >> 32));
-                if (r1 == r2) {
-                    mh = a;
-                } else {
-                    two_sum(a, b, mh, ml);
-                    mh *= 0.5f;
-                    ml *= 0.5f;
+            if (spread && !redo && select(std::false_type{}, fmaf(hint_med, sig, mean), 3.2f * rsn, ka, kb)) {
+                pair_median(ka, kb, r1 != r2, mh, ml);
+                if (!extended) {  // read after the barriers of the MAD's selection
+                    extend(tid, T);
+                    extended = true;
                 }
-            }
-            if (!extended) {  // read after the barriers of the MAD's selection
-                extend(tid, T);
-                extended = true;
-            }
-            done = false;
-            if (spread) done = select(std::true_type{}, hint_mad * sig, 2.6f * rsn, ka, kb);
-            if (!done && prefixed) {  // the profile is gone: once more
-                prefixed = false;
-                sync();
-                continue;
+                done = select(std::true_type{}, hint_mad * sig, 2.6f * rsn, ka, kb);
+                if (!done && prefixed) {  // the profile is gone: once more
+                    prefixed = false;
+                    sync();
+                    continue;
+                }
+                pair_mad(ka, kb, r1 != r2, kmh, kml);
             }
             if (!done) {
-                ka = radix_rank<V, R, ONE, true>(smem, hist, sh, p0, r1, mh, ml, 0);
-                kb = r1 == r2 ? ka : radix_rank<V, R, ONE, true>(smem, hist, sh, p0, r2, mh, ml, 0);
-            }
-            kmh = fkey_inv((uint32_t)(ka >> 32));
-            kml = fkey_inv((uint32_t)ka);
-            if (r1 != r2) {
-                ff_acc(kmh, kml, fkey_inv((uint32_t)(kb >> 32)), fkey_inv((uint32_t)kb));
-                ff_norm(kmh, kml);
-                kmh *= 0.5f;
-                kml *= 0.5f;
+                profile_ranks<R, ONE>(smem, hist, sh, p0, mean, spread ? sig : 0.0f);
+                mh = sh.fa[0];
+                ml = sh.fa[1];
+                kmh = sh.fa[2];
+                kml = sh.fa[3];
+                if (!extended) extend(tid, T);
             }
             if (spread) {
                 const float is = 1.0f / sig;
@@ -951,12 +1096,15 @@ ffa_status score1_t(const void* d_prof, const ScoreGroup& sg, int64_t count, int
             // 2.8k with two warps; 366 bins: 1.25k and 2.2k); above, two for
             // ready profiles (1489 bins: 2.8k, 3.0k with one), one in a search
             // (12 DM trials: 278 ms, 291 ms with two).
-            if (p0 <= 1200 || FF) {
-                score1_shape<V, 8>(p0, wtop, 1, 32, 32, 13, &threads, &lay, &smem);
-                return FFA_SCORE1(8, true, 32, 24);
+            if constexpr (!FF) {
+                if (p0 > 1200) {
+                    score1_shape<V, 8>(p0, wtop, 3, 64, 64, 9, &threads, &lay, &smem);
+                    return FFA_SCORE1(8, false, 64, 12);
+                }
             }
-            score1_shape<V, 8>(p0, wtop, 3, 64, 64, 9, &threads, &lay, &smem);
-            return FFA_SCORE1(8, false, 64, 12);
+            // (80 registers fit 25 CTAs; a bound of 24 spills)
+            score1_shape<V, 8>(p0, wtop, 1, 32, 32, 13, &threads, &lay, &smem);
+            return FFA_SCORE1(8, true, 32, 22);
         }
         case 1:
         case 2: {
@@ -980,12 +1128,13 @@ ffa_status score1_t(const void* d_prof, const ScoreGroup& sg, int64_t count, int
             if (each > 1 && 2 * (smem + sizeof(S1Sh) + 1024) <= 228 * 1024) return FFA_SCORE1(32, false, 448, 2);
             // (threads of the one, 4096 x 29705: float 618 us with 640, 631
             // with 768; int 692 and 678)
-            if (std::is_integral<V>::value) {
+            if constexpr (std::is_integral<V>::value) {
                 score1_shape<V, 32>(p0, wtop, 2, 512, 768, 9, &threads, &lay, &smem);
                 return FFA_SCORE1(32, false, 768, 1);
+            } else {
+                score1_shape<V, 32>(p0, wtop, 3, 512, 640, 9, &threads, &lay, &smem);
+                return FFA_SCORE1(32, false, 640, 1);
             }
-            score1_shape<V, 32>(p0, wtop, 3, 512, 640, 9, &threads, &lay, &smem);
-            return FFA_SCORE1(32, false, 640, 1);
     }
 #undef FFA_SCORE1
 }
