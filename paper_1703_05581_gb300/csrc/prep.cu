@@ -792,11 +792,22 @@ ffa_status launch_detrend(const double* d_raw, int64_t n, int32_t window, double
     size_t smem = sizeof(RmShared);
     ffa_status es = ensure_smem((const void*)k_runmed_tile, smem);
     if (es != FFA_OK) return es;
-    const int threads = T > 32 ? T / 2 : 32;
     const int64_t tiles = (n + T - 1) / T;
-    // persistent: consecutive tiles in one CTA predict each other's bracket
+    // Shared memory fits three CTAs an SM whatever their threads: 512, or 256
+    // for short tiles when every CTA takes many of them (barriers then count
+    // for more than the samples).  Windows of 129 / 257 / 1025 samples: 2^22
+    // samples 2.9 / 1.6 / 0.56 ms (6.1 / 3.5 / 0.67 with half a thread an
+    // output, 3.2 / 1.7 / 0.60 with 512), 2^14 samples 43 / 22 / 20 us (129 / 70
+    // / 27, and 50 / 26 / 20 with 256).
+    // Persistent: consecutive tiles in one CTA predict each other's bracket.
+    auto fn = (const void*)k_runmed_tile;
+    int threads = RM_NT;
     int64_t grid = 0;
-    es = resident_ctas((const void*)k_runmed_tile, threads, smem, &grid);
+    es = resident_ctas(fn, threads, smem, &grid);
+    if (es == FFA_OK && T <= 256 && tiles > 8 * grid) {
+        threads = 256;
+        es = resident_ctas(fn, threads, smem, &grid);
+    }
     if (es != FFA_OK) return es;
     if (grid > tiles) grid = tiles;
     // runs of at most 16 tiles, as many for every CTA: 456 CTAs' runs of 1024

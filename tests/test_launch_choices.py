@@ -70,3 +70,25 @@ emit(out)
             assert grid == n and each * block <= (768 if p0 <= 2048 else 1024)
         if p0 in (700, 1100, 2048, 3001, 9001) and each == 1:
             assert block > full
+
+
+def test_running_median_threads(fake):
+    """A CTA of the running median has at least the threads of its tile's
+    outputs: shared memory bounds how many CTAs an SM holds, so a small CTA
+    leaves the SM idle."""
+    got = fakecuda.run(fake, """
+out = []
+for n in (1 << 14, 1 << 17, 1 << 22):
+    for w in (129, 257, 1025, 4001, 62501):
+        fake.fake_reset()
+        assert lib.ffa_detrend(BUF, C.c_int64(n), C.c_int32(w), BUF, BUF, None) == 0
+        (name, grid, block, smem), = launches()
+        out.append([n, w, block])
+emit(out)
+""")
+    for n, w, block in got:
+        tile = 32
+        while 2 * tile <= min(1024, (w + 1) // 4):
+            tile *= 2
+        assert block >= min(tile, 512)
+        assert block in (256, 512) and (n > 1 << 14 or block == 512)
