@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -37,29 +38,31 @@
 namespace ffa {
 
 
-// Base periods folded by one launch: entry i has p0[i] bins, m_data[i] data
-// rows (all share m_rows), its plane at element offset off[i] of the plane
-// buffers with row pitch ld[i] (>= p0[i]; a multiple of 4 makes every row
-// 16-byte aligned), and owns the launch's CTAs [unit0[i], unit0[i + 1]).  A
-// single base period is a group of one.  The first pass reads the series
-// itself: row g of entry i is src[i][g * p0[i] ...], densely packed (entries
-// of a batch read their own series).
-struct FoldGroup {
+// Base periods folded by one launch: an entry has p0 bins, m_data data rows
+// (all share m_rows), its plane at element offset `off` of the plane buffers
+// with row pitch ld (>= p0; a multiple of 4 makes every row 16-byte aligned),
+// its rows cut into n_ct column tiles, and owns the launch's CTAs from unit0 to
+// the next entry's.  A single base period is a group of one.  The first pass
+// reads the series itself: row g of an entry is src[g * p0 ...], densely
+// packed (entries of a batch read their own series).  An entry's fields lie
+// together: a CTA starts with one or two lines of kernel parameters.
+struct FoldEntry {
+    const void* src;
+    int64_t p0, m_data, off, ld;
+    uint32_t unit0;
+    int32_t n_ct;
+};
+struct alignas(64) FoldGroup {
+    FoldEntry e[FOLD_GROUP_MAX];
     int32_t n;
-    const void* src[FOLD_GROUP_MAX];
-    int64_t p0[FOLD_GROUP_MAX];
-    int64_t m_data[FOLD_GROUP_MAX];
-    int64_t off[FOLD_GROUP_MAX];
-    int64_t ld[FOLD_GROUP_MAX];
-    int64_t unit0[FOLD_GROUP_MAX + 1];
 };
 
-// this CTA's entry and its unit within the entry
-__device__ __forceinline__ int group_entry(const FoldGroup& g, int64_t unit) {
-    int lo = 0, hi = g.n - 1;
+// this CTA's entry
+__device__ __forceinline__ int group_entry(const FoldGroup& g, int n, uint32_t unit) {
+    int lo = 0, hi = n - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
-        if (g.unit0[mid] <= unit) lo = mid;
+        if (g.e[mid].unit0 <= unit) lo = mid;
         else hi = mid - 1;
     }
     return lo;
@@ -162,15 +165,16 @@ __device__ __forceinline__ int as_bits(T v) {
 }
 
 // Four consecutive outputs to global memory: one 128-bit store when the row
-// is 16-byte aligned (vec), else element stores up to `left` columns.
+// is 16-byte aligned (vec; what lies behind its end is padding), else element
+// stores of columns [skip, left).
 template <class T>
-__device__ __forceinline__ void store4(T* d, const T (&v)[4], int left, bool vec) {
+__device__ __forceinline__ void store4(T* d, const T (&v)[4], int left, bool vec, int skip = 0) {
     if (vec) {
         *reinterpret_cast<int4*>(d) = make_int4(as_bits(v[0]), as_bits(v[1]), as_bits(v[2]), as_bits(v[3]));
     } else {
 #pragma unroll
         for (int x = 0; x < 4; ++x)
-            if (x < left) d[x] = v[x];
+            if (x >= skip && x < left) d[x] = v[x];
     }
 }
 
@@ -215,13 +219,18 @@ __device__ __forceinline__ void store_row(T* d, const T (&v)[4], int off) {
 // pitch).  Tiles are B = 256 columns up to 5 stages and 128 for 6 (64 rows).
 //
 // Alignment.  The staging copies are 16 bytes wide, so a row's columns keep
-// the misalignment 0..3 of their address.  It is (t * u) & 3 in row u for one
-// t per CTA -- the rows of the first pass are p0 elements apart (t = p0 & 3),
-// row u of a later pass starts kappa * u columns on (t = kappa & 3) -- and so
-// is the offset k1*u2 of sub-pass 2 (t = k1 & 3, one per warp): both
-// sub-passes are compiled for each t, with every row's offset known, and need
-// no select on it.  Rows off that pattern (they wrapped past p0, or the plane
-// is not 16-byte aligned) are staged element by element onto it.
+// the misalignment 0..3 of their address.  It is (t0 + t * u) & 3 in row u for
+// one t0 and t per CTA -- the rows of the first pass are p0 elements apart (t =
+// p0 & 3), row u of a later pass is (ld << s) elements on and starts kappa * u
+// columns on (t = (kappa + (ld << s)) & 3) -- and so is the offset k1*u2 of
+// sub-pass 2 (t = k1 & 3, one per warp).  The tile starts t0 columns early, so
+// that t0 is 0, and both sub-passes are compiled for each t, with every row's
+// offset known, and need no select on it.  Rows off that pattern (they wrapped
+// past p0) are staged element by element onto it.  t0 is 0 on padded planes;
+// on dense ones it is kappa * p0: without the early start three in four tiles
+// of the later passes were staged by elements (256 x 2001: 8.3 us, 7.2; 4096 x
+// 19977: 424 us, 380).  ALIGNED kernels, of planes where t0 is 0 and every row
+// starts on such a boundary, leave all of it out.
 //
 // What bounds it.  4096 rows of 19977 bins: the six-stage first pass takes
 // 150 us at 38 thread-instructions an element, its shared memory 73 % busy
@@ -230,6 +239,10 @@ __device__ __forceinline__ void store_row(T* d, const T (&v)[4], int off) {
 // traffic (142 us before).
 // ---------------------------------------------------------------------------
 constexpr int FK_THREADS = 256;
+// quads: rows off a boundary of four elements are stored as whole quads
+// (store_row).  That code and the variants of sub-pass 2 do not fit the
+// instruction cache of a short launch: it pays from about a CTA an SM on
+// (32 x 2001: 5.7 us with it, 5.2 without).
 // Six stages (3 + 3): sub-pass 1 works in place, a warp on each of the eight
 // groups, so one buffer of 64 rows (50 KB) serves both sub-passes and four
 // CTAs fit an SM, where two buffers left room for two: 4096 x 19977, first
@@ -250,9 +263,9 @@ __host__ __device__ constexpr int fk_wb(int q, int q1, int b) {
                                               4 * ((4 + (1 << (q - q1)) - 1 + 6) / 4));
 }
 
-template <class T, bool FIRST, int Q1, int Q2, int B>
-__global__ void __launch_bounds__(FK_THREADS, fk_inplace(Q1, Q2) ? 4 : 2) k_fold(const void* __restrict__ src_v, T* __restrict__ dst_all,
-                                                       const FoldGroup fg, int s) {
+template <class T, bool FIRST, int Q1, int Q2, int B, bool ALIGNED>
+__global__ void __launch_bounds__(FK_THREADS, fk_inplace(Q1, Q2) ? 4 : ALIGNED ? 2 : 3) k_fold(const void* __restrict__ src_v, T* __restrict__ dst_all, int s, int n,
+                                                       bool quads, const FoldGroup fg) {
     constexpr int q = Q1 + Q2;
     constexpr bool INPLACE = fk_inplace(Q1, Q2);
     constexpr int rows = 1 << q;
@@ -271,22 +284,30 @@ __global__ void __launch_bounds__(FK_THREADS, fk_inplace(Q1, Q2) ? 4 : 2) k_fold
     constexpr int KPL = ((WT + 6) / 4 + 31) / 32;        // aligned words per lane and row (WIDEN)
 
     struct Tile {
-        int64_t p0, ld, blk, c;
+        int64_t p0, ld, blk, c;  // c: first column, -3 .. -1 in an early first tile
         uint32_t kappa;
         int ei, t;
     };
+    auto source = [&](int ei) { return FIRST ? (const S*)fg.e[ei].src : (const S*)src_v + fg.e[ei].off; };
     auto locate = [&](uint32_t u) {
         Tile w;
-        w.ei = group_entry(fg, u);
-        w.p0 = fg.p0[w.ei];
-        w.ld = fg.ld[w.ei];
-        const uint32_t unit = u - (uint32_t)fg.unit0[w.ei];
-        const uint32_t n_ct = (uint32_t)((w.p0 + B - 1) / B);
+        w.ei = group_entry(fg, n, u);
+        w.p0 = fg.e[w.ei].p0;
+        w.ld = fg.e[w.ei].ld;
+        const uint32_t unit = u - fg.e[w.ei].unit0;
+        const uint32_t n_ct = (uint32_t)fg.e[w.ei].n_ct;
         const uint32_t rest = unit / n_ct;
         w.kappa = rest & ((1u << s) - 1);
         w.blk = rest >> s;
         w.c = (int64_t)(unit - rest * n_ct) * B;
-        w.t = (int)((FIRST ? w.p0 : (int64_t)w.kappa) & 3);
+        w.t = (int)((FIRST ? (uint32_t)w.p0 : w.kappa) & 3);
+        if constexpr (!ALIGNED) {
+            // row 0's first element and the distance of rows, mod 4
+            const uint32_t row0 = FIRST ? (rows % 4 ? (uint32_t)w.blk * rows * (uint32_t)w.p0 : 0u)
+                                        : ((((uint32_t)w.blk * rows) << s) + w.kappa) * (uint32_t)w.ld;
+            w.c -= ((uint32_t)(reinterpret_cast<uintptr_t>(source(w.ei)) / sizeof(S)) + row0) & 3;
+            if (!FIRST) w.t = (int)((w.kappa + ((uint32_t)w.ld << s)) & 3);
+        }
         return w;
     };
     uint32_t wv[WIDEN ? RPW : 1][KPL];  // WIDEN: the tile's words between issue and store
@@ -300,19 +321,20 @@ __global__ void __launch_bounds__(FK_THREADS, fk_inplace(Q1, Q2) ? 4 : 2) k_fold
     auto stage_issue = [&](const Tile& w) {
         // lane j: where row warp + j * NW starts, and how it is staged (0:
         // beyond the data, zeros; 1: 16-byte copies; 2: element by element)
-        const S* __restrict__ src = FIRST ? (const S*)fg.src[w.ei] : (const S*)src_v + fg.off[w.ei];
+        const S* __restrict__ src = source(w.ei);
         my_how = 0;
         {
             const int u = warp + lane * NW;
             if (lane < RPW && u < rows) {
                 const int64_t g = w.blk * rows + u;
+                const int64_t c = !ALIGNED && w.c < 0 ? w.c + 4 * w.p0 : w.c;
                 if (w.p0 < (1 << 25))
-                    my_base = (uint32_t)((uint32_t)w.c + (w.kappa % (uint32_t)w.p0) * (uint32_t)u) % (uint32_t)w.p0;
+                    my_base = ((uint32_t)c + (w.kappa % (uint32_t)w.p0) * (uint32_t)u) % (uint32_t)w.p0;
                 else
-                    my_base = (w.c + (int64_t)w.kappa * u) % w.p0;
+                    my_base = (c + (int64_t)w.kappa * u) % w.p0;
                 my_row = FIRST ? g * w.p0 : ((g << s) + w.kappa) * w.ld;
                 const uintptr_t a = reinterpret_cast<uintptr_t>(src + my_row + my_base) / sizeof(S);
-                if (!FIRST || g < fg.m_data[w.ei]) my_how = my_base + WT <= w.p0 && (a & 3) == ((w.t * u) & 3) ? 1 : 2;
+                if (!FIRST || g < fg.e[w.ei].m_data) my_how = my_base + WT <= w.p0 && (a & 3) == ((w.t * u) & 3) ? 1 : 2;
             }
         }
 #pragma unroll
@@ -369,15 +391,21 @@ __global__ void __launch_bounds__(FK_THREADS, fk_inplace(Q1, Q2) ? 4 : 2) k_fold
     };
 
     const Tile w = locate(blockIdx.x);
+    if (!ALIGNED && w.c >= w.p0) return;  // (an early start may leave the last tile nothing)
     stage_issue(w);
     stage_finish(w.t);
     {
         __syncthreads();
-        T* __restrict__ dst = dst_all + fg.off[w.ei];
+        T* __restrict__ dst = dst_all + fg.e[w.ei].off;
         const int64_t ld = w.ld;
         const int ncols = (w.c + B <= w.p0) ? B : (int)(w.p0 - w.c);
-        const bool vec = (ld & 3) == 0 && ((uintptr_t)dst & 15) == 0;
         T* __restrict__ drow = dst + ((w.blk << (s + q)) + ((int64_t)w.kappa << q)) * ld + w.c;
+
+        // (ALIGNED: always true, but not known to the compiler, which then
+        // schedules the stores worse: 1024 x 2004 12.6 us, 13.3; the 8-bit
+        // beam's search 13.77 ms, 13.98)
+        const bool vec = ALIGNED ? !quads : (ld & 3) == 0 && (w.c & 3) == 0 && ((uintptr_t)dst & 15) == 0;
+        const int early = !ALIGNED && w.c < 0 ? (int)-w.c : 0;  // columns before the row's start
 
         // sub-pass 1: groups of R1 consecutive rows
         auto sub1 = [&](auto tt) {
@@ -418,7 +446,7 @@ __global__ void __launch_bounds__(FK_THREADS, fk_inplace(Q1, Q2) ? 4 : 2) k_fold
                     if (Q2 == 0) {
                         if (x0 < ncols) {
 #pragma unroll
-                            for (int v = 0; v < R1; ++v) store4(drow + v * ld + x0, out[v], ncols - x0, vec);
+                            for (int v = 0; v < R1; ++v) store4(drow + v * ld + x0, out[v], ncols - x0, vec, early - x0);
                         }
                     } else {
                         // group g is input row u2 = g of sub-pass 2
@@ -460,9 +488,10 @@ __global__ void __launch_bounds__(FK_THREADS, fk_inplace(Q1, Q2) ? 4 : 2) k_fold
                     T out[R2][4];
                     F::run(a, out);
                     T* d = drow + (int64_t)(k1 * R2) * ld + x0;
-                    if (q == 6 || vec || whole < 128) {  // (64-row tiles: bound by instructions, not by sectors)
+                    // (64-row tiles: bound by instructions, not by sectors)
+                    if (q == 6 || vec || !quads || whole < 128 || x0 - 4 * lane < early) {
 #pragma unroll
-                        for (int v = 0; v < R2; ++v) store4(d + v * ld, out[v], ncols - x0, vec);
+                        for (int v = 0; v < R2; ++v) store4(d + v * ld, out[v], ncols - x0, vec, early - x0);
                     } else {
 #pragma unroll
                         for (int v = 0; v < R2; ++v) {
@@ -492,14 +521,24 @@ static int split_passes(int m, int qmax, int* qs) {
 }
 
 // Fill the group's CTA ranges for a pass whose CTAs cover `rows` output rows
-// and `tile` columns; returns the launch's CTA count.
-static int64_t group_units(FoldGroup& fg, int64_t m_rows, int rows, int tile) {
+// and `tile` columns; returns the launch's CTA count.  The pass reads rows of
+// `plane` (null: of the series) and writes rows of `dst`; *aligned: every row's
+// tiles start on four-element boundaries in both.  Otherwise a tile may begin
+// up to three columns early.
+static int64_t group_units(FoldGroup& fg, int64_t m_rows, int rows, int tile, const void* plane, const void* dst,
+                           size_t esz, bool* aligned) {
     int64_t u = 0;
+    uint64_t all = reinterpret_cast<uintptr_t>(dst) / 4;
     for (int i = 0; i < fg.n; ++i) {
-        fg.unit0[i] = u;
-        u += (m_rows / rows) * ((fg.p0[i] + tile - 1) / tile);
+        const uint64_t base = reinterpret_cast<uintptr_t>(plane ? plane : fg.e[i].src) / esz;
+        const uint64_t pitch = plane ? (uint64_t)fg.e[i].ld : rows % 4 == 0 ? 0 : (uint64_t)fg.e[i].p0;
+        all |= base | pitch | (uint64_t)fg.e[i].ld | (uint64_t)fg.e[i].off;
+        const int64_t tiles = (fg.e[i].p0 + ((base | pitch) & 3 ? 3 : 0) + tile - 1) / tile;
+        fg.e[i].n_ct = (int32_t)std::min<int64_t>(tiles, INT32_MAX);
+        fg.e[i].unit0 = (uint32_t)u;
+        u += (m_rows / rows) * tiles;
     }
-    fg.unit0[fg.n] = u;
+    *aligned = (all & 3) == 0;
     return u;
 }
 
@@ -509,12 +548,16 @@ static ffa_status launch_k(const void* src, T* dst, FoldGroup& fg, int64_t m_row
     constexpr int rows = 1 << q;
     constexpr int wa = fk_wa(q, Q1, B), wb = fk_wb(q, Q1, B);
     const size_t smem = sizeof(T) * (size_t)rows * (fk_inplace(Q1, Q2) ? fk_max(wa, wb) : wa + (Q2 > 0 ? wb : 0));
-    ffa_status es = ensure_smem((const void*)k_fold<T, FIRST, Q1, Q2, B>, smem);
+    ffa_status es = ensure_smem((const void*)k_fold<T, FIRST, Q1, Q2, B, true>, smem);
+    if (es == FFA_OK) es = ensure_smem((const void*)k_fold<T, FIRST, Q1, Q2, B, false>, smem);
     if (es != FFA_OK) return es;
-    const int64_t units = group_units(fg, m_rows, rows, B);
+    using S = typename std::conditional<FIRST, typename FoldIn<T>::type, T>::type;
+    bool aligned = false;
+    const int64_t units = group_units(fg, m_rows, rows, B, FIRST ? nullptr : src, dst, sizeof(S), &aligned);
     if (units <= 0) return FFA_OK;
     if (units > INT32_MAX) return fail(FFA_ERR_UNSUPPORTED, "fold: plane too large for one launch");
-    k_fold<T, FIRST, Q1, Q2, B><<<(unsigned)units, FK_THREADS, smem, st>>>(src, dst, fg, s);
+    if (aligned) k_fold<T, FIRST, Q1, Q2, B, true><<<(unsigned)units, FK_THREADS, smem, st>>>(src, dst, s, fg.n, false, fg);
+    else k_fold<T, FIRST, Q1, Q2, B, false><<<(unsigned)units, FK_THREADS, smem, st>>>(src, dst, s, fg.n, units >= sm_count(), fg);
     FFA_LAUNCH_CHECK("k_fold");
     count_launch();
     return FFA_OK;
@@ -545,7 +588,7 @@ static ffa_status pass_q(int q, bool wide, const void* src, T* dst, FoldGroup& f
 }
 
 // The fold's launch shape: at most `qmax` stages per pass, tiles of `tile`
-// columns (0: 256 below six stages, 128 at six, so that two CTAs fit an SM).
+// columns (0: 256 below six stages, 128 at six, so that four CTAs fit an SM).
 struct FoldShape {
     int qmax;
     int tile;
@@ -596,9 +639,10 @@ int log2i(int64_t v) {
 
 FoldShape tuned_shape(int precision, int stages, int64_t p0, int64_t ld) {
     // Untuned, twelve stages on dense rows that are not 16-byte aligned: three
-    // passes of four instead of two of six, whose unaligned rows cost more
-    // than a pass (4096 x 19977: 428 us, 461; 4096 x 4001: 106, 117; 2048 rows,
-    // six and five stages: 293 us, 377 as four, four and three).
+    // passes of four instead of two of six (4096 x 366 / 1489 / 4001 / 7001 /
+    // 19977: 19 / 38 / 86 / 142 / 373 us, 17 / 37 / 85 / 138 / 376; int8 20 / 38
+    // / 84 / 140 / 367, 23 / 39 / 82 / 128 / 346).  Eleven stages stay two
+    // passes (2048 x 19977: 167 us, 229 as four, four and three).
     const FoldShape none = (ld & 3) != 0 && stages == 12 ? FoldShape{5, 0} : SHAPE_DEFAULT;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return none;
@@ -619,11 +663,11 @@ static ffa_status fold_with(const void* d_z, int32_t precision, int64_t p0, int6
                             int stages, int64_t ld, void* d_plane, void* d_tmp, cudaStream_t st, FoldShape fs) {
     FoldGroup fg;
     fg.n = 1;
-    fg.p0[0] = p0;
-    fg.m_data[0] = m_data;
-    fg.off[0] = 0;
-    fg.ld[0] = ld;
-    fg.src[0] = d_z;
+    fg.e[0].p0 = p0;
+    fg.e[0].m_data = m_data;
+    fg.e[0].off = 0;
+    fg.e[0].ld = ld;
+    fg.e[0].src = d_z;
     return fold_group(d_z, precision, fg, m_rows, stages, d_plane, d_tmp, st, fs);
 }
 
@@ -679,11 +723,11 @@ ffa_status launch_fold_group(const void* d_z, int32_t precision, int n, const in
     FoldGroup fg;
     fg.n = n;
     for (int i = 0; i < n; ++i) {
-        fg.p0[i] = p0[i];
-        fg.m_data[i] = m_data[i];
-        fg.off[i] = off[i];
-        fg.ld[i] = plane_pitch(p0[i]);
-        fg.src[i] = z ? z[i] : d_z;
+        fg.e[i].p0 = p0[i];
+        fg.e[i].m_data = m_data[i];
+        fg.e[i].off = off[i];
+        fg.e[i].ld = plane_pitch(p0[i]);
+        fg.e[i].src = z ? z[i] : d_z;
     }
     return fold_group(d_z, precision, fg, m_rows, stages, d_plane, d_tmp, st,
                       tuned_shape(precision, stages, p0[n - 1], plane_pitch(p0[n - 1])));
