@@ -152,7 +152,10 @@ ffa_status ffa_plan_periods(const ffa_plan* plan, int64_t trial_begin, int64_t c
 
 /* Run the whole search (Section 2.3 pipeline) on the n-sample device series
  * d_series (type cfg.in_type).  Writes n_trials records to d_records.
- * d_workspace: >= workspace_bytes of device memory, 256-byte aligned.
+ * d_workspace: >= workspace_bytes of device memory, 256-byte aligned:
+ * ffa_plan_info's bytes, with room to fold short base periods in large groups;
+ * down to room for the largest base period (and 1024 rows of the shorter ones)
+ * less is taken and the groups are smaller, with the same records.
  * d_status: one int32 device word, zeroed by the caller; device-side checks
  * store an ffa_status there.  Asynchronous on `stream`. */
 ffa_status ffa_search(const ffa_plan* plan, const void* d_series, void* d_workspace,
@@ -350,7 +353,9 @@ ffa_status ffa_server_create(const ffa_server_config* cfg, ffa_server** out);
  * completes).  On completion the server keeps the top_k (<= 4096) candidates
  * with S/N >= snr_min, the best trial, and, if host_records is non-null,
  * copies the whole periodogram there (n_trials records).  *ticket identifies
- * the request.  FFA_ERR_OOM if the request needs more than the whole arena. */
+ * the request.  A request that finds less than ffa_server_request_bytes free
+ * may run in a smaller workspace (see ffa_search); FFA_ERR_OOM if the least it
+ * runs in is more than the whole arena. */
 ffa_status ffa_server_submit(ffa_server* server, const ffa_search_config* cfg, const void* host_series,
                              int64_t n, double snr_min, int32_t top_k, ffa_record* host_records,
                              int64_t* ticket);

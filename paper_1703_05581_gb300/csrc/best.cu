@@ -654,7 +654,7 @@ extern "C" ffa_status ffa2best(const ffa_plan* p, const ffa_record* d_records,
     *n_peaks = 0;
     if (p->n_trials == 0) return FFA_OK;
     if (!d_records || !d_ws) return fail(FFA_ERR_ARG, "ffa2best: null buffer");
-    if (ws_bytes < p->ws_bytes) return fail(FFA_ERR_OOM, "ffa2best: workspace too small");
+    if (ws_bytes < p->ws_min) return fail(FFA_ERR_OOM, "ffa2best: workspace too small");
     cudaStream_t st = as_stream(stream);
     const int64_t n_ent = (int64_t)p->entries.size();
     const Layout L = layout(n_ent, p->n_trials);

@@ -18,12 +18,12 @@ struct ffa_plan {
     int32_t n_octaves = 0;
     int64_t n_trials = 0;
     int64_t max_plane = 0;  // largest m_rows * p0
-    int64_t plane_elems = 0;  // elements of each plane buffer (>= max_plane; room for grouped planes)
     std::vector<ffa_plan_entry> entries;
     std::vector<int64_t> oct_first, oct_count, oct_n;
     // workspace layout (bytes)
-    size_t off_raw_a = 0, off_raw_b = 0, off_resid = 0, off_z = 0, off_stats = 0, off_plane0 = 0,
-           off_plane1 = 0, off_cand = 0, off_best = 0, off_bits = 0, ws_bytes = 0;
+    size_t off_raw_a = 0, off_raw_b = 0, off_resid = 0, off_z = 0, off_stats = 0, off_cand = 0,
+           off_best = 0, off_bits = 0, off_plane0 = 0;
+    size_t ws_bytes = 0, ws_min = 0;  // with planes for groups of base periods; the least that a search runs in
 };
 
 
@@ -113,6 +113,10 @@ ffa_status launch_score_alg2(const void* d_prof, int32_t precision, bool fused, 
 int score_shape(int64_t p0, int wmax);
 // Blocks of one group of a shape's block-offset scan (part of its sums' order).
 int score_scan_group(int shape);
+
+// The least workspace a search of the plan runs in (its base periods are then
+// folded in smaller groups); ffa_plan_info's is the size that it is fastest in.
+size_t plan_workspace_min(const ffa_plan* p);
 
 // ffa2best on a plan's records (defined in best.cu); workspace bytes it needs.
 size_t best_workspace_bytes(int64_t n_entries, int64_t n_trials);

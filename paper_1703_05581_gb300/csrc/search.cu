@@ -118,7 +118,10 @@ struct CandCtl {
     uint32_t n_out;  // min(top_k, records with snr >= snr_min)
     uint32_t pad;
     CandOut out[CAND_MAX];
-    unsigned long long keys[CAND_MAX];
+    union {
+        unsigned long long keys[CAND_MAX];
+        uint32_t hist[CAND_BINS];  // of the passes, which end before the keys are written
+    };
     unsigned long long prefix, mask;  // the wanted key's digits so far
     uint32_t count;                   // records with snr >= snr_min
     uint32_t rank;                    // wanted rank among the keys with the prefix
@@ -127,7 +130,6 @@ struct CandCtl {
     uint32_t n_keys;
     uint32_t done;                    // the keys up to the prefix's end are few enough to sort
     uint32_t ticket[CAND_PASSES];
-    uint32_t hist[CAND_BINS];
 };
 
 // ascending key = descending snr, then ascending trial index
@@ -488,30 +490,45 @@ ffa_status ffa_plan_create(const ffa_search_config* cfg, int64_t n, ffa_plan** o
     off = align256(off + (cfg->precision == FFA_FOLD_F32 ? 4 : 1) * (size_t)n0);
     p->off_stats = off;
     off = align256(off + sizeof(double) * STATS_DOUBLES);
-    // planes: the largest base period, or a group of small ones (no more than
-    // all of them)
-    p->plane_elems = std::max<int64_t>(p->max_plane, 1);
-    int64_t all = 0, widest = 0;
-    for (const ffa_plan_entry& e : p->entries) {
-        all += (int64_t)plane_slot(e);
-        widest = std::max<int64_t>(widest, (int64_t)plane_slot(e));
-    }
-    p->plane_elems = std::max<int64_t>(
-        p->plane_elems, std::min<int64_t>({(int64_t)FOLD_GROUP_MAX * widest, GROUP_ELEMS, all}));
-    p->off_plane0 = off;
-    off = align256(off + 4 * (size_t)p->plane_elems);
-    p->off_plane1 = off;
-    off = align256(off + 4 * (size_t)p->plane_elems);
     p->off_cand = off;
     off = align256(off + sizeof(CandCtl));
     p->off_best = off;
     off = align256(off + ffa::best_workspace_bytes((int64_t)p->entries.size(), p->n_trials));
     p->off_bits = off;
     if (cfg->persistence) off = align256(off + (size_t)n0);
+    // The two planes come last and take what the workspace leaves them: room
+    // for a group of base periods (no more than all of them), or at least for
+    // the largest base period, and for ROWS_MIN rows of the shorter ones.
+    constexpr int64_t ROWS_MIN = 1024;
+    int64_t all = 0, widest = 0, least = std::max<int64_t>(p->max_plane, 1);
+    for (const ffa_plan_entry& e : p->entries) {
+        const int64_t slot = (int64_t)plane_slot(e);
+        all += slot;
+        widest = std::max(widest, slot);
+        if (e.m_rows < ROWS_MIN) least = std::max(least, std::min((ROWS_MIN / e.m_rows) * slot, GROUP_ELEMS));
+    }
+    const int64_t most = std::max(least, std::min<int64_t>({(int64_t)FOLD_GROUP_MAX * widest, GROUP_ELEMS, all}));
+    p->off_plane0 = off;
+    p->ws_min = off + 2 * align256(4 * (size_t)least);
+    off += 2 * align256(4 * (size_t)most);
     p->ws_bytes = off;
     *out = p;
     return FFA_OK;
 }
+
+}  // extern "C"
+
+namespace ffa {
+size_t plan_workspace_min(const ffa_plan* p) { return p->ws_min; }
+}  // namespace ffa
+
+// Elements of each plane in a workspace of ws_bytes (>= ws_min; more than
+// ws_bytes is not used), and the second plane's place.
+static size_t plane_bytes(const ffa_plan* p, size_t ws_bytes) {
+    return (std::min(ws_bytes, p->ws_bytes) - p->off_plane0) / 2 / 256 * 256;
+}
+
+extern "C" {
 
 void ffa_plan_destroy(ffa_plan* plan) { delete plan; }
 
@@ -562,9 +579,9 @@ ffa_status ffa_plan_periods(const ffa_plan* p, int64_t trial_begin, int64_t coun
 // Consecutive base periods folded and scored by one set of launches: same
 // octave, rows, widths and floor(log2 p0) (so the same tuned pass depth and
 // CTA shape), together at most FOLD_GROUP_MAX base periods and GROUP_ELEMS
-// plane elements.  A larger base period goes alone.
+// plane elements (or the workspace's).  A larger base period goes alone.
 
-static int64_t group_end(const ffa_plan* p, int64_t t, int64_t b) {
+static int64_t group_end(const ffa_plan* p, int64_t t, int64_t b, size_t plane_elems) {
     const ffa_plan_entry& e0 = p->entries[(size_t)t];
     auto lg = [](int64_t v) {
         int r = 0;
@@ -579,7 +596,7 @@ static int64_t group_end(const ffa_plan* p, int64_t t, int64_t b) {
             std::memcmp(e.widths, e0.widths, sizeof(int32_t) * (size_t)e0.n_widths) != 0 ||
             score_shape(e.p0, e.widths[e.n_widths - 1]) != score_shape(e0.p0, e0.widths[e0.n_widths - 1]))
             break;
-        if (elems + plane_slot(e) > (size_t)GROUP_ELEMS) break;
+        if (elems + plane_slot(e) > std::min((size_t)GROUP_ELEMS, plane_elems)) break;
         elems += plane_slot(e);
         ++j;
     }
@@ -625,7 +642,7 @@ static ffa_status search_range(const ffa_plan* p, const void* d_series, void* d_
     if (e0 < 0 || e1 > ne || e0 > e1) return fail(FFA_ERR_ARG, "search: entry range out of bounds");
     if (e0 == e1 || p->n_trials == 0) return FFA_OK;
     if (!d_series || !d_ws || !d_records) return fail(FFA_ERR_ARG, "search: null buffer");
-    if (ws_bytes < p->ws_bytes) return fail(FFA_ERR_OOM, "search: workspace too small");
+    if (ws_bytes < p->ws_min) return fail(FFA_ERR_OOM, "search: workspace too small");
     if ((uintptr_t)d_ws % 256 != 0) return fail(FFA_ERR_ARG, "search: workspace not 256-byte aligned");
     char* ws = (char*)d_ws;
     double* raw[2] = {(double*)(ws + p->off_raw_a), (double*)(ws + p->off_raw_b)};
@@ -634,7 +651,7 @@ static ffa_status search_range(const ffa_plan* p, const void* d_series, void* d_
     double* stats = (double*)(ws + p->off_stats);
     int8_t* bits = d_persist ? (int8_t*)(ws + p->off_bits) : nullptr;
     void* plane0 = ws + p->off_plane0;
-    void* plane1 = ws + p->off_plane1;
+    void* plane1 = ws + p->off_plane0 + plane_bytes(p, ws_bytes);
     const ffa_search_config& c = p->cfg;
     const int32_t last_oct = p->entries[(size_t)(e1 - 1)].octave;
     const int32_t first_oct = p->entries[(size_t)e0].octave;
@@ -666,7 +683,7 @@ static ffa_status search_range(const ffa_plan* p, const void* d_series, void* d_
         const int64_t a = std::max<int64_t>(e0, p->oct_first[o]);
         const int64_t b = std::min<int64_t>(e1, p->oct_first[o] + p->oct_count[o]);
         for (int64_t t = a; t < b;) {
-            const int64_t t1 = group_end(p, t, b);
+            const int64_t t1 = group_end(p, t, b, plane_bytes(p, ws_bytes) / 4);
             const ffa_plan_entry& e = p->entries[(size_t)t];
             int m = 0;
             while ((1 << m) < e.m_rows) ++m;
@@ -756,7 +773,7 @@ ffa_status ffa_autotune(const ffa_plan* p, void* d_ws, size_t ws_bytes, void* st
     if (n_tuned) *n_tuned = 0;
     if (p->n_trials == 0) return FFA_OK;
     if (!d_ws) return fail(FFA_ERR_ARG, "autotune: null workspace");
-    if (ws_bytes < p->ws_bytes) return fail(FFA_ERR_OOM, "autotune: workspace too small");
+    if (ws_bytes < p->ws_min) return fail(FFA_ERR_OOM, "autotune: workspace too small");
     char* ws = (char*)d_ws;
     // shapes: (stages before the fused last one, floor(log2 p0)) -> its entries
     std::map<std::pair<int, int>, std::vector<size_t>> groups;
@@ -771,7 +788,7 @@ ffa_status ffa_autotune(const ffa_plan* p, void* d_ws, size_t ws_bytes, void* st
     for (auto& g : groups) {
         const ffa_plan_entry& e = p->entries[g.second[g.second.size() / 2]];  // the median base period
         ffa_status s = tune_fold(ws + p->off_z, p->cfg.precision, e.p0, e.m_data, e.m_rows, g.first.first,
-                                 plane_pitch(e.p0), ws + p->off_plane0, ws + p->off_plane1, as_stream(stream),
+                                 plane_pitch(e.p0), ws + p->off_plane0, ws + p->off_plane0 + plane_bytes(p, ws_bytes), as_stream(stream),
                                  nullptr);
         if (s != FFA_OK) return s;
         ++n;
@@ -810,7 +827,7 @@ ffa_status ffa_search_series(const ffa_plan* p, const void* d_series, int32_t oc
     if (octave < 0 || octave >= p->n_octaves) return fail(FFA_ERR_ARG, "search_series: octave outside the plan");
     if (what != FFA_DUMP_RESID && what != FFA_DUMP_Z) return fail(FFA_ERR_ARG, "search_series: bad `what`");
     if (!d_series || !d_ws || !d_out) return fail(FFA_ERR_ARG, "search_series: null buffer");
-    if (ws_bytes < p->ws_bytes) return fail(FFA_ERR_OOM, "search_series: workspace too small");
+    if (ws_bytes < p->ws_min) return fail(FFA_ERR_OOM, "search_series: workspace too small");
     if ((uintptr_t)d_ws % 256 != 0) return fail(FFA_ERR_ARG, "search_series: workspace not 256-byte aligned");
     cudaStream_t st = as_stream(stream);
     char* ws = (char*)d_ws;
@@ -829,7 +846,7 @@ ffa_status ffa_search_plane(const ffa_plan* p, const void* d_series, int64_t ent
     if (!p) return fail(FFA_ERR_ARG, "search_plane: null plan");
     if (entry < 0 || entry >= (int64_t)p->entries.size()) return fail(FFA_ERR_ARG, "search_plane: entry outside the plan");
     if (!d_series || !d_ws || !d_plane) return fail(FFA_ERR_ARG, "search_plane: null buffer");
-    if (ws_bytes < p->ws_bytes) return fail(FFA_ERR_OOM, "search_plane: workspace too small");
+    if (ws_bytes < p->ws_min) return fail(FFA_ERR_OOM, "search_plane: workspace too small");
     if ((uintptr_t)d_ws % 256 != 0) return fail(FFA_ERR_ARG, "search_plane: workspace not 256-byte aligned");
     cudaStream_t st = as_stream(stream);
     char* ws = (char*)d_ws;
@@ -841,7 +858,7 @@ ffa_status ffa_search_plane(const ffa_plan* p, const void* d_series, int64_t ent
     // densely into the caller's plane
     const int64_t ld = plane_pitch(e.p0);
     s = launch_fold(ws + p->off_z, p->cfg.precision, e.p0, e.m_data, e.m_rows, -1, ld, ws + p->off_plane0,
-                    ws + p->off_plane1, st);
+                    ws + p->off_plane0 + plane_bytes(p, ws_bytes), st);
     if (s != FFA_OK) return s;
     const size_t esz = 4;  // float or int32
     cudaError_t ce = cudaMemcpy2DAsync(d_plane, esz * (size_t)e.p0, ws + p->off_plane0, esz * (size_t)ld,
@@ -1147,7 +1164,7 @@ static ffa_status candidates_range(const ffa_plan* p, int64_t e0, int64_t e1, co
     *best = -1;
     if (e0 == e1 || p->n_trials == 0) return FFA_OK;
     if (!d_records || !d_ws) return fail(FFA_ERR_ARG, "candidates: null buffer");
-    if (ws_bytes < p->ws_bytes) return fail(FFA_ERR_OOM, "candidates: workspace too small");
+    if (ws_bytes < p->ws_min) return fail(FFA_ERR_OOM, "candidates: workspace too small");
     cudaStream_t st = as_stream(stream);
     CandCtl* ctl = (CandCtl*)((char*)d_ws + p->off_cand);
     const int64_t t0 = p->entries[(size_t)e0].first_trial;

@@ -98,7 +98,8 @@ struct Request {
     int32_t top_k = 0;
     ffa_record* host_records = nullptr;
     ffa_plan* plan = nullptr;
-    size_t need = 0, off = 0, in_bytes = 0, rec_bytes = 0;
+    size_t need = 0, need_min = 0;  // arena bytes with the plan's workspace, and with the least one
+    size_t got = 0, off = 0, in_bytes = 0, rec_bytes = 0;
     int bypassed = 0;
     // result
     bool done = false;
@@ -143,7 +144,9 @@ Request* admit(ffa_server* s) {
     const bool head_only = head->bypassed >= MAX_BYPASS;
     for (auto it = s->queue.begin(); it != s->queue.end(); ++it) {
         Request* r = *it;
-        const size_t off = s->arena->alloc(r->need);
+        // a full or small arena: the least that the request runs in
+        size_t off = s->arena->alloc(r->got = r->need);
+        if (off == Arena::none) off = s->arena->alloc(r->got = r->need_min);
         if (off != Arena::none) {
             r->off = off;
             if (r != head) ++head->bypassed;
@@ -162,9 +165,9 @@ void run_request(ffa_server* s, int slot, Request* r) {
     void* d_series = blk;
     ffa_record* d_rec = (ffa_record*)(blk + al(r->in_bytes));
     void* d_ws = blk + al(r->in_bytes) + al(r->rec_bytes);
-    size_t ws_bytes = 0;
+    const size_t ws_bytes = r->got - al(r->in_bytes) - al(r->rec_bytes);
     int64_t n_trials = 0;
-    ffa_plan_info(r->plan, nullptr, &n_trials, nullptr, nullptr, &ws_bytes);
+    ffa_plan_info(r->plan, nullptr, &n_trials, nullptr, nullptr, nullptr);
     ffa_status st_ = FFA_OK;
     auto check = [&](ffa_status x) {
         if (st_ == FFA_OK && x != FFA_OK) {
@@ -210,7 +213,7 @@ void worker(ffa_server* s, int slot) {
         lk.unlock();
         run_request(s, slot, r);
         lk.lock();
-        s->arena->release(r->off, r->need);
+        s->arena->release(r->off, r->got);
         ffa_plan_destroy(r->plan);
         r->plan = nullptr;
         r->t_done = now_ms();
@@ -292,8 +295,9 @@ ffa_status ffa_server_submit(ffa_server* s, const ffa_search_config* cfg, const 
     r->in_bytes = in_bytes_of(*cfg, n);
     r->rec_bytes = sizeof(ffa_record) * (size_t)std::max<int64_t>(nt, 1);
     r->need = al(r->in_bytes) + al(r->rec_bytes) + al(ws);
+    r->need_min = al(r->in_bytes) + al(r->rec_bytes) + al(plan_workspace_min(r->plan));
     std::lock_guard<std::mutex> lk(s->mu);
-    if (r->need > s->arena->capacity()) {
+    if (r->need_min > s->arena->capacity()) {
         ffa_plan_destroy(r->plan);
         return fail(FFA_ERR_OOM, "server_submit: request larger than the whole arena");
     }
