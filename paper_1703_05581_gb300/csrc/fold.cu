@@ -671,11 +671,29 @@ static ffa_status fold_with(const void* d_z, int32_t precision, int64_t p0, int6
     return fold_group(d_z, precision, fg, m_rows, stages, d_plane, d_tmp, st, fs);
 }
 
+// A group of n base periods on padded planes.
+static FoldGroup padded_group(const void* d_z, int n, const int64_t* p0, const int64_t* m_data, const int64_t* off,
+                              const void* const* z) {
+    FoldGroup fg;
+    fg.n = n;
+    for (int i = 0; i < n; ++i) {
+        fg.e[i].p0 = p0[i];
+        fg.e[i].m_data = m_data[i];
+        fg.e[i].off = off[i];
+        fg.e[i].ld = plane_pitch(p0[i]);
+        fg.e[i].src = z ? z[i] : d_z;
+    }
+    return fg;
+}
+
 // Time each maximum pass depth 3..6 with each tile width (128 and 256
-// columns) on one shape (CUDA events, best of 2 after a warm-up) and cache
+// columns) on one group (CUDA events, best of 2 after a warm-up) and cache
 // the fastest.  The planes are scratch.
-ffa_status tune_fold(const void* d_z, int32_t precision, int64_t p0, int64_t m_data, int64_t m_rows,
-                     int stages, int64_t ld, void* d_plane, void* d_tmp, cudaStream_t st, int* best_q) {
+ffa_status tune_fold(const void* d_z, int32_t precision, int n, const int64_t* p0, const int64_t* m_data,
+                     const int64_t* off, int64_t m_rows, int stages, void* d_plane, void* d_tmp, cudaStream_t st) {
+    if (n < 1 || n > FOLD_GROUP_MAX) return fail(FFA_ERR_ARG, "fold group: 1..FOLD_GROUP_MAX base periods");
+    FoldGroup fg = padded_group(d_z, n, p0, m_data, off, nullptr);
+    auto fold = [&](FoldShape fs) { return fold_group(d_z, precision, fg, m_rows, stages, d_plane, d_tmp, st, fs); };
     cudaEvent_t e0, e1;
     FFA_CUDA_TRY(cudaEventCreate(&e0));
     FFA_CUDA_TRY(cudaEventCreate(&e1));
@@ -685,11 +703,11 @@ ffa_status tune_fold(const void* d_z, int32_t precision, int64_t p0, int64_t m_d
     for (int q = 3; q <= 6 && s == FFA_OK; ++q) {
         for (int tile : {128, 256}) {
             const FoldShape fs = {q, tile};
-            s = fold_with(d_z, precision, p0, m_data, m_rows, stages, ld, d_plane, d_tmp, st, fs);  // warm-up
+            s = fold(fs);  // warm-up
             float t_q = 1e30f;
             for (int rep = 0; rep < 2 && s == FFA_OK; ++rep) {
                 cudaEventRecord(e0, st);
-                s = fold_with(d_z, precision, p0, m_data, m_rows, stages, ld, d_plane, d_tmp, st, fs);
+                s = fold(fs);
                 cudaEventRecord(e1, st);
                 if (cudaEventSynchronize(e1) != cudaSuccess) s = cuda_fail(cudaGetLastError(), "tune_fold");
                 float ms = 0.0f;
@@ -710,9 +728,8 @@ ffa_status tune_fold(const void* d_z, int32_t precision, int64_t p0, int64_t m_d
     FFA_CUDA_TRY(cudaGetDevice(&dev));
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        g_tune[std::make_tuple(dev, precision, stages, log2i(p0), (ld & 3) == 0)] = bs;
+        g_tune[std::make_tuple(dev, precision, stages, log2i(p0[n - 1]), true)] = bs;
     }
-    if (best_q) *best_q = bs.qmax * 1000 + bs.tile;
     return FFA_OK;
 }
 
@@ -720,15 +737,7 @@ ffa_status launch_fold_group(const void* d_z, int32_t precision, int n, const in
                              const int64_t* off, int64_t m_rows, int stages, void* d_plane, void* d_tmp,
                              cudaStream_t st, const void* const* z) {
     if (n < 1 || n > FOLD_GROUP_MAX) return fail(FFA_ERR_ARG, "fold group: 1..FOLD_GROUP_MAX base periods");
-    FoldGroup fg;
-    fg.n = n;
-    for (int i = 0; i < n; ++i) {
-        fg.e[i].p0 = p0[i];
-        fg.e[i].m_data = m_data[i];
-        fg.e[i].off = off[i];
-        fg.e[i].ld = plane_pitch(p0[i]);
-        fg.e[i].src = z ? z[i] : d_z;
-    }
+    FoldGroup fg = padded_group(d_z, n, p0, m_data, off, z);
     return fold_group(d_z, precision, fg, m_rows, stages, d_plane, d_tmp, st,
                       tuned_shape(precision, stages, p0[n - 1], plane_pitch(p0[n - 1])));
 }

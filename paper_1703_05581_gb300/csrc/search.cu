@@ -786,10 +786,24 @@ ffa_status ffa_autotune(const ffa_plan* p, void* d_ws, size_t ws_bytes, void* st
     }
     int32_t n = 0;
     for (auto& g : groups) {
-        const ffa_plan_entry& e = p->entries[g.second[g.second.size() / 2]];  // the median base period
-        ffa_status s = tune_fold(ws + p->off_z, p->cfg.precision, e.p0, e.m_data, e.m_rows, g.first.first,
-                                 plane_pitch(e.p0), ws + p->off_plane0, ws + p->off_plane0 + plane_bytes(p, ws_bytes), as_stream(stream),
-                                 nullptr);
+        // the group that a search folds the median base period in
+        const int64_t mid = (int64_t)g.second[g.second.size() / 2];
+        const ffa_plan_entry& e = p->entries[(size_t)mid];
+        const size_t plane = plane_bytes(p, ws_bytes);
+        int64_t t0 = p->oct_first[e.octave];
+        const int64_t end = t0 + p->oct_count[e.octave];
+        int64_t t1 = group_end(p, t0, end, plane / 4);
+        for (; t1 <= mid; t1 = group_end(p, t0, end, plane / 4)) t0 = t1;
+        int64_t p0s[FOLD_GROUP_MAX], mds[FOLD_GROUP_MAX], offs[FOLD_GROUP_MAX], off = 0;
+        for (int64_t t = t0; t < t1; ++t) {
+            const ffa_plan_entry& et = p->entries[(size_t)t];
+            p0s[t - t0] = et.p0;
+            mds[t - t0] = et.m_data;
+            offs[t - t0] = off;
+            off += (int64_t)plane_slot(et);
+        }
+        ffa_status s = tune_fold(ws + p->off_z, p->cfg.precision, (int)(t1 - t0), p0s, mds, offs, e.m_rows, g.first.first,
+                                 ws + p->off_plane0, ws + p->off_plane0 + plane, as_stream(stream));
         if (s != FFA_OK) return s;
         ++n;
     }

@@ -92,3 +92,24 @@ emit(out)
             tile *= 2
         assert block >= min(tile, 512)
         assert block in (256, 512) and (n > 1 << 14 or block == 512)
+
+
+@pytest.mark.parametrize("n,lo,hi", [(1 << 20, 0.53, 0.7), (1 << 22, 0.512, 0.52)])
+def test_autotune_times_the_search_s_groups(fake, n, lo, hi):
+    """The launches that are timed are those of a search: base periods that it
+    folds together are timed together."""
+    got = fakecuda.run(fake, f"""
+ts = 512e-6
+h = plan(config(tsamp_s=ts, period_min_s={lo}, period_max_s={hi}, duty_max=0.2), {n})
+ws, k = C.c_size_t(), C.c_int32()
+lib.ffa_plan_info(h, None, None, None, None, C.byref(ws))
+fake.fake_reset()
+assert lib.ffa_search(h, BUF, BUF, ws, BUF, BUF, None) == 0
+folds = [x[:2] for x in launches() if "k_fold" in x[0]]
+assert lib.ffa_autotune(h, BUF, ws, None, C.byref(k)) == 0 and k.value == 1
+emit([folds, [x[:2] for x in launches()]])
+""")
+    searched, timed = ({tuple(x) for x in v} for v in got)
+    # (one of the search's groups is timed)
+    for name in {name for name, _ in searched}:
+        assert any(x in timed for x in searched if x[0] == name), name
