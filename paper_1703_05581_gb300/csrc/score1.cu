@@ -305,11 +305,33 @@ __device__ __forceinline__ void pair_mad(unsigned long long ka, unsigned long lo
 // finite), else, and where they fail, by a radix select.  One call for all of
 // it: the scorer keeps its registers.
 template <int R, bool ONE>
-__device__ __noinline__ void profile_ranks(const unsigned char* smem, uint32_t* hist, S1Sh& sh, int p0, float mean,
+__device__ __noinline__ void profile_ranks(unsigned char* smem, uint32_t* hist, S1Sh& sh, int p0, float mean,
                                            float sig) {
     const uint32_t r1 = (uint32_t)((p0 - 1) / 2), r2 = (uint32_t)(p0 / 2);
     float mh = 0.0f, ml = 0.0f, kh, kl;
     unsigned long long ka, kb;
+    if (!(sig > 0.0f)) {
+        // Squares that are all 0: float pairs lose their low part near the
+        // smallest numbers (as FP64 does not), so the profile is scored 2^64
+        // times as large, which leaves its S/N as it is.
+        const int T = ONE ? 32 : (int)blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        float top = 0.0f;
+        for (int j = threadIdx.x; j < p0; j += T) top = fmaxf(top, fabsf(load_bin<float, R>(smem, j)));
+        top = warp_max(top);
+        if (!ONE) {
+            if (lane == 0) sh.fa[warp] = top;
+            __syncthreads();
+            top = warp_max(lane < (T >> 5) ? sh.fa[lane] : 0.0f);
+            __syncthreads();
+        }
+        if (top < 1e-12f) {
+            for (int j = threadIdx.x; j < p0; j += T) {
+                float* x = reinterpret_cast<float*>(smem + bin_addr<R>(j));
+                *x *= 18446744073709551616.0f;
+            }
+            cta_sync<ONE>();
+        }
+    }
     if (!(sig > 0.0f && member_ranks<R, ONE, false>(smem, sh, p0, mh, ml, mean, sig, ka, kb))) {
         ka = radix_rank<float, R, ONE, false>(smem, hist, sh, p0, r1, mh, ml, 0);
         kb = r1 == r2 ? ka : radix_rank<float, R, ONE, false>(smem, hist, sh, p0, r2, mh, ml, 0);
