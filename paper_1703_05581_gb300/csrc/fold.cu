@@ -182,8 +182,8 @@ __device__ __forceinline__ void store4(T* d, const T (&v)[4], int left, bool vec
 // 16-byte aligned, off elements past such a boundary: every lane but the first
 // stores the aligned quad that ends in its own values, with the lane before's
 // last `off` in front, so that a sector is written once and not in four parts
-// (dense int8 8192 x 1489, passes of
-// 5 + 4 + 4 stages: 86 -> 78 us).
+// (dense, against
+// element stores: int8 8192 x 1489 81 us, 88; 4096 x 19977 380 us, 442).
 template <class T>
 __device__ __forceinline__ void store_row(T* d, const T (&v)[4], int off) {
     const int lane = threadIdx.x & 31;
@@ -247,7 +247,7 @@ constexpr int FK_THREADS = 256;
 // groups, so one buffer of 64 rows (50 KB) serves both sub-passes and four
 // CTAs fit an SM, where two buffers left room for two: 4096 x 19977, first
 // pass, 163 us with two CTAs that staged the next tile under sub-pass 2, 153
-// in place with three, 145 with four; int8 4096 x 29 500: 230, 200, 181.
+// in place with three, 149 with four; int8 4096 x 29 500: 230, 200, 181.
 __host__ __device__ constexpr bool fk_inplace(int q1, int q2) { return q1 == 3 && q2 == 3; }
 __host__ __device__ constexpr int fk_r4(int x) { return (x + 3) & ~3; }
 __host__ __device__ constexpr int fk_max(int a, int b) { return a > b ? a : b; }

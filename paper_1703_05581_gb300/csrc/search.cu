@@ -341,10 +341,10 @@ struct PhaseTimer {
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// Grouping of base periods (see group_end): elements of a group's plane.  Two
-// planes of 64 MB stay in L2 between the fold's passes and the scorer, and a
-// launch holds enough trials to fill the GPU: an 8-bit beam at D0 = 64 (2^20
-// samples, 920 base periods of about 1.5 M elements) takes 31.8 ms with
+// Grouping of base periods (see group_end): elements of a group's plane.  A
+// launch then holds enough trials to fill the GPU, which counts for more than
+// planes that stay in L2 (two of 64 MB are about all of it): an 8-bit beam at D0
+// = 64 (2^20 samples, 920 base periods of about 1.5 M elements) took 31.8 ms with
 // single base periods, 18.1 / 15.6 / 14.6 ms with groups of 2^22 / 2^23 / 2^24.
 constexpr int64_t GROUP_ELEMS = (int64_t)1 << 24;
 // elements a base period's plane takes in a group (256-byte aligned)
