@@ -591,9 +591,9 @@ def run_gpu(args):
 # DRAM bytes (read + write) per folded-profile bin of one base period's fold
 # and scoring launches on the search's own path: ncu dram__bytes_read.sum +
 # dram__bytes_write.sum of the two fold passes and the scorer of survey entry
-# 4352 (P0 = 19977, M = 4096), 1531.4 MB over 4096 x 19977 bins (one launch
+# 4352 (P0 = 19977, M = 4096), 1529.5 MB over 4096 x 19977 bins (one launch
 # of each).
-DRAM_BYTES_PER_BIN = 1531.4e6 / (4096 * 19977)
+DRAM_BYTES_PER_BIN = 1529.5e6 / (4096 * 19977)
 
 
 # ---------------------------------------------------------------------------

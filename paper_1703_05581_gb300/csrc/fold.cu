@@ -233,9 +233,9 @@ __device__ __forceinline__ void store_row(T* d, const T (&v)[4], int off) {
 // starts on such a boundary, leave all of it out.
 //
 // What bounds it.  4096 rows of 19977 bins: the six-stage first pass takes
-// 150 us at 38 thread-instructions an element, its shared memory 73 % busy
+// 150 us at 39 thread-instructions an element, its shared memory 73 % busy
 // (234 us and 62 with two selects per value on each row's offset and 64-bit
-// divisions for each row); the five-stage second pass 130 us, 4.7 TB/s of DRAM
+// divisions for each row); the five-stage second pass 129 us, 4.7 TB/s of DRAM
 // traffic (142 us before).
 // ---------------------------------------------------------------------------
 constexpr int FK_THREADS = 256;

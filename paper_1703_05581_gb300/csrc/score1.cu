@@ -37,7 +37,7 @@
 // What bounds it.  Long profiles: the width pass's shared-memory reads (one
 // per bin and width) and the load of two rows; short ones: instructions, about
 // 4 per bin and width in all.  A fused launch of 4096 x 19977 takes 0.39 ms at
-// 99 thread-instructions a bin (0.82 ms at 195 with the profile in the
+// 95 thread-instructions a bin (0.82 ms at 195 with the profile in the
 // registers of one 1024-thread CTA per SM and a histogram per profile).
 #include <cuda_runtime.h>
 #include <math.h>
