@@ -548,14 +548,14 @@ static ffa_status launch_k(const void* src, T* dst, FoldGroup& fg, int64_t m_row
     constexpr int rows = 1 << q;
     constexpr int wa = fk_wa(q, Q1, B), wb = fk_wb(q, Q1, B);
     const size_t smem = sizeof(T) * (size_t)rows * (fk_inplace(Q1, Q2) ? fk_max(wa, wb) : wa + (Q2 > 0 ? wb : 0));
-    ffa_status es = ensure_smem((const void*)k_fold<T, FIRST, Q1, Q2, B, true>, smem);
-    if (es == FFA_OK) es = ensure_smem((const void*)k_fold<T, FIRST, Q1, Q2, B, false>, smem);
-    if (es != FFA_OK) return es;
     using S = typename std::conditional<FIRST, typename FoldIn<T>::type, T>::type;
     bool aligned = false;
     const int64_t units = group_units(fg, m_rows, rows, B, FIRST ? nullptr : src, dst, sizeof(S), &aligned);
     if (units <= 0) return FFA_OK;
     if (units > INT32_MAX) return fail(FFA_ERR_UNSUPPORTED, "fold: plane too large for one launch");
+    const ffa_status es = ensure_smem(aligned ? (const void*)k_fold<T, FIRST, Q1, Q2, B, true>
+                                              : (const void*)k_fold<T, FIRST, Q1, Q2, B, false>, smem);
+    if (es != FFA_OK) return es;
     if (aligned) k_fold<T, FIRST, Q1, Q2, B, true><<<(unsigned)units, FK_THREADS, smem, st>>>(src, dst, s, fg.n, false, fg);
     else k_fold<T, FIRST, Q1, Q2, B, false><<<(unsigned)units, FK_THREADS, smem, st>>>(src, dst, s, fg.n, units >= sm_count(), fg);
     FFA_LAUNCH_CHECK("k_fold");

@@ -41,17 +41,15 @@ ffa_status cuda_fail(cudaError_t e, const char* where) {
 static std::atomic<long long> g_launches{0};
 void count_launch(int64_t n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+// (asked for by most launches: no lock and no look-up)
 int sm_count() {
-    static std::mutex mu;
-    static std::map<int, int> cache;
+    static std::atomic<int> cache[64];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 1;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find(dev);
-    if (it != cache.end()) return it->second;
-    int n = 0;
+    int n = dev < 64 ? cache[dev].load(std::memory_order_relaxed) : 0;
+    if (n > 0) return n;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) n = 1;
-    cache[dev] = n;
+    if (dev < 64) cache[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
